@@ -251,9 +251,6 @@ int refresh_l(const moara_ctx* ctx, int m, int n, int r) {
 }
 
 // ------------------------------------------------------------------ refresh
-// Panel width of the fast blocked Cholesky (tensor-core trailing updates).
-constexpr int kFastPanel = 256;
-constexpr int kTriTcMin = 512;   // triangular-inverse levels from this block size run on tensor cores
 
 struct RefreshRunner {
     moara_ctx* ctx;
@@ -297,8 +294,8 @@ struct RefreshRunner {
             p.M = l; p.N = l; p.K = rows[i]; p.lda = l; p.ldb = l; p.ldc = l;
             p.lower_only = 1;
         });
-        cholesky_blocked(rows, shift_rel);
-        tri_inverse(/*have_diag=*/true);
+        cholesky(rows, shift_rel);
+        tri_inverse();
         moara::GemmKind apply{moara::A_KCONTIG, moara::B_KCONTIG, 0, 0, 0, 0, moara::EPI_STORE};
         gemm(apply, [&](int i, moara::GemmProb& p) {
             const int l = it[i].l;
@@ -309,91 +306,15 @@ struct RefreshRunner {
         });
     }
 
-    // Linv <- Cg^-1 for the lower-triangular Cholesky factor in Cg: diagonal
-    // 64 x 64 blocks in shared memory, then the off-diagonal blocks level by
-    // level (block size s = 64, 128, ...) with two grouped GEMMs per level:
-    //   T = L[D, A] Linv[A, A];  Linv[D, A] = -Linv[D, D] T.
-    // Lower Cholesky factor of Cg (+ shift on the diagonal) in place, by 64-wide
-    // panels: factor the diagonal block (its inverse goes to the diagonal block
-    // of Linv), solve the panel below it, update the trailing matrix.
-    void cholesky_blocked(const std::vector<int>& rows, float shift_rel, bool fast = false) {
-        int lmax = 0;
-        moara::SmallBatch sb = small();
-        sb.shift_rel = shift_rel;
-        for (size_t i = 0; i < it.size(); ++i) {
-            chk(cudaMemsetAsync(it[i].Linv, 0, sizeof(float) * (size_t)it[i].l * it[i].l, s));
-            sb.l[i] = it[i].l; sb.rows[i] = rows[i]; sb.a[i] = it[i].Cg; sb.b[i] = it[i].scal;
-            sb.c[i] = it[i].Linv; sb.fail[i] = it[i].fail;
-            lmax = std::max(lmax, it[i].l);
-        }
-        chk(moara::launch_trace_shift(sb, s, &ctx->launches));
-        const int nb = moara::kTriBase;
-        moara::GemmKind solve{moara::A_KCONTIG, moara::B_KCONTIG, 0, 0, 0, 0, moara::EPI_STORE, 1};
-        moara::GemmKind upd{moara::A_KCONTIG, moara::B_KCONTIG, 0, 0, 0, 0, moara::EPI_SUB, 1};
-        for (int j0 = 0; j0 < lmax; j0 += nb) {
-            chk(moara::launch_chol_diag(sb, j0, s, &ctx->launches));
-            // fast: the 64-wide steps update only the rest of their
-            // kFastPanel-wide panel; the trailing matrix past the panel gets
-            // one tensor-core update per panel
-            const int pend = fast ? (j0 / kFastPanel + 1) * kFastPanel : lmax;
-            for (int pass = 0; pass < 2; ++pass) {
-                moara::GemmBatch b{};
-                b.B = 1;
-                for (int i = 0; i < static_cast<int>(it.size()); ++i) {
-                    const auto& x = it[i];
-                    const long long l = x.l;
-                    const int j1 = j0 + nb;
-                    if (j1 >= x.l) continue;
-                    const int cend = std::min(x.l, pend);
-                    if (pass == 1 && cend <= j1) continue;
-                    moara::GemmProb& p = b.p[b.count++];
-                    p = moara::GemmProb{};
-                    p.lda = p.ldb = p.ldc = x.l;
-                    if (pass == 0) {      // L[j1:, panel] = A[j1:, panel] * Ljj^-T (in place)
-                        p.A = x.Cg + j1 * l + j0;
-                        p.Bm = x.Linv + j0 * l + j0;
-                        p.C = x.Cg + j1 * l + j0;
-                        p.M = x.l - j1; p.N = nb; p.K = nb;
-                    } else {              // A[j1:, j1:cend] -= L[j1:, panel] L[j1:cend, panel]^T (lower tiles)
-                        p.A = x.Cg + j1 * l + j0;
-                        p.Bm = x.Cg + j1 * l + j0;
-                        p.C = x.Cg + j1 * l + j1;
-                        p.M = x.l - j1; p.N = cend - j1; p.K = nb;
-                        p.lower_only = 1;
-                    }
-                }
-                if (b.count > 0) chk(moara::launch_gemm(pass == 0 ? solve : upd, b, s, &ctx->launches));
-            }
-            if (fast && j0 + nb == pend) trailing_update_tc(pend);
-        }
-    }
-
-    // A[pe:, pe:] -= L[pe:, pe - kFastPanel : pe] L[pe:, ...]^T (lower tiles)
-    // for every item with l > pe, as a two-plane split-precision product
-    // (16 significant bits): the panel's transposed planes go to P1.
-    void trailing_update_tc(int pe) {
-        moara::SmallBatch sq{};
-        std::vector<moara::TcSplitGemmItem> g;
-        for (size_t i = 0; i < it.size(); ++i) {
-            const auto& x = it[i];
-            if (x.l <= pe) continue;
-            const int rest = x.l - pe;
-            const int q = sq.count++;
-            sq.a[q] = x.Cg + (size_t)pe * x.l + (pe - kFastPanel);
-            sq.h[q] = x.P1;
-            sq.rows[q] = rest;
-            sq.l[q] = kFastPanel;
-            sq.ld[q] = x.l;
-            const size_t pl = (size_t)rest * kFastPanel;
-            moara::TcSplitGemmItem item{x.P1, x.P1, pl, pl, x.Cg + (size_t)pe * x.l + pe, rest, rest, kFastPanel, 0};
-            item.ldo = x.l;
-            item.sub = 1;
-            item.lower = 1;
-            g.push_back(item);
-        }
-        if (g.empty()) return;
-        chk(moara::launch_split3(sq, 1, s, &ctx->launches));
-        ks_run(g, 2);
+    // Lower Cholesky factor of Cg (+ shift on the diagonal) in place and the
+    // inverse of its diagonal superblocks (512 columns) in Linv.
+    void cholesky(const std::vector<int>& rows, float shift_rel) {
+        moara::CholBatch b{};
+        b.count = static_cast<int>(it.size());
+        b.shift_rel = shift_rel;
+        for (int i = 0; i < b.count; ++i)
+            b.p[i] = moara::CholItem{it[i].Cg, it[i].Linv, it[i].scal, it[i].fail, it[i].l, rows[i]};
+        chk(moara::launch_cholesky(b, s, &ctx->launches));
     }
 
     // One level of the blocked triangular inverse on tensor cores, for the
@@ -446,21 +367,16 @@ struct RefreshRunner {
         }
     }
 
-    void tri_inverse(bool have_diag) {
+    // Linv <- Cg^-1 from the inverse of the superblocks, level by level (block
+    // size sz = 512, 1024, ...) with two grouped products per level:
+    //   T = L[D, A] Linv[A, A];  Linv[D, A] = -Linv[D, D] T.
+    void tri_inverse() {
         int lmax = 0;
-        for (auto& x : it) {
-            if (!have_diag) chk(cudaMemsetAsync(x.Linv, 0, sizeof(float) * (size_t)x.l * x.l, s));
-            lmax = std::max(lmax, x.l);
-        }
-        if (!have_diag) {
-            moara::SmallBatch sb = small();
-            for (size_t i = 0; i < it.size(); ++i) { sb.l[i] = it[i].l; sb.a[i] = it[i].Cg; sb.c[i] = it[i].Linv; }
-            chk(moara::launch_tri_inverse_diag(sb, s, &ctx->launches));
-        }
+        for (auto& x : it) lmax = std::max(lmax, x.l);
         moara::GemmKind mul{moara::A_KCONTIG, moara::B_NCONTIG, 0, 0, 0, 0, moara::EPI_STORE};
         moara::GemmKind neg{moara::A_KCONTIG, moara::B_NCONTIG, 0, 0, 0, 0, moara::EPI_STORE_NEG};
         const bool tc = !it.empty() && it[0].tc && ctx->tc != nullptr;
-        for (int sz = moara::kTriBase; sz < lmax; sz *= 2) {
+        for (int sz = moara::kTriBase * moara::kTriSuper; sz < lmax; sz *= 2) {
             struct Pair { int mod, a0, d0, dn; };
             std::vector<Pair> pairs;
             for (int i = 0; i < static_cast<int>(it.size()); ++i) {
@@ -468,7 +384,7 @@ struct RefreshRunner {
                 for (int a0 = 0; a0 + sz < l; a0 += 2 * sz)
                     pairs.push_back({i, a0, a0 + sz, std::min(sz, l - a0 - sz)});
             }
-            if (tc && sz >= kTriTcMin) {
+            if (tc) {
                 tri_level_tc(sz, pairs.size(), [&](size_t q) {
                     const Pair& pr = pairs[q];
                     return std::array<int, 4>{pr.mod, pr.a0, pr.d0, pr.dn};
@@ -569,8 +485,8 @@ struct RefreshRunner {
             gram.push_back(g);
         }
         tc_gemm(0, gram);
-        cholesky_blocked(rows, shift_rel, /*fast=*/true);
-        tri_inverse(/*have_diag=*/true);
+        cholesky(rows, shift_rel);
+        tri_inverse();
         {   // (R^-1) in bf16: the transpose of the lower-triangular Linv, into Tt
             moara::SmallBatch sb = small();
             for (size_t i = 0; i < it.size(); ++i) {
@@ -623,7 +539,7 @@ struct RefreshRunner {
     // reads only the planes).  `pl` holds 3 * rows * l bf16 entries: the
     // planes of X for the Gram matrix, then those of X^T for the apply.
     void ks_cholqr_tall(std::vector<float*>& X, const std::vector<uint16_t*>& pl, const std::vector<int>& rows,
-                        float shift_rel, int planes, bool fast_chol = true) {
+                        float shift_rel, int planes) {
         const size_t n_it = it.size();
         auto split_rows = [&](int transpose) {
             moara::SmallBatch sb = small();
@@ -640,8 +556,8 @@ struct RefreshRunner {
             g.push_back({pl[i], pl[i], pm, pm, it[i].Cg, l, l, rows[i], 0});
         }
         ks_run(g, planes);                  // Gram X^T X
-        cholesky_blocked(rows, shift_rel, fast_chol);
-        tri_inverse(/*have_diag=*/true);
+        cholesky(rows, shift_rel);
+        tri_inverse();
         std::vector<float*> linv(n_it);
         std::vector<uint16_t*> p2(n_it);
         for (size_t i = 0; i < n_it; ++i) { linv[i] = it[i].Linv; p2[i] = it[i].P2; }
@@ -659,15 +575,15 @@ struct RefreshRunner {
     // triangular apply as split-precision tensor-core products (fp32-accurate):
     // Xout = Win R^-1, R^T R = Win^T Win + shift.
     void ks_cholqr_pass(std::vector<float*>& Win, std::vector<float*>& Xout, const std::vector<int>& rows_l,
-                        float shift_rel, int planes, bool fast_chol = true) {
+                        float shift_rel, int planes) {
         std::vector<uint16_t*> p1(it.size()), p2(it.size());
         for (size_t i = 0; i < it.size(); ++i) { p1[i] = it[i].P1; p2[i] = it[i].P2; }
         std::vector<float*> cg(it.size());
         for (size_t i = 0; i < it.size(); ++i) cg[i] = it[i].Cg;
         split3(Win, p1, 0);                 // W (as A = W^T, MN-major, and as B)
         ks_gemm(p1, p1, cg, 0, planes);     // Gram W^T W
-        cholesky_blocked(rows_l, shift_rel, fast_chol);
-        tri_inverse(/*have_diag=*/true);
+        cholesky(rows_l, shift_rel);
+        tri_inverse();
         std::vector<float*> linv(it.size());
         for (size_t i = 0; i < it.size(); ++i) linv[i] = it[i].Linv;
         split3(linv, p2, 1);                // B = Linv^T (upper triangular)
@@ -769,7 +685,7 @@ struct RefreshRunner {
                 // scales Q's columns alike and is removed by the unit-length
                 // store of P; the off-diagonal orthogonality it gives is that
                 // of the fp32 pass
-                ks_cholqr_tall(Qa, qpl, rows_m, 0.0f, 3, /*fast_chol=*/false);
+                ks_cholqr_tall(Qa, qpl, rows_m, 0.0f, 3);
                 for (int i = 0; i < n_it; ++i)                  // Q in Qb (fp32) and qbf
                     chk(moara::launch_f32_to_bf16(Qa[i], Qb[i], qbf[i], (long long)it[i].m * it[i].l, s,
                                                   &ctx->launches));
@@ -873,7 +789,7 @@ struct RefreshRunner {
                 // planes and an fp32 Cholesky (the tensor cores' short
                 // diagonal of the Gram matrix scales the columns of X alike;
                 // P's columns are stored at unit length)
-                ks_cholqr_pass(Xa, Xb, rows_l, 0.0f, planes, /*fast_chol=*/!last);
+                ks_cholqr_pass(Xa, Xb, rows_l, 0.0f, planes);
                 std::swap(Xa, Xb);                       // X in Xa
             } else {
                 gemm(prod, [&](int i, moara::GemmProb& p) {

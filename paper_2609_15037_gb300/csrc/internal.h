@@ -64,7 +64,7 @@ struct DecompBatch {
 
 // ------------------------------------------------------------- SIMT GEMM
 // C (M x N) = op(A) (M x K) * op(B) (K x N), fp32 accumulate.
-enum Epi { EPI_STORE = 0, EPI_ADAM = 1, EPI_UPDATE = 2, EPI_STORE_NEG = 3, EPI_SUB = 4 };
+enum Epi { EPI_STORE = 0, EPI_ADAM = 1, EPI_UPDATE = 2, EPI_STORE_NEG = 3 };
 
 // Triangular operands of the SIMT GEMM (zeros stored explicitly): the K loop
 // of an output tile at (m0, n0) covers only the range that can be nonzero.
@@ -113,7 +113,6 @@ enum BLayout { B_NCONTIG = 0, B_KCONTIG = 1 };
 
 struct GemmKind {
     int a_layout, b_layout, a_scale, b_scale, a_bf16, b_bf16, epi;
-    int narrow = 0;       // 128 x 64 output tiles, four CTAs per SM (plain fp32 operands, short K)
 };
 
 // Host launchers (return cudaError_t of the launch).
@@ -197,14 +196,27 @@ struct SmallBatch {
 };
 
 cudaError_t launch_philox_gaussian(const SmallBatch& b, cudaStream_t s, int64_t* launches);
-// Inverts the diagonal blocks [64j, 64j+64) of each lower-triangular a into c.
+// Lower Cholesky factor of each a (l x l, the lower triangle given) plus
+// shift_rel * sqrt(rows) * trace(a) on its diagonal, in place, and in X the
+// inverse of the factor's diagonal superblocks of kTriSuper 64-column blocks
+// (zero elsewhere).  A pivot that is not positive and finite counts as 1 and
+// sets *fail.  launch_cholesky fills step and tile_start.
 constexpr int kTriBase = 64;
-cudaError_t launch_tri_inverse_diag(const SmallBatch& b, cudaStream_t s, int64_t* launches);
-// Blocked Cholesky pieces: the diagonal shift shift_rel*sqrt(rows)*trace(a)
-// into b[0]; and the factorisation of the diagonal block starting at j0
-// (a: matrix, b: shift, c: inverse of the factor's block, written in place).
-cudaError_t launch_trace_shift(const SmallBatch& b, cudaStream_t s, int64_t* launches);
-cudaError_t launch_chol_diag(const SmallBatch& b, int j0, cudaStream_t s, int64_t* launches);
+constexpr int kTriSuper = 8;
+struct CholItem {
+    float* A;
+    float* X;
+    float* shift;         // scratch: the shift
+    int* fail;
+    int l, rows;
+};
+struct CholBatch {
+    int count, step;
+    float shift_rel;
+    int tile_start[kMaxGroup + 1];
+    CholItem p[kMaxGroup];
+};
+cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches);
 cudaError_t launch_set_identity(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 cudaError_t launch_ritz_sort(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 // Exact Rayleigh-Ritz (Jacobi) on the leading min(64, l) columns of X (a)

@@ -1,9 +1,7 @@
 // Small dense kernels of the projector refresh (TruncatedSVD of Algorithm 1
-// computed by randomized subspace iteration): the Gaussian test matrix, the
-// diagonal blocks of the blocked Cholesky factorisation and of the triangular
-// inverse used by CholeskyQR, the ordering of Ritz vectors, and the final sign
-// convention.  One CTA per problem (or per diagonal block); the problems of a
-// group run side by side in one launch.
+// computed by randomized subspace iteration): the Gaussian test matrix, plane
+// splits and transposes, the ordering of Ritz vectors, and the final sign
+// convention.  The problems of a group run side by side in one launch.
 #include <algorithm>
 #include <cuda_bf16.h>
 
@@ -93,231 +91,6 @@ __device__ float block_sum(float v, float* red) {
     }
     __syncthreads();
     return red[32];
-}
-
-// ---------------------------------------------------------------------------
-// Diagonal blocks of a lower-triangular inverse: block j of problem y covers
-// rows/cols [64j, min(64j + 64, l)); the block of a is inverted in shared
-// memory by forward substitution and written to the same place in c.  The
-// off-diagonal blocks are filled afterwards level by level with GEMMs:
-//   inv([A 0; C D]) = [A^-1 0; -D^-1 C A^-1  D^-1].
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_tri_inverse_diag(const __grid_constant__ SmallBatch b) {
-    __shared__ float Ls[kTriBase][kTriBase + 1];
-    __shared__ float Xs[kTriBase][kTriBase + 1];
-    const int pi = blockIdx.y;
-    const int l = b.l[pi];
-    const int i0 = blockIdx.x * kTriBase;
-    if (i0 >= l) return;
-    const int sz = min(kTriBase, l - i0);
-    const float* L = b.a[pi];
-    float* X = b.c[pi];
-    for (int e = threadIdx.x; e < sz * sz; e += blockDim.x) {
-        const int i = e / sz, c = e - i * sz;
-        Ls[i][c] = L[(long long)(i0 + i) * l + i0 + c];
-    }
-    __syncthreads();
-    // row by row; thread c owns column c
-    for (int i = 0; i < sz; ++i) {
-        if (threadIdx.x < sz) {
-            const int c = threadIdx.x;
-            float v = 0.0f;
-            if (c <= i) {
-                float acc = (c == i) ? 1.0f : 0.0f;
-                for (int k = c; k < i; ++k) acc = fmaf(-Ls[i][k], Xs[k][c], acc);
-                v = acc / Ls[i][i];
-            }
-            Xs[i][c] = v;
-        }
-        __syncthreads();
-    }
-    for (int e = threadIdx.x; e < sz * sz; e += blockDim.x) {
-        const int i = e / sz, c = e - i * sz;
-        X[(long long)(i0 + i) * l + i0 + c] = Xs[i][c];
-    }
-}
-
-cudaError_t launch_tri_inverse_diag(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
-    if (b.count <= 0) return cudaSuccess;
-    int lmax = 1;
-    for (int i = 0; i < b.count; ++i) lmax = b.l[i] > lmax ? b.l[i] : lmax;
-    dim3 grid((lmax + kTriBase - 1) / kTriBase, b.count);
-    k_tri_inverse_diag<<<grid, 256, 0, s>>>(b);
-    ++*launches;
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Blocked right-looking Cholesky.  k_trace_shift stores the diagonal shift of
-// the shifted CholeskyQR pass; k_chol_diag factors the (at most 64 x 64)
-// diagonal block at j0 in shared memory after the trailing updates of the
-// earlier panels, checks its pivots, writes the factor in place and its
-// inverse into the same block of c (the diagonal blocks of the triangular
-// inverse).  The panel below the block and the trailing matrix are updated by
-// grouped GEMMs on the host side.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_trace_shift(const __grid_constant__ SmallBatch b) {
-    __shared__ float red[33];
-    const int pi = blockIdx.x;
-    const int l = b.l[pi];
-    const float* A = b.a[pi];
-    float tr = 0.0f;
-    for (int i = threadIdx.x; i < l; i += blockDim.x) tr += A[(long long)i * l + i];
-    tr = block_sum(tr, red);
-    if (threadIdx.x == 0) b.b[pi][0] = b.shift_rel * sqrtf(static_cast<float>(b.rows[pi])) * tr;
-}
-
-cudaError_t launch_trace_shift(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
-    if (b.count <= 0) return cudaSuccess;
-    k_trace_shift<<<b.count, 256, 0, s>>>(b);
-    ++*launches;
-    return cudaGetLastError();
-}
-
-// 128 threads, two per row: thread (i, h) keeps columns 32 h .. 32 h + 31 of
-// row i of the block in registers (the two threads of a row are adjacent
-// lanes of one warp).  The step loops stay rolled (a fully unrolled 64 x 64
-// factorisation is too large for the instruction cache and stalls on
-// instruction fetch): during the factorisation each row is shifted left by
-// one column per step, the column crossing from the upper to the lower half
-// by a lane shuffle, so the column being eliminated is always a[0] of the
-// h = 0 thread and every register index is a compile-time constant; the
-// finished column j of the factor is broadcast through shared memory from
-// index 0, read as aligned 16-byte vectors.  The inverse then runs by
-// forward substitution, thread (i, h) holding half of row i of the inverse;
-// the finished row k is broadcast (its entries past k are exact zeros, so
-// every row update may run over all 64 columns).  Each step costs two
-// barriers of four warps.  The block moves between global and shared memory
-// coalesced.
-__global__ void __launch_bounds__(128) k_chol_diag(const __grid_constant__ SmallBatch b, int j0) {
-    constexpr int NB = kTriBase;
-    constexpr int HB = NB / 2;
-    __shared__ float tile[NB][NB + 1];   // the block; the factor's lower part as it is finished
-    __shared__ __align__(16) float bc[NB];   // broadcast column of the factor / row of the inverse
-    __shared__ float piv;
-    __shared__ int s_fail;
-    const int pi = blockIdx.x;
-    const int l = b.l[pi];
-    if (j0 >= l) return;
-    const int sz = min(NB, l - j0);
-    float* A = b.a[pi];
-    float* X = b.c[pi];
-    const float shift = b.b[pi][0];
-    const int t = threadIdx.x;
-    const int i = t >> 1, h = t & 1, c0 = h * HB;
-    const int lane = t & 31;
-    // rows and columns past sz are padded with the identity
-    for (int r = t >> 6; r < NB; r += 2) {
-        const int c = t & 63;
-        tile[r][c] = (r < sz && c < sz) ? A[(long long)(j0 + r) * l + j0 + c] + (r == c ? shift : 0.0f)
-                                        : (r == c ? 1.0f : 0.0f);
-    }
-    if (t == 0) s_fail = 0;
-    if (t < NB) bc[t] = 0.0f;
-    __syncthreads();
-    float a[HB];
-#pragma unroll
-    for (int k = 0; k < HB; ++k) a[k] = tile[i][c0 + k];
-    // right-looking factorisation; at step j, a[k] of thread (i, h) holds
-    // column j + 32 h + k of the updated row i.  A pivot that is not positive
-    // and finite is replaced by 1 and marks the failure.
-    const float4* col4 = reinterpret_cast<const float4*>(bc) + h * (HB / 4);
-#pragma unroll 1
-    for (int j = 0; j < NB; ++j) {
-        if (i == j && h == 0) {
-            float d = a[0];
-            if (!(d > 0.0f) || !isfinite(d)) {
-                d = 1.0f;
-                s_fail = 1;
-            }
-            d = sqrtf(d);
-            piv = d;
-            tile[j][j] = d;
-        }
-        __syncthreads();
-        float lij = 0.0f;
-        if (i > j && h == 0) {
-            lij = a[0] / piv;
-            bc[i - j - 1] = lij;       // column j of L below the diagonal, from index 0
-            tile[i][j] = lij;
-        }
-        lij = __shfl_sync(0xffffffffu, lij, lane & ~1);
-        const float up = __shfl_sync(0xffffffffu, a[0], lane | 1);   // column j + 32, before its update
-        __syncthreads();
-        // row i -= L[i][j] * (column j of L)^T over columns j + 1 .., shifted
-        // left by one: a[k] (column j + 32 h + k) takes bc[32 h + k - 1] =
-        // L[j + 32 h + k][j].  Past index 62 - j, bc holds earlier columns'
-        // values; they reach only slots of columns past the block or above
-        // the diagonal (and rows i <= j, which are finished), none of which
-        // is read again.
-#pragma unroll
-        for (int k = 1; k < HB; k += 4) {
-            const float4 lk = col4[(k - 1) / 4];
-            a[k - 1] = fmaf(-lij, lk.x, a[k]);
-            a[k] = fmaf(-lij, lk.y, a[k + 1]);
-            a[k + 1] = fmaf(-lij, lk.z, a[k + 2]);
-            if (k + 3 < HB) a[k + 2] = fmaf(-lij, lk.w, a[k + 3]);
-        }
-        // the last slot: column j + 32 crosses from the upper half (h = 0
-        // takes it, updated with bc[31]); past the block for h = 1
-        a[HB - 1] = h == 0 ? fmaf(-lij, bc[HB - 1], up) : 0.0f;
-    }
-    // inverse by forward substitution: row k of the inverse is finished at
-    // step k (divided by the pivot) and broadcast; rows below subtract
-    // L[i][k] times it
-    float x[HB];
-#pragma unroll
-    for (int c = 0; c < HB; ++c) x[c] = (c0 + c == i) ? 1.0f : 0.0f;
-    float4* bc4 = reinterpret_cast<float4*>(bc) + h * (HB / 4);
-#pragma unroll 1
-    for (int k = 0; k < NB; ++k) {
-        if (i == k) {
-            const float inv = 1.0f / tile[k][k];
-#pragma unroll
-            for (int c = 0; c < HB; c += 4) {
-                x[c] *= inv; x[c + 1] *= inv; x[c + 2] *= inv; x[c + 3] *= inv;
-                bc4[c / 4] = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
-            }
-        }
-        __syncthreads();
-        if (i > k) {
-            const float lik = tile[i][k];
-#pragma unroll
-            for (int c = 0; c < HB; c += 4) {
-                const float4 r = bc4[c / 4];
-                x[c] = fmaf(-lik, r.x, x[c]);
-                x[c + 1] = fmaf(-lik, r.y, x[c + 1]);
-                x[c + 2] = fmaf(-lik, r.z, x[c + 2]);
-                x[c + 3] = fmaf(-lik, r.w, x[c + 3]);
-            }
-        }
-        __syncthreads();
-    }
-    // the factor (zeros above the diagonal) in place, the inverse into c
-#pragma unroll
-    for (int k = 0; k < HB; ++k)
-        if (c0 + k > i) tile[i][c0 + k] = 0.0f;
-    __syncthreads();
-    for (int r = t >> 6; r < sz; r += 2) {
-        const int c = t & 63;
-        if (c < sz) A[(long long)(j0 + r) * l + j0 + c] = tile[r][c];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < HB; ++k) tile[i][c0 + k] = (c0 + k <= i) ? x[k] : 0.0f;
-    __syncthreads();
-    for (int r = t >> 6; r < sz; r += 2) {
-        const int c = t & 63;
-        if (c < sz) X[(long long)(j0 + r) * l + j0 + c] = tile[r][c];
-    }
-    if (t == 0 && s_fail && b.fail[pi] != nullptr) *b.fail[pi] = 1;
-}
-
-cudaError_t launch_chol_diag(const SmallBatch& b, int j0, cudaStream_t s, int64_t* launches) {
-    if (b.count <= 0) return cudaSuccess;
-    k_chol_diag<<<b.count, 128, 0, s>>>(b, j0);
-    ++*launches;
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

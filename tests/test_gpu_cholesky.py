@@ -1,0 +1,43 @@
+"""The refresh's blocked Cholesky and superblock inverse at sketch widths l
+around its tiles: below, at and past one 64-column block, several blocks, the
+512-column superblock and the levels of the inverse past it.  The projector's
+r columns come through sixteen (bf16: two or more per product) such
+factorisations, so orthonormality to 1e-5 and the leading singular vectors of
+a spectrum with clear gaps (ratio 0.8 down to a noise floor) pin them."""
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("bf16,l", [(False, 1), (False, 2), (False, 63), (False, 64), (False, 65), (False, 130),
+                                    (False, 511), (False, 512), (False, 513), (False, 579), (False, 640),
+                                    (True, 72), (True, 512), (True, 520), (True, 1032)])
+def test_refresh_sketch_widths(bf16, l):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_15037_gb300 as M
+    m, n = (1152, 1100) if l > 640 else (704, 656)
+    n = n // 8 * 8
+    r = 1 if l < 8 else 8
+    u, v = synth.lowrank_factors(m, n, 24, seed=l)
+    G = (u * (10.0 * 0.8 ** np.arange(24))) @ v.T
+    G += 0.01 / np.sqrt(n) * np.random.default_rng(l).standard_normal((m, n))
+    G = synth.to_bf16_exact(G) if bf16 else G.astype(np.float32).astype(np.float64)
+    g = M.MoaraGroup(block_size=64, decompose=0, oversample=l - r)
+    g.add(m, n, r, "bf16" if bf16 else "f32")
+    t = torch.tensor(G, dtype=torch.float32).cuda()
+    g.refresh([t.to(torch.bfloat16) if bf16 else t])
+    torch.cuda.synchronize()
+    assert g.status() == 0
+    P = g.modules[0].P.double().cpu().numpy()
+    g.close()
+    assert np.abs(P.T @ P - np.eye(r)).max() <= 1e-5
+    U = np.linalg.svd(G, full_matrices=False)[0][:, :r]
+    if l >= 8:      # a one- or two-column sketch holds a mixture of close directions
+        assert np.min(np.abs(np.sum(P * U, axis=0))) >= 0.9999
