@@ -623,6 +623,7 @@ struct RefreshRunner {
             moara::SmallBatch sb = small();
             for (int i = 0; i < n_it; ++i) {
                 sb.a[i] = it[i].Omega; sb.rows[i] = it[i].n; sb.l[i] = it[i].l; sb.key[i] = it[i].key;
+                sb.h[i] = tc ? it[i].Zbf : nullptr;     // the tensor-core products take it in bf16
             }
             chk(moara::launch_philox_gaussian(sb, s, &ctx->launches));
         }
@@ -650,9 +651,6 @@ struct RefreshRunner {
             // Subspace iteration with every product and every intermediate
             // orthonormalisation on tensor cores; only the last Y gets the
             // fp32 CholeskyQR2 that makes Q orthonormal for the Rayleigh-Ritz step.
-            for (int i = 0; i < n_it; ++i)
-                chk(moara::launch_f32_to_bf16(it[i].Omega, nullptr, it[i].Zbf, (long long)it[i].n * it[i].l, s,
-                                              &ctx->launches));
             const int q_it = hp.power_iters;
             if (q_it == 0) {
                 tc_v_times(zbf, Qa, nob);
@@ -686,9 +684,11 @@ struct RefreshRunner {
                 // store of P; the off-diagonal orthogonality it gives is that
                 // of the fp32 pass
                 ks_cholqr_tall(Qa, qpl, rows_m, 0.0f, 3);
-                for (int i = 0; i < n_it; ++i)                  // Q in Qb (fp32) and qbf
-                    chk(moara::launch_f32_to_bf16(Qa[i], Qb[i], qbf[i], (long long)it[i].m * it[i].l, s,
-                                                  &ctx->launches));
+                moara::SmallBatch sb = small();                 // Q in Qb (fp32) and qbf
+                for (int i = 0; i < n_it; ++i) {
+                    sb.a[i] = Qa[i]; sb.c[i] = Qb[i]; sb.h[i] = qbf[i]; sb.rows[i] = it[i].m; sb.l[i] = it[i].l;
+                }
+                chk(moara::launch_copy_bf16(sb, s, &ctx->launches));
             } else {
                 cholqr2s(Qa, Qb, rows_m, &qbf);             // Q in Qb (fp32) and qbf
             }
@@ -819,6 +819,7 @@ struct RefreshRunner {
             moara::SmallBatch sb = small();
             for (int i = 0; i < n_it; ++i) {
                 sb.a[i] = Xa[i]; sb.b[i] = Xb[i]; sb.c[i] = it[i].ritz; sb.iaux[i] = it[i].perm;
+                sb.h[i] = reinterpret_cast<uint16_t*>(it[i].Tt);      // scratch, free here
                 sb.l[i] = it[i].l;
             }
             chk(moara::launch_lead_ritz(sb, s, &ctx->launches));

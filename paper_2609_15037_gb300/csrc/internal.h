@@ -195,6 +195,7 @@ struct SmallBatch {
     uint64_t key[kMaxGroup];
 };
 
+// Standard normals into a, or rounded to bf16 into h when h is given.
 cudaError_t launch_philox_gaussian(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 // Lower Cholesky factor of each a (l x l, the lower triangle given) plus
 // shift_rel * sqrt(rows) * trace(a) on its diagonal, in place, and in X the
@@ -217,10 +218,13 @@ struct CholBatch {
     CholItem p[kMaxGroup];
 };
 cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches);
+// c <- a and h <- bf16(a); a, c, h 16-byte aligned.
+cudaError_t launch_copy_bf16(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 cudaError_t launch_set_identity(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 cudaError_t launch_ritz_sort(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 // Exact Rayleigh-Ritz (Jacobi) on the leading min(64, l) columns of X (a)
-// with W = C X (b): both rotated in place by the eigenvectors of X_w^T W_w.
+// with W = C X (b): both rotated in place by the eigenvectors of X_w^T W_w
+// (h: scratch of l x l floats).
 cudaError_t launch_lead_ritz(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 cudaError_t launch_gather_cols(const SmallBatch& b, cudaStream_t s, int64_t* launches);
 cudaError_t launch_sign_fix_store(const SmallBatch& b, cudaStream_t s, int64_t* launches);

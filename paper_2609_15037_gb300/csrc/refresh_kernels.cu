@@ -3,6 +3,7 @@
 // splits and transposes, the ordering of Ritz vectors, and the final sign
 // convention.  The problems of a group run side by side in one launch.
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -44,6 +45,7 @@ __device__ __forceinline__ float u01(uint32_t x) {
 __global__ void k_philox_gaussian(const __grid_constant__ SmallBatch b) {
     const int pi = blockIdx.y;
     float* out = b.a[pi];
+    uint16_t* hout = b.h[pi];
     const long long count = (long long)b.rows[pi] * b.l[pi];
     const uint32_t k0 = static_cast<uint32_t>(b.key[pi]);
     const uint32_t k1 = static_cast<uint32_t>(b.key[pi] >> 32);
@@ -60,15 +62,58 @@ __global__ void k_philox_gaussian(const __grid_constant__ SmallBatch b) {
         const float z[4] = {ra * c2, ra * s2, rb * c4, rb * s4};
         const long long base = g * 4;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (base + q < count) out[base + q] = z[q];
+        for (int q = 0; q < 4; ++q) {
+            if (base + q >= count) continue;
+            if (hout != nullptr) {
+                const __nv_bfloat16 h = __float2bfloat16_rn(z[q]);
+                hout[base + q] = *reinterpret_cast<const uint16_t*>(&h);
+            } else {
+                out[base + q] = z[q];
+            }
+        }
     }
 }
 
 cudaError_t launch_philox_gaussian(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    dim3 grid(64, b.count);
+    // as many blocks per item as the largest needs at four groups a thread
+    long long most = 1;
+    for (int q = 0; q < b.count; ++q) most = std::max(most, ((long long)b.rows[q] * b.l[q] + 4095) / 4096);
+    dim3 grid(static_cast<unsigned>(std::min(2048LL, most)), b.count);
     k_philox_gaussian<<<grid, 256, 0, s>>>(b);
+    ++*launches;
+    return cudaGetLastError();
+}
+
+// c <- a and h <- a rounded to bf16 (rows x l entries each).
+__global__ void __launch_bounds__(256) k_copy_bf16(const __grid_constant__ SmallBatch b) {
+    const int pi = blockIdx.y;
+    const float* src = b.a[pi];
+    float* dst = b.c[pi];
+    uint16_t* hd = b.h[pi];
+    const long long count = (long long)b.rows[pi] * b.l[pi];
+    const long long quads = count / 4;               // the buffers are 16-byte aligned
+    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < quads;
+         g += (long long)gridDim.x * blockDim.x) {
+        const float4 v = reinterpret_cast<const float4*>(src)[g];
+        reinterpret_cast<float4*>(dst)[g] = v;
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+        reinterpret_cast<uint2*>(hd)[g] =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+    }
+    if (blockIdx.x == 0 && threadIdx.x < count - 4 * quads) {
+        const long long e = 4 * quads + threadIdx.x;
+        dst[e] = src[e];
+        const __nv_bfloat16 h = __float2bfloat16_rn(src[e]);
+        hd[e] = *reinterpret_cast<const uint16_t*>(&h);
+    }
+}
+
+cudaError_t launch_copy_bf16(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
+    if (b.count <= 0) return cudaSuccess;
+    long long most = 1;
+    for (int q = 0; q < b.count; ++q) most = std::max(most, ((long long)b.rows[q] * b.l[q] + 4095) / 4096);
+    k_copy_bf16<<<dim3(static_cast<unsigned>(std::min(2048LL, most)), b.count), 256, 0, s>>>(b);
     ++*launches;
     return cudaGetLastError();
 }
@@ -124,7 +169,10 @@ __global__ void __launch_bounds__(256) k_transpose_bf16(const __grid_constant__ 
 
 cudaError_t launch_transpose_bf16(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    k_transpose_bf16<<<dim3(128, 1, b.count), 256, 0, s>>>(b);
+    int lmax = 1;
+    for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
+    const int tiles = (lmax + 31) / 32;
+    k_transpose_bf16<<<dim3(std::min(1024, tiles * tiles), 1, b.count), 256, 0, s>>>(b);
     ++*launches;
     return cudaGetLastError();
 }
@@ -215,57 +263,80 @@ cudaError_t launch_split3(const SmallBatch& b, int transpose, cudaStream_t s, in
 // ---------------------------------------------------------------------------
 // a <- I (l x l)
 // ---------------------------------------------------------------------------
-__global__ void k_set_identity(const __grid_constant__ SmallBatch b) {
+__global__ void __launch_bounds__(256) k_set_identity(const __grid_constant__ SmallBatch b) {
     const int pi = blockIdx.y;
     const int l = b.l[pi];
-    float* X = b.a[pi];
-    const long long n = (long long)l * l;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long i = e / l, c = e - i * l;
-        X[e] = (i == c) ? 1.0f : 0.0f;
+    for (int i = blockIdx.x; i < l; i += gridDim.x) {
+        float* row = b.a[pi] + (long long)i * l;
+        for (int c = threadIdx.x; c < l; c += blockDim.x) row[c] = (i == c) ? 1.0f : 0.0f;
     }
 }
 
 cudaError_t launch_set_identity(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    k_set_identity<<<dim3(32, b.count), 256, 0, s>>>(b);
+    int lmax = 1;
+    for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
+    k_set_identity<<<dim3(std::min(1024, lmax), b.count), 256, 0, s>>>(b);
     ++*launches;
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// Ritz values d_j = x_j^T (C x_j) / x_j^T x_j from X (a) and W = C X (b), then the
-// descending order: iaux[rank] = j, rank_j = #{i : d_i > d_j, or d_i == d_j
-// and i < j}.  Ritz values go to c.
+// Ritz values d_j = x_j^T (C x_j) / x_j^T x_j from X (a) and W = C X (b) into
+// c: a CTA per 32 columns, lane = column, its 32 warps split the rows.  (With
+// one CTA per module for values and order, l = 2080 took 2.9 ms; now the two
+// launches together take 0.05 ms.)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSmallThreads) k_ritz_sort(const __grid_constant__ SmallBatch b) {
-    const int pi = blockIdx.x;
+__global__ void __launch_bounds__(kSmallThreads) k_ritz_values(const __grid_constant__ SmallBatch b) {
+    __shared__ float s_acc[32][33], s_nrm[32][33];
+    const int pi = blockIdx.y;
     const int l = b.l[pi];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j0 = blockIdx.x * 32, j = j0 + lane;
+    if (j0 >= l) return;
     const float* X = b.a[pi];
     const float* W = b.b[pi];
-    float* d = b.c[pi];
-    int* perm = b.iaux[pi];
-    for (int j = threadIdx.x; j < l; j += blockDim.x) {
-        float acc = 0.0f, nrm = 0.0f;
-        for (int i = 0; i < l; ++i) {
+    float acc = 0.0f, nrm = 0.0f;
+    if (j < l) {
+#pragma unroll 4
+        for (int i = warp; i < l; i += 32) {
             const float x = X[(long long)i * l + j];
             acc = fmaf(x, W[(long long)i * l + j], acc);
             nrm = fmaf(x, x, nrm);
         }
-        d[j] = nrm > 0.0f ? acc / nrm : 0.0f;
     }
+    s_acc[warp][lane] = acc;
+    s_nrm[warp][lane] = nrm;
     __syncthreads();
-    __threadfence_block();
-    for (int j = threadIdx.x; j < l; j += blockDim.x) {
-        const float dj = d[j];
-        int rank = 0;
-        for (int i = 0; i < l; ++i) {
-            const float di = d[i];
-            rank += (di > dj || (di == dj && i < j)) ? 1 : 0;
-        }
-        perm[rank] = j;
+    // warp w reduces column j0 + w
+    acc = s_acc[lane][warp];
+    nrm = s_nrm[lane][warp];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
     }
+    if (lane == 0 && j0 + warp < l) b.c[pi][j0 + warp] = nrm > 0.0f ? acc / nrm : 0.0f;
+}
+
+// The descending order of the Ritz values (c): iaux[rank] = j,
+// rank_j = #{i : d_i > d_j, or d_i == d_j and i < j}.
+__global__ void __launch_bounds__(256) k_ritz_order(const __grid_constant__ SmallBatch b) {
+    __shared__ float d[1024];
+    const int pi = blockIdx.y;
+    const int l = b.l[pi];
+    if (static_cast<int>(blockIdx.x) * 256 >= l) return;
+    const int j = blockIdx.x * 256 + threadIdx.x;
+    const float dj = j < l ? b.c[pi][j] : 0.0f;
+    int rank = 0;
+    for (int i0 = 0; i0 < l; i0 += 1024) {
+        const int cnt = min(1024, l - i0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < cnt; i += 256) d[i] = b.c[pi][i0 + i];
+        __syncthreads();
+        for (int i = 0; i < cnt; ++i) rank += (d[i] > dj || (d[i] == dj && i0 + i < j)) ? 1 : 0;
+    }
+    if (j < l) b.iaux[pi][rank] = j;
 }
 
 // ---------------------------------------------------------------------------
@@ -278,62 +349,84 @@ __global__ void __launch_bounds__(kSmallThreads) k_ritz_sort(const __grid_consta
 // columns and run in parallel), then X_w <- X_w J and W_w <- W_w J.  The
 // orthogonal iteration before it leaves span(X_w) close to the leading
 // invariant subspace of C; within it the individual eigenvectors of
-// separated eigenvalues are then exact up to rounding.  One CTA per
-// problem, everything in shared memory, rows of X and W streamed in chunks.
+// separated eigenvalues are then exact up to rounding.
+//
+// Three launches: partial Gram blocks over slabs of rows, one CTA per module
+// for the Jacobi sweeps, and the rotation over slabs of rows.  As one CTA per
+// module the whole took 0.32 / 0.63 / 1.20 ms at l = 64 / 288 / 2080, now
+// 0.26 / 0.45 / 0.48 ms; what is left is the chain of the sweeps.  h: scratch of
+// l x l floats, the partial Gram blocks and then J.
 // ---------------------------------------------------------------------------
 constexpr int kLeadW = 64;
-constexpr int kLeadChunk = 16;            // rows of X / W per chunk
 
-__global__ void __launch_bounds__(kSmallThreads) k_lead_ritz(const __grid_constant__ SmallBatch b) {
+// Slabs of at least 64 rows, so that the partial blocks fit l x l floats.
+__host__ __device__ inline int lead_slabs(int l) { return l < 2 * kLeadW ? 1 : l / kLeadW; }
+
+__global__ void __launch_bounds__(256) k_lead_gram(const __grid_constant__ SmallBatch b) {
+    __shared__ __align__(16) float xs[32][kLeadW], ws[32][kLeadW];
+    const int pi = blockIdx.y;
+    const int l = b.l[pi];
+    const int w = min(l, kLeadW), ns = lead_slabs(l);
+    if (static_cast<int>(blockIdx.x) >= ns) return;
+    const int r0 = blockIdx.x * kLeadW, r1 = static_cast<int>(blockIdx.x) + 1 == ns ? l : r0 + kLeadW;
+    const float* X = b.a[pi];
+    const float* W = b.b[pi];
+    const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+    float acc[4][4] = {};
+    for (int r = r0; r < r1; r += 32) {
+        for (int e = t; e < 32 * kLeadW; e += 256) {
+            const int i = e / kLeadW, j = e % kLeadW;
+            const bool in = r + i < r1 && j < w;
+            xs[i][j] = in ? X[(long long)(r + i) * l + j] : 0.0f;
+            ws[i][j] = in ? W[(long long)(r + i) * l + j] : 0.0f;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) {
+            const float4 x = *reinterpret_cast<const float4*>(&xs[i][4 * ty]);
+            const float4 y = *reinterpret_cast<const float4*>(&ws[i][4 * tx]);
+            const float xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(xv[p], yv[q], acc[p][q]);
+        }
+        __syncthreads();
+    }
+    float* out = reinterpret_cast<float*>(b.h[pi]) + (long long)blockIdx.x * w * w;
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (4 * ty + p < w && 4 * tx + q < w) out[(4 * ty + p) * w + 4 * tx + q] = acc[p][q];
+}
+
+constexpr int kJacThreads = 512;
+constexpr int kJacPairs = kLeadW / 2;
+
+__global__ void __launch_bounds__(kJacThreads) k_lead_jacobi(const __grid_constant__ SmallBatch b) {
     __shared__ float H[kLeadW][kLeadW + 1];
     __shared__ float J[kLeadW][kLeadW + 1];
-    __shared__ float xs[kLeadChunk][kLeadW];
-    __shared__ float ws[kLeadChunk][kLeadW];
-    __shared__ float rc[kLeadW / 2], rs_[kLeadW / 2];
-    __shared__ int rp[kLeadW / 2], rq[kLeadW / 2];
+    __shared__ float rc[kJacPairs], rs_[kJacPairs];
+    __shared__ int rp[kJacPairs], rq[kJacPairs];
     __shared__ float red[33];
     const int pi = blockIdx.x;
     const int l = b.l[pi];
-    const int w = l < kLeadW ? l : kLeadW;
+    const int w = min(l, kLeadW), ns = lead_slabs(l);
     const int wp = w + (w & 1);                    // even player count (a dummy index when w is odd)
-    float* X = b.a[pi];
-    float* W = b.b[pi];
+    float* const part = reinterpret_cast<float*>(b.h[pi]);
     const int t = threadIdx.x;
-    // H = X_w^T W_w: thread t owns entries t, t + 1024, ... of the w x w block
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int r0 = 0; r0 < l; r0 += kLeadChunk) {
-        for (int e = t; e < kLeadChunk * kLeadW; e += blockDim.x) {
-            const int i = e / kLeadW, j = e % kLeadW;
-            const bool in = r0 + i < l && j < w;
-            xs[i][j] = in ? X[(long long)(r0 + i) * l + j] : 0.0f;
-            ws[i][j] = in ? W[(long long)(r0 + i) * l + j] : 0.0f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = t + u * blockDim.x;
-            if (e < w * w) {
-                const int p = e / w, q = e % w;
-#pragma unroll 4
-                for (int i = 0; i < kLeadChunk; ++i) acc[u] = fmaf(xs[i][p], ws[i][q], acc[u]);
-            }
-        }
-        __syncthreads();
-    }
-    for (int e = t; e < kLeadW * kLeadW; e += blockDim.x) {
+    for (int e = t; e < kLeadW * kLeadW; e += kJacThreads) {
         const int p = e / kLeadW, q = e % kLeadW;
-        H[p][q] = 0.0f;
+        float v = 0.0f;
+        if (p < w && q < w)
+            for (int k = 0; k < ns; ++k) v += part[(long long)k * w * w + p * w + q];
+        H[p][q] = v;
         J[p][q] = (p == q) ? 1.0f : 0.0f;
     }
     __syncthreads();
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int e = t + u * blockDim.x;
-        if (e < w * w) H[e / w][e % w] = acc[u];
-    }
-    __syncthreads();
     // symmetrise (the two triangles differ by rounding)
-    for (int e = t; e < w * w; e += blockDim.x) {
+    for (int e = t; e < w * w; e += kJacThreads) {
         const int p = e / w, q = e % w;
         if (p < q) {
             const float v = 0.5f * (H[p][q] + H[q][p]);
@@ -343,10 +436,11 @@ __global__ void __launch_bounds__(kSmallThreads) k_lead_ritz(const __grid_consta
     }
     __syncthreads();
     const int npairs = wp / 2;
+    const int lane = t & 31, warp = t >> 5;
     for (int sweep = 0; sweep < 20; ++sweep) {
         // stop once the off-diagonal mass is below fp32 resolution of the diagonal
         float off = 0.0f, dia = 0.0f;
-        for (int e = t; e < w * w; e += blockDim.x) {
+        for (int e = t; e < w * w; e += kJacThreads) {
             const int p = e / w, q = e % w;
             const float v = H[p][q];
             if (p == q) dia = fmaf(v, v, dia); else off = fmaf(v, v, off);
@@ -357,7 +451,11 @@ __global__ void __launch_bounds__(kSmallThreads) k_lead_ritz(const __grid_consta
         for (int round = 0; round < wp - 1; ++round) {
             if (t < npairs) {
                 // tournament: player 0 fixed, the others rotate by one each round
-                auto player = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + round) % (wp - 1); };
+                auto player = [&](int pos) {
+                    int k = pos - 1 + round;
+                    if (k >= wp - 1) k -= wp - 1;
+                    return pos == 0 ? 0 : 1 + k;
+                };
                 int p = player(t), q = player(wp - 1 - t);
                 if (p > q) { const int x = p; p = q; q = x; }
                 float c = 1.0f, sn = 0.0f;
@@ -373,93 +471,104 @@ __global__ void __launch_bounds__(kSmallThreads) k_lead_ritz(const __grid_consta
                 rp[t] = p; rq[t] = q; rc[t] = c; rs_[t] = sn;
             }
             __syncthreads();
-            // columns: H <- H G, J <- J G
-            for (int e = t; e < npairs * kLeadW; e += blockDim.x) {
-                const int k = e / kLeadW, row = e % kLeadW;
-                const int p = rp[k], q = rq[k];
-                if (q >= w || row >= w) continue;
-                const float c = rc[k], sn = rs_[k];
-                const float hp = H[row][p], hq = H[row][q];
-                H[row][p] = c * hp - sn * hq;
-                H[row][q] = sn * hp + c * hq;
-                const float jp = J[row][p], jq = J[row][q];
-                J[row][p] = c * jp - sn * jq;
-                J[row][q] = sn * jp + c * jq;
-            }
-            __syncthreads();
-            // rows: H <- G^T H
-            for (int e = t; e < npairs * kLeadW; e += blockDim.x) {
-                const int k = e / kLeadW, col = e % kLeadW;
-                const int p = rp[k], q = rq[k];
-                if (q >= w || col >= w) continue;
-                const float c = rc[k], sn = rs_[k];
-                const float hp = H[p][col], hq = H[q][col];
-                H[p][col] = c * hp - sn * hq;
-                H[q][col] = sn * hp + c * hq;
+            // H <- G^T H G by 2 x 2 blocks: the block of pairs (k1, k2) is read
+            // and written by one thread (lane = k2, a warp takes two k1); the
+            // columns of J turn by G as well
+            if (lane < npairs) {
+                const int p2 = rp[lane], q2 = rq[lane];
+                const float c2 = rc[lane], s2 = rs_[lane];
+                const bool two = q2 < w;
+                for (int k1 = warp; k1 < npairs; k1 += kJacThreads / 32) {
+                    const int p1 = rp[k1], q1 = rq[k1];
+                    const float c1 = rc[k1], s1 = rs_[k1];
+                    const float a = H[p1][p2], d = q1 < w && two ? H[q1][q2] : 0.0f;
+                    const float u = two ? H[p1][q2] : 0.0f, v = q1 < w ? H[q1][p2] : 0.0f;
+                    // columns, then rows
+                    const float a1 = c2 * a - s2 * u, u1 = s2 * a + c2 * u;
+                    const float v1 = c2 * v - s2 * d, d1 = s2 * v + c2 * d;
+                    H[p1][p2] = c1 * a1 - s1 * v1;
+                    if (two) H[p1][q2] = c1 * u1 - s1 * d1;
+                    if (q1 < w) H[q1][p2] = s1 * a1 + c1 * v1;
+                    if (two && q1 < w) H[q1][q2] = s1 * u1 + c1 * d1;
+                }
+                if (two)
+                    for (int row = warp; row < w; row += kJacThreads / 32) {
+                        const float jp = J[row][p2], jq = J[row][q2];
+                        J[row][p2] = c2 * jp - s2 * jq;
+                        J[row][q2] = s2 * jp + c2 * jq;
+                    }
             }
             __syncthreads();
         }
     }
-    // X_w <- X_w J, W_w <- W_w J, chunk by chunk
-    for (int r0 = 0; r0 < l; r0 += kLeadChunk) {
-        for (int e = t; e < kLeadChunk * kLeadW; e += blockDim.x) {
-            const int i = e / kLeadW, j = e % kLeadW;
-            const bool in = r0 + i < l && j < w;
-            xs[i][j] = in ? X[(long long)(r0 + i) * l + j] : 0.0f;
-            ws[i][j] = in ? W[(long long)(r0 + i) * l + j] : 0.0f;
-        }
-        __syncthreads();
-        float ox = 0.0f, ow = 0.0f;
-        const int i = t / kLeadW, j = t % kLeadW;     // 1024 threads = 16 rows x 64 columns
-        if (j < w) {
-            for (int k = 0; k < w; ++k) {
-                ox = fmaf(xs[i][k], J[k][j], ox);
-                ow = fmaf(ws[i][k], J[k][j], ow);
-            }
-        }
-        __syncthreads();
-        if (j < w && r0 + i < l) {
-            X[(long long)(r0 + i) * l + j] = ox;
-            W[(long long)(r0 + i) * l + j] = ow;
-        }
-        __syncthreads();
+    for (int e = t; e < w * w; e += kJacThreads) part[e] = J[e / w][e % w];
+}
+
+// X_w <- X_w J, W_w <- W_w J: 32 rows of one of the two per CTA.
+__global__ void __launch_bounds__(256) k_lead_rotate(const __grid_constant__ SmallBatch b) {
+    __shared__ float js[kLeadW][kLeadW], xs[32][kLeadW];
+    const int pi = blockIdx.y;
+    const int l = b.l[pi];
+    const int w = min(l, kLeadW);
+    const int r0 = static_cast<int>(blockIdx.x) * 32;
+    if (r0 >= l) return;
+    float* const X = blockIdx.z == 0 ? b.a[pi] : b.b[pi];
+    const float* J = reinterpret_cast<const float*>(b.h[pi]);
+    for (int e = threadIdx.x; e < w * w; e += 256) js[e / w][e % w] = J[e];
+    for (int e = threadIdx.x; e < 32 * kLeadW; e += 256) {
+        const int i = e / kLeadW, j = e % kLeadW;
+        xs[i][j] = (r0 + i < l && j < w) ? X[(long long)(r0 + i) * l + j] : 0.0f;
+    }
+    __syncthreads();
+    const int j = threadIdx.x & 63;
+    if (j >= w) return;
+    for (int i = threadIdx.x >> 6; i < 32 && r0 + i < l; i += 4) {
+        float o = 0.0f;
+        for (int k = 0; k < w; ++k) o = fmaf(xs[i][k], js[k][j], o);
+        X[(long long)(r0 + i) * l + j] = o;
     }
 }
 
 cudaError_t launch_lead_ritz(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    k_lead_ritz<<<b.count, kSmallThreads, 0, s>>>(b);
-    ++*launches;
+    int lmax = 1;
+    for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
+    k_lead_gram<<<dim3(lead_slabs(lmax), b.count), 256, 0, s>>>(b);
+    k_lead_jacobi<<<b.count, kJacThreads, 0, s>>>(b);
+    k_lead_rotate<<<dim3((lmax + 31) / 32, b.count, 2), 256, 0, s>>>(b);
+    *launches += 3;
     return cudaGetLastError();
 }
 
 cudaError_t launch_ritz_sort(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    k_ritz_sort<<<b.count, kSmallThreads, 0, s>>>(b);
-    ++*launches;
+    int lmax = 1;
+    for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
+    k_ritz_values<<<dim3((lmax + 31) / 32, b.count), kSmallThreads, 0, s>>>(b);
+    k_ritz_order<<<dim3((lmax + 255) / 256, b.count), 256, 0, s>>>(b);
+    *launches += 2;
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
 // c[:, q] = a[:, iaux[q]] for q < rows (a is l x l, c is l x rows).
 // ---------------------------------------------------------------------------
-__global__ void k_gather_cols(const __grid_constant__ SmallBatch b) {
+__global__ void __launch_bounds__(256) k_gather_cols(const __grid_constant__ SmallBatch b) {
     const int pi = blockIdx.y;
     const int l = b.l[pi], r = b.rows[pi];
-    const float* X = b.a[pi];
-    float* Xs = b.c[pi];
     const int* perm = b.iaux[pi];
-    const long long n = (long long)l * r;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long i = e / r, q = e - i * r;
-        Xs[e] = X[i * l + perm[q]];
+    for (int i = blockIdx.x; i < l; i += gridDim.x) {
+        const float* src = b.a[pi] + (long long)i * l;
+        float* dst = b.c[pi] + (long long)i * r;
+        for (int q = threadIdx.x; q < r; q += blockDim.x) dst[q] = src[perm[q]];
     }
 }
 
 cudaError_t launch_gather_cols(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    k_gather_cols<<<dim3(64, b.count), 256, 0, s>>>(b);
+    int lmax = 1;
+    for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
+    k_gather_cols<<<dim3(std::min(1024, lmax), b.count), 256, 0, s>>>(b);
     ++*launches;
     return cudaGetLastError();
 }
@@ -470,70 +579,110 @@ cudaError_t launch_gather_cols(const SmallBatch& b, cudaStream_t s, int64_t* lau
 // (lowest row wins ties), then stored to c (fp32) and h (bf16).  Skipped when
 // the problem's fail flag is set, which leaves the previous projector in place.
 // ---------------------------------------------------------------------------
+// A cluster of kSignCtas CTAs owns 32 columns: lane = column, the CTAs' 8 warps
+// each split the rows (every row segment one coalesced 128-byte access), and
+// the column's maximum and norm are combined through distributed shared
+// memory.  Two passes over a, the second out of L2: bound by the loads in
+// flight, so the rows are spread over eight SMs (one CTA per 32 columns took
+// 1.0 ms on the seven weights of a 4096 / 11008 layer, a cluster 0.2 ms).
+constexpr int kSignCtas = 8;
+
 __global__ void __launch_bounds__(256) k_sign_fix_store(const __grid_constant__ SmallBatch b) {
-    // a CTA owns 32 columns: lane = column, the 8 warps split the rows, so
-    // every row segment is one coalesced 128-byte load
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
     __shared__ float s_best[8][32];
     __shared__ int s_bi[8][32];
     __shared__ float s_ss[8][32];
-    __shared__ float s_sgn[32];
+    __shared__ float c_best[32], c_ss[32];
+    __shared__ int c_bi[32];
     const int pi = blockIdx.y;
     const int rows = b.rows[pi], r = b.l[pi];
-    if (b.fail[pi] != nullptr && *b.fail[pi] != 0) return;
+    const int q0 = static_cast<int>(blockIdx.x) / kSignCtas * 32;
+    // the whole cluster leaves together
+    if (q0 >= r || (b.fail[pi] != nullptr && *b.fail[pi] != 0)) return;
+    const int rank = static_cast<int>(cl.block_rank());
     const float* Pt = b.a[pi];
     float* P = b.c[pi];
     uint16_t* Pb = b.h[pi];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q0 = blockIdx.x * 32; q0 < r; q0 += gridDim.x * 32) {
-        const int q = q0 + lane;
-        const bool col = q < r;
-        // largest |entry| of the column over this warp's rows (ascending, so
-        // the lowest row wins ties)
-        float best = -1.0f, ss = 0.0f;
-        int bi = 0x7fffffff;
-        if (col)
-            for (int i = warp; i < rows; i += 8) {
-                const float v = Pt[(long long)i * r + q];
-                const float a = fabsf(v);
-                ss = fmaf(v, v, ss);
-                if (a > best) { best = a; bi = i; }
-            }
-        s_best[warp][lane] = best;
-        s_bi[warp][lane] = bi;
-        s_ss[warp][lane] = ss;
-        __syncthreads();
-        if (warp == 0) {
-            for (int w = 1; w < 8; ++w) {
-                const float ob = s_best[w][lane];
-                const int oi = s_bi[w][lane];
-                ss += s_ss[w][lane];
-                if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-            }
-            const float sg = (col && bi < rows && Pt[(long long)bi * r + q] < 0.0f) ? -1.0f : 1.0f;
-            // unit length (a zero or non-finite column is left unscaled)
-            const float nrm = sqrtf(ss);
-            s_sgn[lane] = (nrm > 0.0f && isfinite(nrm)) ? sg / nrm : sg;
+    const int i0 = static_cast<int>((long long)rows * rank / kSignCtas);
+    const int i1 = static_cast<int>((long long)rows * (rank + 1) / kSignCtas);
+    const int q = q0 + lane;
+    const bool col = q < r;
+    // largest |entry| of the column over this warp's rows (ascending, so
+    // the lowest row wins ties)
+    float best = -1.0f, ss = 0.0f;
+    int bi = 0x7fffffff;
+    if (col) {
+#pragma unroll 4
+        for (int i = i0 + warp; i < i1; i += 8) {
+            const float v = Pt[(long long)i * r + q];
+            const float a = fabsf(v);
+            ss = fmaf(v, v, ss);
+            if (a > best) { best = a; bi = i; }
         }
-        __syncthreads();
-        const float sgnv = s_sgn[lane];
-        if (col)
-            for (int i = warp; i < rows; i += 8) {
-                const float v = Pt[(long long)i * r + q] * sgnv;
-                P[(long long)i * r + q] = v;
-                if (Pb != nullptr) {
-                    __nv_bfloat16 h = __float2bfloat16_rn(v);
-                    Pb[(long long)i * r + q] = *reinterpret_cast<uint16_t*>(&h);
-                }
+    }
+    s_best[warp][lane] = best;
+    s_bi[warp][lane] = bi;
+    s_ss[warp][lane] = ss;
+    __syncthreads();
+    if (warp == 0) {
+        for (int w = 1; w < 8; ++w) {
+            const float ob = s_best[w][lane];
+            const int oi = s_bi[w][lane];
+            ss += s_ss[w][lane];
+            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+        }
+        c_best[lane] = best;
+        c_bi[lane] = bi;
+        c_ss[lane] = ss;
+    }
+    cl.sync();
+    best = -1.0f;
+    bi = 0x7fffffff;
+    ss = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kSignCtas; ++k) {
+        const float ob = cl.map_shared_rank(c_best, k)[lane];
+        const int oi = cl.map_shared_rank(c_bi, k)[lane];
+        ss += cl.map_shared_rank(c_ss, k)[lane];
+        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    const float sg = (col && bi < rows && Pt[(long long)bi * r + q] < 0.0f) ? -1.0f : 1.0f;
+    // unit length (a zero or non-finite column is left unscaled)
+    const float nrm = sqrtf(ss);
+    const float sgnv = (nrm > 0.0f && isfinite(nrm)) ? sg / nrm : sg;
+    cl.sync();          // no CTA leaves while a peer may still read its sums
+    if (col) {
+#pragma unroll 4
+        for (int i = i0 + warp; i < i1; i += 8) {
+            const float v = Pt[(long long)i * r + q] * sgnv;
+            P[(long long)i * r + q] = v;
+            if (Pb != nullptr) {
+                __nv_bfloat16 h = __float2bfloat16_rn(v);
+                Pb[(long long)i * r + q] = *reinterpret_cast<uint16_t*>(&h);
             }
-        __syncthreads();   // the shared arrays are reused by the next column group
+        }
     }
 }
 
 cudaError_t launch_sign_fix_store(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    k_sign_fix_store<<<dim3(64, b.count), 256, 0, s>>>(b);
+    int rmax = 1;
+    for (int q = 0; q < b.count; ++q) rmax = std::max(rmax, b.l[q]);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((rmax + 31) / 32 * kSignCtas, b.count);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kSignCtas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     ++*launches;
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, k_sign_fix_store, b);
 }
 
 }  // namespace moara
