@@ -93,17 +93,20 @@ struct GemmProb {
     uint16_t* c_bf16;     // EPI_STORE: also write C rounded to bf16 here (same layout), or null
 };
 
-struct GemmBatch {
+template <int CAP>
+struct GemmBatchT {
     int count;
     int B;                        // block size (scales, dM repetition)
     int log2B;                    // log2(B) when B is a power of two, else -1 (set at launch)
     float beta1, beta2, adam_eps, bc1, bc2;
     float step_scale;             // lr * alpha (EPI_UPDATE)
     const float* clip;            // EPI_ADAM: clipping coefficient (device) applied to R, or null
-    int tiles_n[kMaxGroup];
-    int tile_start[kMaxGroup + 1];
-    GemmProb p[kMaxGroup];
+    int tiles_n[CAP];
+    int tile_start[CAP + 1];
+    GemmProb p[CAP];
 };
+using GemmBatch = GemmBatchT<kMaxGroup>;
+constexpr int kFewGroup = 8;          // problems that a launch with a small parameter block carries
 
 // Operand layouts of the SIMT GEMM.
 //   A: KCONTIG  A[i][k] = A[i*lda + k];  MCONTIG  A[i][k] = A[k*lda + i]
@@ -118,8 +121,6 @@ struct GemmKind {
 // Host launchers (return cudaError_t of the launch).
 cudaError_t launch_decompose(const DecompBatch& b, cudaStream_t s, int64_t* launches);
 cudaError_t launch_gemm(const GemmKind& kind, GemmBatch& b, cudaStream_t s, int64_t* launches);
-int gemm_tile_m();
-int gemm_tile_n();
 
 cudaError_t launch_f32_to_bf16(const float* src, float* dst_f32, uint16_t* dst_bf16,
                                long long count, cudaStream_t s, int64_t* launches);

@@ -1,8 +1,10 @@
 // fp32 SIMT kernels of the step: block decomposition with the magnitude
-// branch's Adam, and a grouped tiled GEMM whose operand loaders apply the
-// block scales of the decomposition and whose epilogues run the direction
-// branch's Adam or the weight update.  Every product is an fp32 FMA, so this
+// branch's Adam, and grouped tiled GEMMs (128 x 128 tiles, or 64 x 64 tiles
+// with a split K range) whose operand loaders apply the block scales of the
+// decomposition and whose epilogues run the direction branch's Adam or the
+// weight update.  Every product is an fp32 FMA, so this
 // path meets the all-fp32 tolerance; it also serves the refresh.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -127,9 +129,6 @@ cudaError_t launch_decompose(const DecompBatch& b, cudaStream_t s, int64_t* laun
 constexpr int TM = 128, TN = 128, TK = 16, TPAD = 4;
 constexpr int NQ = TK * 128 / 256;   // elements of A (and of B) each thread stages per k-tile
 
-int gemm_tile_m() { return TM; }
-int gemm_tile_n() { return TN; }
-
 // Index of the block holding column c: a shift when B is a power of two.
 __device__ __forceinline__ int block_of(int c, int B, int log2B) { return log2B >= 0 ? (c >> log2B) : c / B; }
 
@@ -194,8 +193,8 @@ struct TileLoader {
     }
 };
 
-template <int EPI>
-__device__ __forceinline__ void epilogue(const GemmBatch& b, const GemmProb& p, int i, int j, float acc) {
+template <int EPI, int CAP>
+__device__ __forceinline__ void epilogue(const GemmBatchT<CAP>& b, const GemmProb& p, int i, int j, float acc) {
     const long long o = (long long)i * p.ldc + j;
     if (EPI == EPI_STORE) {
         p.C[o] = acc;
@@ -335,6 +334,167 @@ __global__ void __launch_bounds__(256, 2) k_gemm(const __grid_constant__ GemmBat
     }
 }
 
+// ---------------------------------------------------------------------------
+// Small variant for problems whose 128 x 128 tiles leave SMs idle: 64 x 64
+// tiles, and the K range of a tile split over the CTAs of a cluster (up to
+// eight), whose partial tiles are summed through distributed shared memory in
+// rank order; CTA q of the cluster then runs the epilogue on its 64 / S rows.
+// A 128-tile at K = 1024 is a serial chain of 64 k-tiles, each with a global
+// load latency: the projection of a 1024 x 1024 weight at r = 128 (8 tiles)
+// took 413 us, here 31 us (32 tiles x 8 CTAs, cold); of 256 x 256 at r = 32
+// (2 tiles) 122 us, here 12 us.
+// ---------------------------------------------------------------------------
+constexpr int SM_T = 64, SM_K = 32, SM_LD = SM_T + 4;
+
+// This thread's eight elements of a 32-deep, 64-wide operand slice.
+template <int LAY_K, bool SC, bool BF>
+struct SliceLoader {
+    float r[8];
+    // LAY_K: element (x, k) at x * ld + k (k contiguous): a warp takes 4 x 8
+    // (x, k) pieces, 32 bytes per row; else at k * ld + x: 32 consecutive x
+    static __device__ __forceinline__ void place(int q, int& x, int& k) {
+        const int t = threadIdx.x;
+        if (LAY_K) { k = (t & 7) + 8 * (q & 3); x = (t >> 3) + 32 * (q >> 2); }
+        else       { x = t & 63; k = (t >> 6) + 4 * q; }
+    }
+    __device__ __forceinline__ void load(const void* base, const float* inv, int ld, int kb, int x0, int X, int k0, int K,
+                                         int B, int log2B) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            int x, k;
+            place(q, x, k);
+            const int gx = x0 + x, gk = k0 + k;
+            float v = 0.0f;
+            if (gx < X && gk < K) {
+                const long long row = LAY_K ? gx : gk;
+                const int col = LAY_K ? gk : gx;
+                v = load_elem<BF>(base, row * ld + col);
+                if (SC) v *= __ldg(inv + row * kb + block_of(col, B, log2B));
+            }
+            r[q] = v;
+        }
+    }
+    __device__ __forceinline__ void store(float (*dst)[SM_LD]) const {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            int x, k;
+            place(q, x, k);
+            dst[k][x] = r[q];
+        }
+    }
+};
+
+template <int CAP, int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
+__global__ void __launch_bounds__(256, 4) k_gemm_small(const __grid_constant__ GemmBatchT<CAP> b) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ __align__(16) float As[2][SM_K][SM_LD];
+    __shared__ __align__(16) float Bs[2][SM_K][SM_LD];
+    const int S = static_cast<int>(cl.num_blocks()), rank = static_cast<int>(cl.block_rank());
+    const int tile = blockIdx.x / S;
+    int lo = 0, hi = b.count - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (b.tile_start[mid] <= tile) lo = mid; else hi = mid - 1;
+    }
+    const GemmProb& p = b.p[lo];
+    const int local = tile - b.tile_start[lo];
+    const int tn = b.tiles_n[lo];
+    const int m0 = (local / tn) * SM_T;
+    const int n0 = (local % tn) * SM_T;
+    if (p.lower_only && n0 >= m0 + SM_T) return;      // the whole cluster
+
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    float acc[4][4] = {};
+    int kbeg = 0, kend = p.K;
+    if (p.k_tri == KTRI_B_UPPER) kend = min(p.K, n0 + SM_T);
+    else if (p.k_tri == KTRI_B_LOWER) kbeg = min(p.K, n0);
+    else if (p.k_tri == KTRI_A_LOWER) kend = min(p.K, m0 + SM_T);
+    const int chunks = kend > kbeg ? (kend - kbeg + SM_K - 1) / SM_K : 0;
+    const int c0 = chunks * rank / S, c1 = chunks * (rank + 1) / S;
+    SliceLoader<ALAY == A_KCONTIG, ASC, ABF> la;
+    SliceLoader<BLAY == B_KCONTIG, BSC, BBF> lb;
+    auto load = [&](int c) {
+        const int k0 = kbeg + c * SM_K;
+        la.load(p.A, p.a_inv, p.lda, p.kb, m0, p.M, k0, kend, b.B, b.log2B);
+        lb.load(p.Bm, p.b_inv, p.ldb, p.kb, n0, p.N, k0, kend, b.B, b.log2B);
+    };
+    if (c0 < c1) load(c0);
+    for (int c = c0; c < c1; ++c) {
+        const int cur = (c - c0) & 1;
+        la.store(As[cur]);
+        lb.store(Bs[cur]);
+        __syncthreads();
+        if (c + 1 < c1) load(c + 1);
+#pragma unroll 8
+        for (int k = 0; k < SM_K; ++k) {
+            const float4 x = *reinterpret_cast<const float4*>(&As[cur][k][4 * ty]);
+            const float4 y = *reinterpret_cast<const float4*>(&Bs[cur][k][4 * tx]);
+            const float xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xv[i], yv[j], acc[i][j]);
+        }
+    }
+    // partial tiles in A's buffers, then S row slabs
+    __syncthreads();
+    float (*part)[SM_LD] = As[0];
+    static_assert(2 * SM_K == SM_T, "the partial tile fills both A slices");
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4*>(&part[4 * ty + i][4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    if (S > 1) cl.sync();
+    else __syncthreads();
+    const int R = SM_T / S;
+    for (int e = threadIdx.x; e < R * SM_T; e += 256) {
+        const int i = rank * R + e / SM_T, j = e % SM_T;
+        float v = 0.0f;
+        if (S > 1) {
+            for (int q = 0; q < S; ++q) v += *cl.map_shared_rank(&part[i][j], q);
+        } else {
+            v = part[i][j];
+        }
+        if (m0 + i < p.M && n0 + j < p.N) epilogue<EPI>(b, p, m0 + i, n0 + j, v);
+    }
+    if (S > 1) cl.sync();       // no CTA leaves while a peer may still read its partial tile
+}
+
+constexpr int kWideTiles = 304;       // two 128 x 128 tiles per SM
+constexpr int kSmallCtas = 608;       // four 64 x 64 CTAs per SM
+
+template <int CAP, int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
+static cudaError_t launch_small(const GemmBatch& b, int total, int split, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(total * split);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = split;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    auto fn = k_gemm_small<CAP, ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>;
+    if constexpr (CAP == kMaxGroup) {
+        return cudaLaunchKernelEx(&cfg, fn, b);
+    } else {
+        GemmBatchT<CAP> f;
+        f.count = b.count; f.B = b.B; f.log2B = b.log2B;
+        f.beta1 = b.beta1; f.beta2 = b.beta2; f.adam_eps = b.adam_eps; f.bc1 = b.bc1; f.bc2 = b.bc2;
+        f.step_scale = b.step_scale;
+        f.clip = b.clip;
+        for (int i = 0; i < b.count; ++i) {
+            f.tiles_n[i] = b.tiles_n[i];
+            f.tile_start[i] = b.tile_start[i];
+            f.p[i] = b.p[i];
+        }
+        f.tile_start[b.count] = b.tile_start[b.count];
+        return cudaLaunchKernelEx(&cfg, fn, f);
+    }
+}
+
 template <int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
 static cudaError_t launch_one(GemmBatch& b, cudaStream_t s, int64_t* launches) {
     b.log2B = -1;
@@ -343,20 +503,36 @@ static cudaError_t launch_one(GemmBatch& b, cudaStream_t s, int64_t* launches) {
         while ((1 << lg) < b.B) ++lg;
         b.log2B = lg;
     }
-    int total = 0;
-    for (int i = 0; i < b.count; ++i) {
-        const GemmProb& p = b.p[i];
-        const int tm = (p.M + TM - 1) / TM;
-        const int tn = (p.N + TN - 1) / TN;
-        b.tiles_n[i] = tn;
-        b.tile_start[i] = total;
-        total += tm * tn;
-    }
-    b.tile_start[b.count] = total;
+    auto enumerate = [&](int tm_, int tn_) {
+        int total = 0;
+        for (int i = 0; i < b.count; ++i) {
+            const GemmProb& p = b.p[i];
+            const int tm = (p.M + tm_ - 1) / tm_;
+            const int tn = (p.N + tn_ - 1) / tn_;
+            b.tiles_n[i] = tn;
+            b.tile_start[i] = total;
+            total += tm * tn;
+        }
+        b.tile_start[b.count] = total;
+        return total;
+    };
+    int total = enumerate(TM, TN);
     if (total == 0) return cudaSuccess;
-    k_gemm<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI><<<total, 256, 0, s>>>(b);
     ++*launches;
-    return cudaGetLastError();
+    if (total >= kWideTiles) {
+        // enough 128 x 128 tiles for every SM: half the shared-memory reads
+        // per FMA of the small kernel
+        k_gemm<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI><<<total, 256, 0, s>>>(b);
+        return cudaGetLastError();
+    }
+    total = enumerate(SM_T, SM_T);
+    int kmax = 0;
+    for (int i = 0; i < b.count; ++i) kmax = b.p[i].K > kmax ? b.p[i].K : kmax;
+    int split = 1;
+    while (split < 8 && 2 * split * total <= kSmallCtas && kmax >= 2 * split * SM_K) split *= 2;
+    if (b.count <= kFewGroup)
+        return launch_small<kFewGroup, ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(b, total, split, s);
+    return launch_small<kMaxGroup, ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(b, total, split, s);
 }
 
 // Dispatch over the operand/epilogue combinations the library uses.
