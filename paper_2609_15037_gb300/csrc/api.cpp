@@ -307,7 +307,7 @@ struct RefreshRunner {
     }
 
     // Lower Cholesky factor of Cg (+ shift on the diagonal) in place and the
-    // inverse of its diagonal superblocks (512 columns) in Linv.
+    // inverse of its diagonal superblocks (2304 columns) in Linv.
     void cholesky(const std::vector<int>& rows, float shift_rel) {
         moara::CholBatch b{};
         b.count = static_cast<int>(it.size());
@@ -368,7 +368,7 @@ struct RefreshRunner {
     }
 
     // Linv <- Cg^-1 from the inverse of the superblocks, level by level (block
-    // size sz = 512, 1024, ...) with two grouped products per level:
+    // size sz = 2304, 4608, ...) with two grouped products per level:
     //   T = L[D, A] Linv[A, A];  Linv[D, A] = -Linv[D, D] T.
     void tri_inverse() {
         int lmax = 0;

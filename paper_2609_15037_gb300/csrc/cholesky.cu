@@ -3,7 +3,8 @@
 // group, one launch per 64 columns.
 //
 // Launch `step` = s (s = -1 .. nb - 1, nb = ceil(l / 64)) holds, for each
-// module, tiles of 64 x 64 that depend on earlier launches only:
+// module, tiles (64 x 64; bulk and ibulk 128 x 128) that depend on earlier
+// launches only:
 //
 //   crit    L[d, s], then the factor of the diagonal block d = s + 1 and its
 //           inverse: the chain that the next launch waits for
@@ -15,9 +16,9 @@
 //   ibulk   U[t, c] -= L[t, s-1] Linv[s-1, c], t > s (U grows in Linv's place)
 //   zero    the rest of Linv's row block s
 //
-// islab and ibulk stay within superblocks of kTriSuper blocks (512 columns);
-// the larger levels of the inverse are products of their own.  All sums are
-// fp32 FMAs.
+// islab and ibulk stay within superblocks of kTriSuper blocks (2304 columns,
+// the whole of every sketch up to r = 2272); the levels of the inverse past
+// that are products of their own.  All sums are fp32 FMAs.
 //
 // What bounds it is the chain, one CTA per module and step: two 64-deep
 // products, then 64 pivots one after the other.  With a factor kernel that
@@ -39,7 +40,9 @@ namespace {
 
 constexpr int NB = kTriBase;          // 64
 constexpr int LD = NB + 4;            // pitch of a k-major operand tile (16-byte rows, 2-way conflicts on the fill)
+constexpr int LDW = 2 * NB + 4;       // pitch of a 128-wide one
 constexpr int NT = 256;
+constexpr int CHOL_SMEM = 2 * NB * LDW * sizeof(float);
 constexpr int SP = 8;                 // pivots per sub-panel of the diagonal block
 
 // Tile counts of one module at step s; the same on the host and the device.
@@ -61,10 +64,10 @@ __host__ __device__ inline CholTiles chol_tiles(int l, int s) {
     t.islab = s - s / kTriSuper * kTriSuper;
     t.zero = (l + ZCOLS - 1) / ZCOLS;
     if (s >= 1) {
-        const int q = nb - (s + 1);
-        t.bulk = q > 0 ? q * (q + 1) / 2 - 1 : 0;      // all but the block the chain takes
+        const int q = (nb - (s + 1) + 1) / 2;          // pairs of blocks from s + 1 on
+        t.bulk = q > 0 ? q * (q + 1) / 2 : 0;
         const int b1 = (s - 1) / kTriSuper * kTriSuper;
-        t.ibulk = imax(0, imin(b1 + kTriSuper, nb) - (s + 1)) * (s - b1);
+        t.ibulk = (imax(0, imin(b1 + kTriSuper, nb) - (s + 1)) + 1) / 2 * ((s - b1 + 1) / 2);
     }
     return t;
 }
@@ -100,6 +103,23 @@ struct Block {
             dst[k + 2][i] = v[kk].z;
             dst[k + 3][i] = v[kk].w;
         }
+    }
+    // the same into a tile of 128 columns, from column off on
+    __device__ __forceinline__ void store_t(float (*dst)[LDW], int off) const {
+        const int i = (threadIdx.x >> 2) + off, k0 = (threadIdx.x & 3) * 4;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            const int k = kk * 16 + k0;
+            dst[k][i] = v[kk].x;
+            dst[k + 1][i] = v[kk].y;
+            dst[k + 2][i] = v[kk].z;
+            dst[k + 3][i] = v[kk].w;
+        }
+    }
+    __device__ __forceinline__ void store_n(float (*dst)[LDW], int off) const {
+        const int i = threadIdx.x >> 2, k0 = (threadIdx.x & 3) * 4 + off;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) *reinterpret_cast<float4*>(&dst[i][kk * 16 + k0]) = v[kk];
     }
     // as stored: dst[i][k]
     __device__ __forceinline__ void store_n(float (*dst)[LD]) const {
@@ -335,9 +355,60 @@ __device__ __forceinline__ void tri_index(int e, int& i, int& j) {
     j = e - i * (i + 1) / 2;
 }
 
+// C (128 x 128 at row i0, column j0 of C, of which nr x nc exist) -= A B from
+// k-major tiles, in four 64 x 64 quadrants: thread (ty, tx) holds rows
+// 4 ty .. + 3 and columns 4 tx .. + 3 of each.  zero[h]: column half h starts
+// from zero instead of C; quadrant (0, 0) is left alone when skip.
+__device__ __forceinline__ void wide_update(const float (*As)[LDW], const float (*Bs)[LDW], float* C, long long l,
+                                            int nr, int nc, bool vec, bool zero0, bool zero1, bool skip) {
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    float acc[8][8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[p][q] = 0.0f;
+#pragma unroll 4
+    for (int k = 0; k < NB; ++k) {
+        const float4 a0 = *reinterpret_cast<const float4*>(&As[k][4 * ty]);
+        const float4 a1 = *reinterpret_cast<const float4*>(&As[k][NB + 4 * ty]);
+        const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][4 * tx]);
+        const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][NB + 4 * tx]);
+        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc[p][q] = fmaf(av[p], bv[q], acc[p][q]);
+    }
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        const int i = (p >> 2) * NB + 4 * ty + (p & 3);
+        if (i >= nr) continue;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = h * NB + 4 * tx;
+            if (j >= nc || (skip && h == 0 && p < 4)) continue;
+            const bool z = h == 0 ? zero0 : zero1;
+            float* c = C + i * l + j;
+            const float* x = &acc[p][4 * h];
+            if (vec && j + 3 < nc) {
+                const float4 o = z ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : *reinterpret_cast<const float4*>(c);
+                *reinterpret_cast<float4*>(c) = make_float4(o.x - x[0], o.y - x[1], o.z - x[2], o.w - x[3]);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (j + q < nc) c[q] = (z ? 0.0f : c[q]) - x[q];
+            }
+        }
+    }
+}
+
 __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ CholBatch b) {
-    __shared__ __align__(16) float buf0[NB][LD];
-    __shared__ __align__(16) float buf1[NB][LD];
+    extern __shared__ __align__(16) float smem[];
+    float (*const buf0)[LD] = reinterpret_cast<float (*)[LD]>(smem);
+    float (*const buf1)[LD] = reinterpret_cast<float (*)[LD]>(smem + NB * LD);
+    float (*const wide0)[LDW] = reinterpret_cast<float (*)[LDW]>(smem);
+    float (*const wide1)[LDW] = reinterpret_cast<float (*)[LDW]>(smem + NB * LDW);
     __shared__ float red[NT / 32];
     const int s = b.step;
     if (static_cast<int>(blockIdx.x) < b.count) {
@@ -410,7 +481,7 @@ __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ Cho
         if (b.tile_start[mid] <= tile) lo = mid; else hi = mid - 1;
     }
     const CholItem& p = b.p[lo];
-    const int l = p.l;
+    const int l = p.l, nb = (l + NB - 1) / NB;
     const CholTiles n = chol_tiles(l, s);
     int e = tile - b.tile_start[lo];
     const bool vec = (l & 3) == 0;
@@ -467,36 +538,44 @@ __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ Cho
     }
     e -= n.islab;
     if (e < n.bulk) {
-        // entry 0 of the triangle is the chain's block
+        // pairs of row blocks and of column blocks from s + 1 on; of the first
+        // the chain has block (s + 1, s + 1)
         int i, t;
-        tri_index(e + 1, i, t);
-        i += s + 1;
-        t += s + 1;
-        r0.load(at(A, i, s - 1), l, rows(i), NB, vec);
-        r1.load(at(A, t, s - 1), l, rows(t), NB, vec);
-        c.load(at(A, i, t), l, rows(i), rows(t), vec);
-        r0.store_t(buf0);
-        r1.store_t(buf1);
+        tri_index(e, i, t);
+        i = s + 1 + 2 * i;
+        t = s + 1 + 2 * t;
+        const int nr = min(2 * NB, l - i * NB), nc = min(2 * NB, l - t * NB);
+        Block q0, q1;
+        r0.load(at(A, i, s - 1), l, nr, NB, vec);
+        r1.load(at(A, i + 1, s - 1), l, nr - NB, NB, vec);
+        q0.load(at(A, t, s - 1), l, nc, NB, vec);
+        q1.load(at(A, t + 1, s - 1), l, nc - NB, NB, vec);
+        r0.store_t(wide0, 0);
+        r1.store_t(wide0, NB);
+        q0.store_t(wide1, 0);
+        q1.store_t(wide1, NB);
         __syncthreads();
-        acc.mac(buf0, buf1);
-        acc.sub_from(c);
-        acc.store(at(A, i, t), l, rows(i), rows(t), vec);
+        wide_update(wide0, wide1, at(A, i, t), l, nr, nc, vec, false, false, e == 0);
         return;
     }
     e -= n.bulk;
     if (e < n.ibulk) {
-        const int b1 = (s - 1) / kTriSuper * kTriSuper, w = s - b1;
-        const int t = s + 1 + e / w, cb = b1 + e % w;
-        r0.load(at(A, t, s - 1), l, rows(t), NB, vec);
-        r1.load(at(X, s - 1, cb), l, NB, NB, vec);
-        if (cb < s - 1) c.load(at(X, t, cb), l, rows(t), NB, vec);
-        else c.zero();
-        r0.store_t(buf0);
-        r1.store_n(buf1);
+        const int b1 = (s - 1) / kTriSuper * kTriSuper, w = (s - b1 + 1) / 2;
+        const int t = s + 1 + e / w * 2, cb = b1 + e % w * 2;
+        const int tend = min(b1 + kTriSuper, nb);
+        const int nr = min(min(2, tend - t) * NB, l - t * NB), nc = min(2, s - cb) * NB;
+        Block q0, q1;
+        r0.load(at(A, t, s - 1), l, nr, NB, vec);
+        r1.load(at(A, t + 1, s - 1), l, nr - NB, NB, vec);
+        q0.load(at(X, s - 1, cb), l, NB, NB, vec);
+        q1.load(at(X, s - 1, cb + 1), l, nc > NB ? NB : 0, NB, vec);
+        r0.store_t(wide0, 0);
+        r1.store_t(wide0, NB);
+        q0.store_n(wide1, 0);
+        q1.store_n(wide1, NB);
         __syncthreads();
-        acc.mac(buf0, buf1);
-        acc.sub_from(c);
-        acc.store(at(X, t, cb), l, rows(t), NB, vec);
+        // column block s - 1 is touched for the first time
+        wide_update(wide0, wide1, at(X, t, cb), l, nr, nc, vec, cb == s - 1, cb + 1 == s - 1, false);
         return;
     }
     e -= n.ibulk;
@@ -513,6 +592,8 @@ __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ Cho
 
 cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
+    const cudaError_t ea = cudaFuncSetAttribute(k_chol_step, cudaFuncAttributeMaxDynamicSharedMemorySize, CHOL_SMEM);
+    if (ea != cudaSuccess) return ea;
     int nbmax = 0;
     for (int i = 0; i < b.count; ++i) nbmax = std::max(nbmax, (b.p[i].l + NB - 1) / NB);
     for (int step = -1; step < nbmax; ++step) {
@@ -523,7 +604,7 @@ cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches) {
         }
         b.tile_start[b.count] = total;
         b.step = step;
-        k_chol_step<<<b.count + total, NT, 0, s>>>(b);
+        k_chol_step<<<b.count + total, NT, CHOL_SMEM, s>>>(b);
         ++*launches;
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -204,7 +204,7 @@ cudaError_t launch_philox_gaussian(const SmallBatch& b, cudaStream_t s, int64_t*
 // (zero elsewhere).  A pivot that is not positive and finite counts as 1 and
 // sets *fail.  launch_cholesky fills step and tile_start.
 constexpr int kTriBase = 64;
-constexpr int kTriSuper = 8;
+constexpr int kTriSuper = 36;
 struct CholItem {
     float* A;
     float* X;

@@ -1,6 +1,6 @@
 """The refresh's blocked Cholesky and superblock inverse at sketch widths l
 around its tiles: below, at and past one 64-column block, several blocks, the
-512-column superblock and the levels of the inverse past it.  The projector's
+2304-column superblock and the levels of the inverse past it.  The projector's
 columns come through up to sixteen such factorisations, so orthonormality to
 1e-5 and the leading singular vectors of a spectrum with clear gaps pin them.
 The noise floor (per-direction, of the largest singular value) is that of the
@@ -12,6 +12,8 @@ import pytest
 
 import synth
 
+from gpu_helpers import top_subspace
+
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
@@ -19,13 +21,13 @@ torch = pytest.importorskip("torch")
 
 @pytest.mark.parametrize("bf16,l", [(False, 1), (False, 2), (False, 63), (False, 64), (False, 65), (False, 130),
                                     (False, 511), (False, 512), (False, 513), (False, 579), (False, 640),
-                                    (True, 72), (True, 512), (True, 520), (True, 1032)])
+                                    (True, 72), (True, 512), (True, 520), (True, 1032),
+                                    (False, 2318), (True, 2320)])
 def test_refresh_sketch_widths(bf16, l):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import paper_2609_15037_gb300 as M
-    m, n = (1152, 1100) if l > 640 else (704, 656)
-    n = n // 8 * 8
+    m, n = (2400, 4800) if l > 1096 else (1152, 1096) if l > 640 else (704, 656)
     r = 1 if l < 8 else 8
     u, v = synth.lowrank_factors(m, n, 8, seed=l)
     G = (u * (10.0 * 0.8 ** np.arange(8))) @ v.T
@@ -40,6 +42,6 @@ def test_refresh_sketch_widths(bf16, l):
     P = g.modules[0].P.double().cpu().numpy()
     g.close()
     assert np.abs(P.T @ P - np.eye(r)).max() <= 1e-5
-    U = np.linalg.svd(G, full_matrices=False)[0][:, :r]
+    U = top_subspace(G, r)[0]
     if l >= 8:      # a one- or two-column sketch holds a mixture of close directions
         assert np.min(np.abs(np.sum(P * U, axis=0))) >= 0.9999
