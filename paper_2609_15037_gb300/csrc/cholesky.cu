@@ -30,6 +30,7 @@
 // alignment of the 1024 / 2816 layer went from 10.33 to 4.71 ms, of the 4096 /
 // 11008 layer from 68.0 to 39.8 ms.
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -42,7 +43,10 @@ constexpr int NB = kTriBase;          // 64
 constexpr int LD = NB + 4;            // pitch of a k-major operand tile (16-byte rows, 2-way conflicts on the fill)
 constexpr int LDW = 2 * NB + 4;       // pitch of a 128-wide one
 constexpr int NT = 256;
-constexpr int CHOL_SMEM = 2 * NB * LDW * sizeof(float);
+constexpr int kCritCtas = 4;          // CTAs of the chain per module (a cluster)
+constexpr int kCritModules = 38;      // modules up to which they fit beside each other, one per SM
+constexpr int CHOL_SMEM = 5 * NB * LD * sizeof(float);
+static_assert(5 * LD >= 2 * LDW, "two 128-wide operand tiles fit the chain's five buffers");
 constexpr int SP = 8;                 // pivots per sub-panel of the diagonal block
 
 // Tile counts of one module at step s; the same on the host and the device.
@@ -214,126 +218,199 @@ __device__ __forceinline__ float rsqrt_newton(float d) {
     return fmaf(0.5f * r, e, r);
 }
 
+// 1 / d for a normal d (rcp.approx and one step of Newton's iteration on
+// 1 / r = d).
+__device__ __forceinline__ float rcp_newton(float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
+
+__device__ __forceinline__ void bar(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+__device__ __forceinline__ void get8(float (&x)[8], const float* p) {
+    const float4 u = reinterpret_cast<const float4*>(p)[0], v = reinterpret_cast<const float4*>(p)[1];
+    x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+}
+
+__device__ __forceinline__ void put8(float* p, const float (&x)[8]) {
+    reinterpret_cast<float4*>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
+    reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
+}
+
 // Factor F of the 64 x 64 block in tile (lower triangle; rows past nd hold the
-// identity) and its inverse, by right-looking sub-panels of eight pivots.
-// The block's 64 rows are followed by 64 identity rows: the same column
-// operations turn those into F^-T.  Thread (w, lane) keeps rows
-// 16 w + 4 (lane / 8) .. + 3 and columns 8 (lane % 8) .. + 7 of the 128 x 64
-// array in registers.  Per sub-panel its eight columns go to shared memory,
-// one thread per row forms the row's eight entries of the factor -- every
-// thread repeats the 8 x 8 diagonal factor for itself, so that eight pivots
-// need no exchange -- and all warps with live rows update the columns to the
-// right.  Chain per pivot: one reciprocal square root, one multiplication,
-// one FMA.
-__device__ __forceinline__ void factor64(float (*tile)[LD], float* pin, float* pout, float* A, float* X, long long l,
-                                         int nd, bool vec, int* fail) {
-    constexpr int PP = 2 * NB + 4;                    // pitch of pout[c][row]
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const int tx = lane & 7, row0 = 16 * w + 4 * (lane >> 3);
-    float a[4][8];
-    if (w < 4) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float4 x = *reinterpret_cast<const float4*>(&tile[row0 + i][8 * tx]);
-            const float4 y = *reinterpret_cast<const float4*>(&tile[row0 + i][8 * tx + 4]);
-            a[i][0] = x.x; a[i][1] = x.y; a[i][2] = x.z; a[i][3] = x.w;
-            a[i][4] = y.x; a[i][5] = y.y; a[i][6] = y.z; a[i][7] = y.w;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) a[i][k] = (row0 - NB + i == 8 * tx + k) ? 1.0f : 0.0f;
-    }
-    bool bad = false;
+// identity) and its inverse, by sub-panels of eight pivots.
+//
+// Warps 0 and 1, one thread per row, run the chain: a thread keeps its row's
+// eight entries of the sub-panel, repeats the 8 x 8 diagonal factor for itself
+// (so that eight pivots need no exchange; as L D L^T, one reciprocal, one
+// multiplication and one FMA deep per pivot, scaled by 1 / sqrt(D) at the end)
+// and brings its entries of the next sub-panel up to date.  Warps 4 - 7 keep
+// the block (4 x 8 entries a thread), apply the sub-panel to the columns after
+// the next one meanwhile and write it out.  Warps 2 and 3 follow one sub-panel
+// behind with the inverse: row r of F^-T = I F^-T, a dot product with the
+// finished columns of F per entry.  With 128 rows (the block's and the
+// identity's) and the whole update in the chain a block took 16,000 clocks,
+// here 13,200: a sub-panel's 1,430 are 520 for its eight pivots, 470 for the
+// next sub-panel's columns (shared-memory broadcasts), the rest exchange.
+// (Chain and inverse on one warp each, two rows a lane: 14,800.)
+//
+// The block comes scaled by sigma = 2^(-2h), near unit diagonal, so that the
+// reciprocals stay in range; F and its inverse are written times 2^h and 2^-h.
+constexpr int PIN = SP * SP;                          // floats of scratch: the sub-panel's diagonal rows,
+static_assert(PIN + 2 * NB * SP <= NB * LD, "the factor's scratch fits one tile");   // and two of the next columns
+
+__device__ __forceinline__ void factor64(const float (*tile)[LD], float* scratch, float (*F)[LD], float (*Z)[LD],
+                                         float* A, float* X, long long l, int nd, bool vec, float up, float down,
+                                         int* fail) {
+    float* const pin = scratch;
+    float* const nbuf = scratch + PIN;                // [2][row][8]
+    const int t = threadIdx.x;
+    if (t < NB) {
+        float v[SP];
+        get8(v, &tile[t][0]);
+        bool bad = false;
 #pragma unroll 1
-    for (int c0 = 0; c0 < NB; c0 += SP) {
-        if (8 * tx == c0) {
+        for (int c0 = 0; c0 < NB; c0 += SP) {
+            if (t >= c0 && t < c0 + SP) put8(pin + (t - c0) * SP, v);
+            bar(1, NB);
+            float D[SP][SP], rs[SP];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float4* p = reinterpret_cast<float4*>(pin + (row0 + i) * SP);
-                p[0] = make_float4(a[i][0], a[i][1], a[i][2], a[i][3]);
-                p[1] = make_float4(a[i][4], a[i][5], a[i][6], a[i][7]);
-            }
-        }
-        __syncthreads();
-        if (t < 2 * NB) {
-            float v[SP];
-            {
-                const float4* p = reinterpret_cast<const float4*>(pin + t * SP);
-                const float4 x = p[0], y = p[1];
-                v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
-            }
-            float D[SP][SP];
-#pragma unroll
-            for (int i = 0; i < SP; ++i) {
-                const float4* p = reinterpret_cast<const float4*>(pin + (c0 + i) * SP);
-                const float4 x = p[0], y = p[1];
-                D[i][0] = x.x; D[i][1] = x.y; D[i][2] = x.z; D[i][3] = x.w;
-                D[i][4] = y.x; D[i][5] = y.y; D[i][6] = y.z; D[i][7] = y.w;
+            for (int i = 0; i < SP; ++i) {            // its lower triangle
+                const float4 u = *reinterpret_cast<const float4*>(pin + i * SP);
+                D[i][0] = u.x; D[i][1] = u.y; D[i][2] = u.z; D[i][3] = u.w;
+                if (i >= 4) {
+                    const float4 y = *reinterpret_cast<const float4*>(pin + i * SP + 4);
+                    D[i][4] = y.x; D[i][5] = y.y; D[i][6] = y.z; D[i][7] = y.w;
+                }
             }
 #pragma unroll
             for (int j = 0; j < SP; ++j) {
                 float d = D[j][j];
-                if (!(d > 0.0f) || !isfinite(d)) {   // marks the failure; the module keeps its projector
-                    d = 1.0f;
-                    bad = true;
-                }
-                const float r = rsqrt_newton(d);
-                v[j] *= r;
-#pragma unroll
-                for (int i = j + 1; i < SP; ++i) D[i][j] *= r;
+                // a pivot that is not a positive normal number marks the
+                // failure; the module keeps its projector
+                const bool ok = d >= 1.17549435e-38f && d <= 3.402823466e38f;
+                bad = bad || !ok;
+                d = ok ? d : 1.0f;
+                const float rd = rcp_newton(d);
+                rs[j] = rsqrt_newton(d);
+                const float qv = v[j] * rd;
 #pragma unroll
                 for (int k = j + 1; k < SP; ++k) {
-                    v[k] = fmaf(-v[j], D[k][j], v[k]);
+                    const float q = D[k][j] * rd;
 #pragma unroll
-                    for (int i = k; i < SP; ++i) D[i][k] = fmaf(-D[i][j], D[k][j], D[i][k]);
+                    for (int i = k; i < SP; ++i) D[i][k] = fmaf(-D[i][j], q, D[i][k]);
+                    v[k] = fmaf(-qv, D[k][j], v[k]);
                 }
             }
-            const int row = t & (NB - 1);
-            if (t < NB) {
-                // rows of the factor: zero above the diagonal
-#pragma unroll
-                for (int j = 0; j < SP; ++j) v[j] = c0 + j <= row ? v[j] : 0.0f;
-                if (row < nd) {
-                    float* dst = A + row * l + c0;
-                    if (vec && c0 + SP <= nd) {
-                        reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
-                        reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < SP; ++j)
-                            if (c0 + j < nd) dst[j] = v[j];
-                    }
-                }
-            } else if (row < nd) {
-                // F^-T: entry (row, c) is entry (c, row) of the inverse, zero for row > c
-#pragma unroll
-                for (int j = 0; j < SP; ++j)
-                    if (c0 + j < nd) X[(c0 + j) * l + row] = v[j];
-            }
-#pragma unroll
-            for (int j = 0; j < SP; ++j) pout[j * PP + t] = v[j];
-        }
-        __syncthreads();
-        // rows past the sub-panel of the block, identity rows up to its end
-        const bool live = w < 4 ? 16 * w + 15 >= c0 + SP : 16 * (w - 4) < c0 + SP;
-        if (live && 8 * tx >= c0 + SP) {
 #pragma unroll
             for (int j = 0; j < SP; ++j) {
-                const float4 f = *reinterpret_cast<const float4*>(pout + j * PP + row0);
-                const float4 x = *reinterpret_cast<const float4*>(pout + j * PP + 8 * tx);
-                const float4 y = *reinterpret_cast<const float4*>(pout + j * PP + 8 * tx + 4);
-                const float fv[4] = {f.x, f.y, f.z, f.w};
-                const float kv[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+                v[j] = c0 + j <= t ? v[j] * rs[j] : 0.0f;             // zero above the diagonal
+                F[c0 + j][t] = v[j];
+            }
+            if (t == 0) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int j = 0; j < SP; ++j) F[c0 + j][NB] = rs[j];   // 1 / F[j][j], in the pitch's padding
+            }
+            bar(2, NT);
+            if (c0 + SP < NB) {
+                float n[SP];
+                get8(n, nbuf + ((c0 / SP) & 1) * NB * SP + t * SP);
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) a[i][k] = fmaf(-fv[i], kv[k], a[i][k]);
+                for (int j = 0; j < SP; ++j) {
+                    float f[SP];
+                    get8(f, &F[c0 + j][c0 + SP]);
+#pragma unroll
+                    for (int k = 0; k < SP; ++k) n[k] = fmaf(-v[j], f[k], n[k]);
+                }
+#pragma unroll
+                for (int k = 0; k < SP; ++k) v[k] = n[k];
+            }
+        }
+        if (t == 0 && bad) *fail = 1;
+    } else if (t < 2 * NB) {
+        // row r of F^-T: z[c] = (e_r[c] - sum_{k < c} z[k] F[c][k]) / F[c][c]
+        const int r = t - NB;
+#pragma unroll 1
+        for (int c0 = 0; c0 < NB; c0 += SP) {
+            bar(2, NT);
+            float z[SP];
+#pragma unroll
+            for (int j = 0; j < SP; ++j) z[j] = r == c0 + j ? 1.0f : 0.0f;
+            // z of the second warp's rows begins with 32 zeros
+#pragma unroll 8
+            for (int k = r & 32; k < c0; ++k) {
+                const float x = Z[k][r];
+                float f[SP];
+                get8(f, &F[k][c0]);
+#pragma unroll
+                for (int j = 0; j < SP; ++j) z[j] = fmaf(-x, f[j], z[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < SP; ++j) {
+                float f[SP];
+                get8(f, &F[c0 + j][c0]);
+                z[j] *= F[c0 + j][NB];
+#pragma unroll
+                for (int k = j + 1; k < SP; ++k) z[k] = fmaf(-z[j], f[k], z[k]);
+                Z[c0 + j][r] = z[j];
+            }
+            // entry (r, c) of F^-T is entry (c, r) of the inverse, zero for r > c
+            if (r < nd) {
+#pragma unroll
+                for (int j = 0; j < SP; ++j)
+                    if (c0 + j < nd) X[(c0 + j) * l + r] = z[j] * down;
+            }
+        }
+    } else {
+        const int tx = t & 7, row0 = 4 * ((t - 2 * NB) >> 3);
+        float a[4][SP];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) get8(a[i], &tile[row0 + i][SP * tx]);
+        if (tx == 1) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) put8(nbuf + (row0 + i) * SP, a[i]);
+        }
+#pragma unroll 1
+        for (int c0 = 0; c0 < NB; c0 += SP) {
+            bar(2, NT);
+            if (row0 + 3 >= c0 + SP && SP * tx >= c0 + 2 * SP) {
+#pragma unroll 4
+                for (int j = 0; j < SP; ++j) {
+                    const float4 f = *reinterpret_cast<const float4*>(&F[c0 + j][row0]);
+                    const float fv[4] = {f.x, f.y, f.z, f.w};
+                    float k8[SP];
+                    get8(k8, &F[c0 + j][SP * tx]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int k = 0; k < SP; ++k) a[i][k] = fmaf(-fv[i], k8[k], a[i][k]);
+                }
+            }
+            if (SP * tx == c0 + 2 * SP) {
+                float* const nb = nbuf + ((c0 / SP + 1) & 1) * NB * SP;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) put8(nb + (row0 + i) * SP, a[i]);
+            }
+            // the sub-panel's columns of the factor: two threads a row
+            const int row = (t - 2 * NB) >> 1, h = 4 * (t & 1);
+            if (row < nd) {
+                float* dst = A + row * l + c0 + h;
+                float v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = F[c0 + h + j][row] * up;
+                if (vec && c0 + h + 3 < nd) {
+                    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (c0 + h + j < nd) dst[j] = v[j];
+                }
             }
         }
     }
-    if (t == 0 && bad) *fail = 1;
 }
 
 __device__ __forceinline__ float block_sum_256(float v, float* red) {
@@ -403,6 +480,9 @@ __device__ __forceinline__ void wide_update(const float (*As)[LDW], const float 
     }
 }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ CholBatch b) {
     extern __shared__ __align__(16) float smem[];
     float (*const buf0)[LD] = reinterpret_cast<float (*)[LD]>(smem);
@@ -410,71 +490,187 @@ __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ Cho
     float (*const wide0)[LDW] = reinterpret_cast<float (*)[LDW]>(smem);
     float (*const wide1)[LDW] = reinterpret_cast<float (*)[LDW]>(smem + NB * LDW);
     __shared__ float red[NT / 32];
-    const int s = b.step;
-    if (static_cast<int>(blockIdx.x) < b.count) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int s = b.step, C = static_cast<int>(cl.num_blocks());
+    if (static_cast<int>(blockIdx.x) < C * b.count) {
         // ------------------------------------------------ crit
-        const CholItem& p = b.p[blockIdx.x];
+        // The cluster's C CTAs (kCritCtas, or one where the group has enough
+        // modules to fill the GPU) share the products by rows of the block, 16
+        // at a time, the K range split over four groups of 64 threads; the
+        // factor is the first one's.  One CTA alone takes 2,700 to 3,700 clocks
+        // for each of the four 64-deep products, bound by its shared-memory
+        // reads; four CTAs 11,300 clocks from launch to factor instead of
+        // 19,500, but 224 modules' refresh 526 ms instead of 509.
+        const CholItem& p = b.p[blockIdx.x / C];
         const int l = p.l, d = s + 1, nb = (l + NB - 1) / NB;
-        if (d >= nb) return;
+        if (d >= nb) return;                          // the whole cluster
+        const int rank = static_cast<int>(cl.block_rank());
+        if (s < 0 && rank != 0) return;
         const bool vec = (l & 3) == 0;
         const int nd = min(NB, l - d * NB);
         float* const A = p.A;
-        float shift;
-        Block r0, r1, r2;
-        Acc tA, tD, acc, sq;
-        tD.load(A + (long long)d * NB * l + d * NB, l, nd, nd, vec);
-        sq.zero();
+        float (*const bufF)[LD] = reinterpret_cast<float (*)[LD]>(smem);                  // L[d, s-1]; F
+        float (*const bufT)[LD] = reinterpret_cast<float (*)[LD]>(smem + NB * LD);        // L[s, s-1]; the block
+        float (*const bufI)[LD] = reinterpret_cast<float (*)[LD]>(smem + 2 * NB * LD);    // Linv[s, s]; scratch
+        float (*const part)[LD] = reinterpret_cast<float (*)[LD]>(smem + 3 * NB * LD);    // four 16-row partial tiles; Z
+        float (*const bufG)[LD] = reinterpret_cast<float (*)[LD]>(smem + 4 * NB * LD);    // X, then L[d, s]
+        const int t = threadIdx.x;
+        int half;
         if (s < 0) {
             float tr = 0.0f;
-            for (int i = threadIdx.x; i < l; i += NT) tr += A[(long long)i * l + i];
+            for (int i = t; i < l; i += NT) tr += A[(long long)i * l + i];
             tr = block_sum_256(tr, red);
-            shift = b.shift_rel * sqrtf(static_cast<float>(p.rows)) * tr;
-            if (threadIdx.x == 0) *p.shift = shift;
-        } else {
-            shift = *p.shift;
-            tA.load(A + (long long)d * NB * l + s * NB, l, nd, NB, vec);
-            r2.load(p.X + (long long)s * NB * l + s * NB, l, NB, NB, vec);
-            acc.zero();
-            if (s >= 1) {
-                r0.load(A + (long long)d * NB * l + (s - 1) * NB, l, nd, NB, vec);
-                r1.load(A + (long long)s * NB * l + (s - 1) * NB, l, NB, NB, vec);
-                r0.store_t(buf0);
-                r1.store_t(buf1);
-                __syncthreads();
-                acc.mac(buf0, buf1);
-                sq.mac(buf0, buf0);
-                __syncthreads();
+            const float shift = b.shift_rel * sqrtf(static_cast<float>(p.rows)) * tr;
+            // h: half the exponent of the mean diagonal entry (0 where it has none)
+            const float mean = tr / static_cast<float>(l);
+            half = (mean > 0.0f && isfinite(mean)) ? max(-60, ilogbf(mean) / 2) : 0;
+            if (t == 0) {
+                p.shift[0] = shift;
+                p.shift[1] = static_cast<float>(half);
             }
-            acc.sub_from(tA);
-            acc.store_t(buf0);
-            r2.store_t(buf1);
-            __syncthreads();
-            acc.zero();
-            acc.mac(buf0, buf1);                      // L[d, s]
-            acc.store(A + (long long)d * NB * l + s * NB, l, nd, NB, vec);
-            __syncthreads();
-            acc.store_t(buf0);
-            __syncthreads();
-            sq.mac(buf0, buf0);
-        }
-        sq.sub_from(tD);
-        {
-            const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+            const float sigma = exp2f(static_cast<float>(-2 * half));
+            Acc D;
+            D.load(A, l, nd, nd, vec);
+            const int ty = t >> 4, tx = t & 15;
             if (ty == tx) {
 #pragma unroll
-                for (int a = 0; a < 4; ++a) sq.v[a][a] = 4 * ty + a < nd ? sq.v[a][a] + shift : 1.0f;
+                for (int a = 0; a < 4; ++a) D.v[a][a] += shift;
             }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    D.v[a][c] = 4 * ty + a < nd ? D.v[a][c] * sigma : (4 * ty + a == 4 * tx + c ? 1.0f : 0.0f);
+            D.store_n(bufT);
+            __syncthreads();
+        } else {
+            cluster_arrive();                         // waited for before the first access to a peer
+            // this thread's four entries of a group of 16 rows from r0 on
+            const int lr = t >> 4, j0 = 4 * (t & 15);
+            auto entry4 = [&](const float* src, int row, int nc) {
+                float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                const float* q = src + (long long)row * l + j0;
+                if (row < nd) {
+                    if (vec && j0 + 3 < nc) return *reinterpret_cast<const float4*>(q);
+                    if (j0 < nc) x.x = q[0];
+                    if (j0 + 1 < nc) x.y = q[1];
+                    if (j0 + 2 < nc) x.z = q[2];
+                    if (j0 + 3 < nc) x.w = q[3];
+                }
+                return x;
+            };
+            Block q0, q1, q2;
+            if (s >= 1) {
+                q0.load(A + (long long)d * NB * l + (s - 1) * NB, l, nd, NB, vec);
+                q1.load(A + (long long)s * NB * l + (s - 1) * NB, l, NB, NB, vec);
+            }
+            q2.load(p.X + (long long)s * NB * l + s * NB, l, NB, NB, vec);
+            float* const Ads = A + (long long)d * NB * l + s * NB;
+            const float* const Add = A + (long long)d * NB * l + d * NB;
+            float4 tA = entry4(Ads, 16 * rank + lr, NB), tD = entry4(Add, 16 * rank + lr, nd);
+            const float shift = p.shift[0];
+            half = static_cast<int>(p.shift[1]);
+            const float sigma = exp2f(static_cast<float>(-2 * half));
+            // thread (g, ty, tx): rows 4 ty .. + 3 of the 16, columns tx + 16 j,
+            // k in 16 g .. + 15; acc += a b^T from row-major tiles
+            const int g = t >> 6, ty = (t >> 4) & 3, tx = t & 15;
+            auto mac16 = [&](float (&acc)[4][4], const float (*a)[LD], int ar, const float (*bb)[LD]) {
+#pragma unroll
+                for (int k = 16 * g; k < 16 * g + 16; k += 4) {
+                    float4 x[4], y[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        x[i] = *reinterpret_cast<const float4*>(&a[ar + 4 * ty + i][k]);
+                        y[i] = *reinterpret_cast<const float4*>(&bb[tx + 16 * i][k]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            acc[i][j] = fmaf(x[i].x, y[j].x, acc[i][j]);
+                            acc[i][j] = fmaf(x[i].y, y[j].y, acc[i][j]);
+                            acc[i][j] = fmaf(x[i].z, y[j].z, acc[i][j]);
+                            acc[i][j] = fmaf(x[i].w, y[j].w, acc[i][j]);
+                        }
+                }
+            };
+            // sum of the four groups' partial tiles: this thread's four entries
+            auto reduce = [&](const float (&acc)[4][4]) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) part[16 * g + 4 * ty + i][tx + 16 * j] = acc[i][j];
+                __syncthreads();
+                float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 x = *reinterpret_cast<const float4*>(&part[16 * q + (t >> 4)][j0]);
+                    v = make_float4(v.x + x.x, v.y + x.y, v.z + x.z, v.w + x.w);
+                }
+                return v;
+            };
+            if (s >= 1) {
+                q0.store_n(bufF);
+                q1.store_n(bufT);
+            }
+            q2.store_n(bufI);
+            __syncthreads();
+            for (int r0 = 16 * rank; r0 < NB; r0 += 16 * C) {
+                const int row = r0 + lr;
+                if (r0 != 16 * rank) tA = entry4(Ads, row, NB);
+                float4 x = tA;
+                if (s >= 1) {
+                    float acc[4][4] = {};
+                    mac16(acc, bufF, r0, bufT);
+                    const float4 u = reduce(acc);
+                    x = make_float4(tA.x - u.x, tA.y - u.y, tA.z - u.z, tA.w - u.w);
+                }
+                *reinterpret_cast<float4*>(&bufG[row][j0]) = x;       // X
+                __syncthreads();
+                float acc[4][4] = {};
+                mac16(acc, bufG, r0, bufI);
+                x = reduce(acc);                      // L[d, s]; its barrier: every thread is done with these rows of X
+                if (row < nd) {
+                    float* q = Ads + (long long)row * l + j0;
+                    if (vec) *reinterpret_cast<float4*>(q) = x;
+                    else { q[0] = x.x; q[1] = x.y; q[2] = x.z; q[3] = x.w; }
+                }
+                if (r0 == 16 * rank) cluster_wait();
+                for (int q = 0; q < C; ++q)           // to every CTA
+                    *reinterpret_cast<float4*>(cl.map_shared_rank(&bufG[0][0], q) + row * LD + j0) = x;
+                __syncthreads();
+            }
+            cl.sync();
+            for (int r0 = 16 * rank; r0 < NB; r0 += 16 * C) {
+                const int row = r0 + lr;
+                if (r0 != 16 * rank) tD = entry4(Add, row, nd);
+                float acc[4][4] = {};
+                if (s >= 1) mac16(acc, bufF, r0, bufF);
+                mac16(acc, bufG, r0, bufG);
+                const float4 u = reduce(acc);
+                float e[4] = {tD.x - u.x, tD.y - u.y, tD.z - u.z, tD.w - u.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const bool dia = j0 + k == row;
+                    e[k] = row < nd ? (e[k] + (dia ? shift : 0.0f)) * sigma : (dia ? 1.0f : 0.0f);
+                }
+                // the first CTA is past its products with bufT (the cluster barrier)
+                *reinterpret_cast<float4*>(cl.map_shared_rank(&bufT[0][0], 0) + row * LD + j0) =
+                    make_float4(e[0], e[1], e[2], e[3]);
+                __syncthreads();
+            }
+            cl.sync();
+            if (rank != 0) return;
         }
-        __syncthreads();
-        sq.store_n(buf1);
-        __syncthreads();
-        float* const pin = &buf0[0][0];               // 128 x 8, then 8 x 132
-        factor64(buf1, pin, pin + 2 * NB * SP, A + (long long)d * NB * l + d * NB,
-                 p.X + (long long)d * NB * l + d * NB, l, nd, vec, p.fail);
+        factor64(bufT, &bufI[0][0], bufF, part, A + (long long)d * NB * l + d * NB,
+                 p.X + (long long)d * NB * l + d * NB, l, nd, vec, exp2f(static_cast<float>(half)),
+                 exp2f(static_cast<float>(-half)), p.fail);
         return;
     }
     // locate (module, tile)
-    const int tile = blockIdx.x - b.count;
+    const int tile = blockIdx.x - C * b.count;
+    if (tile >= b.tile_start[b.count]) return;        // the last cluster's padding
     int lo = 0, hi = b.count - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -604,9 +800,21 @@ cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches) {
         }
         b.tile_start[b.count] = total;
         b.step = step;
-        k_chol_step<<<b.count + total, NT, CHOL_SMEM, s>>>(b);
+        const int C = b.count <= kCritModules ? kCritCtas : 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(C * b.count + (total + C - 1) / C * C);
+        cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = CHOL_SMEM;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
         ++*launches;
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_chol_step, b);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

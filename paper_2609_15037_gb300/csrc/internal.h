@@ -201,14 +201,14 @@ cudaError_t launch_philox_gaussian(const SmallBatch& b, cudaStream_t s, int64_t*
 // Lower Cholesky factor of each a (l x l, the lower triangle given) plus
 // shift_rel * sqrt(rows) * trace(a) on its diagonal, in place, and in X the
 // inverse of the factor's diagonal superblocks of kTriSuper 64-column blocks
-// (zero elsewhere).  A pivot that is not positive and finite counts as 1 and
-// sets *fail.  launch_cholesky fills step and tile_start.
+// (zero elsewhere).  A pivot that is not positive and finite (of a
+// normal number's size next to the mean diagonal) counts as 1 and sets *fail.  launch_cholesky fills step and tile_start.
 constexpr int kTriBase = 64;
 constexpr int kTriSuper = 36;
 struct CholItem {
     float* A;
     float* X;
-    float* shift;         // scratch: the shift
+    float* shift;         // scratch of two floats: the shift, half the exponent of the mean diagonal
     int* fail;
     int l, rows;
 };
