@@ -26,6 +26,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "tc.h"
@@ -37,7 +38,7 @@ namespace {
 
 constexpr int kTcGroup = 224;                 // modules per launch (G maps in params)
 constexpr long long kWaitLimit = 1LL << 32;   // ~2 s of SM clocks
-constexpr int kMaps = 9;                      // tensor maps per module
+constexpr int kMaps = 10;                     // tensor maps per module
 
 struct TcMod {
     int m, n, r, kb;
@@ -113,7 +114,7 @@ struct K1Params {
     const int* cta_start;              // tiles of CTA c: tiles[cta_start[c] .. cta_start[c+1])
     const TcTile* tiles;
     const TcMod* mods;
-    const CUtensorMap* maps;           // per module: P (K1), P (K2), N, W, V_hi, V_lo, exp_avg, exp_avg_sq
+    const CUtensorMap* maps;           // per module: P (K1), P (K2), N, W, V_hi, V_lo, exp_avg, exp_avg_sq, W (3-D), N_lo
     int* status;
     float beta1, beta2, adam_eps, bc1, bc2;
     float inv_bc1, inv_bc2;            // 1 / bias corrections
@@ -136,11 +137,16 @@ constexpr int K2_STAGE_BYTES = K2_A_BYTES + K2_B_BYTES;
 // not reproduce): a four-chunk ring, TMA in and out, five operand stages.
 constexpr int K2_WCOLS = 32;
 constexpr int K2_WBYTES = K2_BM * K2_WCOLS * 4;         // 16 KB
-template <bool SB> struct K2Cfg {
-    static constexpr int STAGES = SB ? 5 : 6;
-    static constexpr int WBUF = SB ? 4 : 2;
-    static constexpr int BYTES = STAGES * K2_STAGE_BYTES + WBUF * K2_WBYTES;
+// ALIGN (the alignment diagnostic): the product is reduced against G instead of
+// applied; N (a right projector: V Q) comes as two planes, the residual in a
+// third 16 KB slot of each stage.
+template <bool SB, bool ALIGN = false> struct K2Cfg {
+    static constexpr int STAGES = ALIGN ? 4 : SB ? 5 : 6;
+    static constexpr int STAGE_BYTES = K2_STAGE_BYTES + (ALIGN ? K2_B_BYTES : 0);
+    static constexpr int WBUF = ALIGN ? 0 : SB ? 4 : 2;
+    static constexpr int BYTES = STAGES * STAGE_BYTES + WBUF * K2_WBYTES;
 };
+static_assert(K2Cfg<false, true>::BYTES <= K2Cfg<true>::BYTES, "the alignment stages fit K2's shared memory");
 constexpr int K2_WARPS = 12;                            // 0 TMA, 1 MMA, 2 W loader, 3 W storer, 4-11 epilogue
 constexpr int K2_THREADS = K2_WARPS * 32;
 constexpr int K2_SMEM = 1024 + (K2Cfg<true>::BYTES > K2Cfg<false>::BYTES ? K2Cfg<true>::BYTES : K2Cfg<false>::BYTES) +
@@ -154,6 +160,11 @@ struct K2Params {
     int* status;
     float step_scale;                  // lr * alpha
     int decompose;
+};
+
+struct K2AlignParams : K2Params {
+    const uint16_t* G[kTcGroup];       // gradient of each launch slot (m x n)
+    double* acc;                       // three sums per launch slot: <G, a>, <a, a>, <G, G>
 };
 
 struct SmemCtl {
@@ -705,20 +716,28 @@ k1_project(const __grid_constant__ K1Params p) {
 // ===========================================================================
 // K2: back-projection dV = P N and the weight update in the epilogue.
 // ===========================================================================
-template <int BLK, bool SB>
+// ALIGN: S(W, t) of §3.2 instead of the update: each entry of P N (or N Q^T,
+// with N = R in two planes) times its block norm M is dotted with G.  The
+// reduction of a tile runs beside the next tile's MMAs, and a thread reads its
+// row of G 16 entries at a time, the next ones before it needs them.  (As a
+// transposed product with one tile per CTA, whose reduction read G down its
+// columns after the MMAs, two layers' 4096 / 11008 diagnostic took 4.72 ms;
+// now 2.84 ms.)
+template <int BLK, bool SB, bool ALIGN = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(K2_THREADS, 1)
-k2_backproject(const __grid_constant__ K2Params p) {
+k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignParams, K2Params>::type p) {
     constexpr int WC = StateCols<SB>::N;              // W columns per ring chunk
     constexpr int HC = WC / 2;                        // columns per epilogue thread and chunk
     // fp32 W, blocks of >= 32 columns: 64 x 64 update chunks through the 3-D
     // map where the module allows it (TcMod::w3d)
-    constexpr bool W3D = !SB && BLK >= 32 && K2_BN % BLK == 0;
+    constexpr bool W3D = !ALIGN && !SB && BLK >= 32 && K2_BN % BLK == 0;
     static_assert(!SB || BLK >= 32, "bf16 states: a thread's 32 columns lie in one block");
-    constexpr int K2_STAGES = K2Cfg<SB>::STAGES, K2_WBUF = K2Cfg<SB>::WBUF;
+    constexpr int K2_STAGES = K2Cfg<SB, ALIGN>::STAGES, K2_WBUF = ALIGN ? 1 : K2Cfg<SB>::WBUF;
+    constexpr int STAGE_BYTES = K2Cfg<SB, ALIGN>::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    uint8_t* wring = smem + K2_STAGES * K2_STAGE_BYTES;
-    SmemCtl* ctl = reinterpret_cast<SmemCtl*>(wring + K2_WBUF * K2_WBYTES);
+    uint8_t* wring = smem + K2_STAGES * STAGE_BYTES;
+    SmemCtl* ctl = reinterpret_cast<SmemCtl*>(smem + K2Cfg<SB, ALIGN>::BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int crank = static_cast<int>(ptx::cluster_ctarank());   // row tile 2 t0 + crank of each pair tile
     const int cluster = blockIdx.x >> 1;
@@ -767,6 +786,8 @@ k2_backproject(const __grid_constant__ K2Params p) {
                 const TcMod& md = p.mods[tl.mod];
                 const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 1];
                 const CUtensorMap* bmap = &p.maps[tl.mod * kMaps + 2];
+                const CUtensorMap* lmap = &p.maps[tl.mod * kMaps + 9];
+                const bool right = ALIGN && md.right != 0;
                 const int i0 = (2 * tl.t0 + crank) * K2_BM, n0 = tl.t1 * K2_BN;
                 const int nk = (md.r + K2_BK - 1) / K2_BK;
                 for (int kb = 0; kb < nk; ++kb) {
@@ -774,15 +795,18 @@ k2_backproject(const __grid_constant__ K2Params p) {
                                         MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
                     const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
                     const uint32_t fb = ptx::mapa(own, 0);
-                    if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * K2_STAGE_BYTES);
-                    const uint32_t a = ptx::smem_u32(smem + stage * K2_STAGE_BYTES);
+                    if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * STAGE_BYTES);
+                    const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
                     const uint32_t b = a + K2_A_BYTES;
                     ptx::tma_load_2d_pair(a, amap, fb, kb * K2_BK, i0);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int c = 2 * crank + h;
                         ptx::tma_load_2d_pair(b + h * 8192, bmap, fb, n0 + 64 * c, kb * K2_BK);
+                        if (ALIGN && !right)
+                            ptx::tma_load_2d_pair(b + K2_B_BYTES + h * 8192, lmap, fb, n0 + 64 * c, kb * K2_BK);
                     }
+                    if (right) ptx::tma_load_2d_pair(b + K2_B_BYTES, lmap, fb, kb * K2_BK, i0);
                     issued |= 1u << stage;
                     last_par = (last_par & ~(1u << stage)) | (phase << stage);
                     if (++stage == K2_STAGES) { stage = 0; phase ^= 1; }
@@ -807,6 +831,7 @@ k2_backproject(const __grid_constant__ K2Params p) {
                 const TcTile tl = p.tiles[t];
                 const TcMod& md = p.mods[tl.mod];
                 const int nk = (md.r + K2_BK - 1) / K2_BK;
+                const bool right = ALIGN && md.right != 0;
                 if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->acce[buf]), acc_phase ^ 1, abort_flag, p.status,
                                             MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
                 ptx::tc_fence_after();
@@ -815,13 +840,21 @@ k2_backproject(const __grid_constant__ K2Params p) {
                     if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag, p.status,
                                                 MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
                     ptx::tc_fence_after();
-                    const uint32_t a = ptx::smem_u32(smem + stage * K2_STAGE_BYTES);
+                    const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
                     const uint32_t b = a + K2_A_BYTES;
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const uint64_t adesc = ptx::smem_desc_sw128(a + kk * 32, 16, 1024);
                         const uint64_t bdesc = ptx::smem_desc_sw128(b + kk * 2048, 8192, 1024);
                         ptx::mma2_f16(d0, adesc, bdesc, idesc, (kb | kk) != 0);
+                        if constexpr (ALIGN) {   // the residual plane, of N (K-major rows with a right projector)
+                            if (!right)
+                                ptx::mma2_f16(d0, adesc, ptx::smem_desc_sw128(b + K2_B_BYTES + kk * 2048, 8192, 1024),
+                                              idesc, 1);
+                            else
+                                ptx::mma2_f16(d0, ptx::smem_desc_sw128(b + K2_B_BYTES + kk * 32, 16, 1024), bdesc,
+                                              idesc, 1);
+                        }
                     }
                     ptx::mma2_commit_mc(ptx::smem_u32(&ctl->empty[stage]), 0x3);
                     if (++stage == K2_STAGES) { stage = 0; phase ^= 1; }
@@ -836,7 +869,7 @@ k2_backproject(const __grid_constant__ K2Params p) {
     } else if (warp == 2) {
         // ------------------------------------------- W chunk loader (TMA in)
         // (bf16 W only: an fp32 W is updated by reduce-add, never loaded)
-        if (SB && lane == 0) {
+        if (SB && !ALIGN && lane == 0) {
             uint32_t g = 0;
             uint32_t issued = 0, last_par = 0;
             bool ok = true;
@@ -865,7 +898,7 @@ k2_backproject(const __grid_constant__ K2Params p) {
         }
     } else if (warp == 3) {
         // ------------------------------ W chunk storer (TMA store / reduce-add)
-        if (lane == 0) {
+        if (!ALIGN && lane == 0) {
             uint32_t g = 0;
             bool ok = true;
             for (int t = t_begin; t < t_end && ok; ++t) {
@@ -891,6 +924,88 @@ k2_backproject(const __grid_constant__ K2Params p) {
                 }
             }
             ptx::bulk_wait_all();
+        }
+    } else if constexpr (ALIGN) {
+        // ------------------------------------ epilogue warps (alignment)
+        // 8 warps: TMEM lane quarter q = warp % 4, column half ch of the tile
+        const int q = warp & 3, ch = (warp - 4) >> 2;
+        const int il = q * 32 + lane;
+        int buf = 0;
+        uint32_t acc_phase = 0;
+        for (int t = t_begin; t < t_end; ++t) {
+            const TcTile tl = p.tiles[t];
+            const TcMod& md = p.mods[tl.mod];
+            const int nn = md.n, mkb = md.kb;
+            const int i = (2 * tl.t0 + crank) * K2_BM + il, c0 = tl.t1 * K2_BN + ch * (K2_BN / 2);
+            const bool row_ok = i < md.m;
+            const uint16_t* const grow = p.G[tl.slot] + (long long)i * nn;
+            const float* const mrow = md.mag + (long long)i * mkb;
+            // 16 entries of this row of G and the norms of their blocks (n is
+            // a multiple of 8; zero past n)
+            constexpr int NM = BLK >= 16 ? 1 : 16 / BLK;
+            auto load = [&](int c, uint4 (&g)[2], float (&mg)[NM]) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    g[h] = make_uint4(0u, 0u, 0u, 0u);
+                    if (row_ok && c + 8 * h < nn) g[h] = __ldg(reinterpret_cast<const uint4*>(grow + c + 8 * h));
+                }
+#pragma unroll
+                for (int d = 0; d < NM; ++d)
+                    mg[d] = row_ok && c + d * BLK < nn ? __ldg(mrow + (c + d * BLK) / BLK) : 0.0f;
+            };
+            uint4 g[2], gn[2];
+            float mg[NM], mgn[NM];
+            load(c0, g, mg);
+            const bool got = ptx::mbar_wait(ptx::smem_u32(&ctl->accf[buf]), acc_phase, abort_flag, p.status,
+                                            MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit);
+            if (!__all_sync(0xffffffffu, got)) break;
+            ptx::tc_fence_after();
+            float dot = 0.0f, na = 0.0f, gg = 0.0f;
+#pragma unroll 1
+            for (int c = 0; c < K2_BN / 2; c += 16) {
+                if (c0 + c >= nn) break;                   // warp-uniform
+                load(c0 + c + 16, gn, mgn);                // zeros past the tile's half are not used
+                float v[16];
+                __syncwarp();
+                ptx::tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + buf * 256 + ch * (K2_BN / 2) + c, v);
+                const uint32_t w[8] = {g[0].x, g[0].y, g[0].z, g[0].w, g[1].x, g[1].y, g[1].z, g[1].w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const float x = bf_lo(w[e]), y = bf_hi(w[e]);
+                    const float m = mg[NM == 1 ? 0 : 2 * e / BLK];
+                    // columns past n: G and the product's columns are zero
+                    const float a0 = m * v[2 * e], a1 = m * v[2 * e + 1];
+                    dot = fmaf(x, a0, dot);
+                    dot = fmaf(y, a1, dot);
+                    na = fmaf(a0, a0, na);
+                    na = fmaf(a1, a1, na);
+                    gg = fmaf(x, x, gg);
+                    gg = fmaf(y, y, gg);
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) g[h] = gn[h];
+#pragma unroll
+                for (int d = 0; d < NM; ++d) mg[d] = mgn[d];
+            }
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {   // the even CTA's issuer waits for both CTAs' epilogues
+                if (crank == 0) ptx::mbar_arrive(ptx::smem_u32(&ctl->acce[buf]));
+                else ptx::mbar_arrive_remote(ptx::mapa(ptx::smem_u32(&ctl->acce[buf]), 0));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                na += __shfl_xor_sync(0xffffffffu, na, o);
+                gg += __shfl_xor_sync(0xffffffffu, gg, o);
+            }
+            if (lane == 0) {
+                double* acc = p.acc + 3 * tl.slot;
+                atomicAdd(acc + 0, static_cast<double>(dot));
+                atomicAdd(acc + 1, static_cast<double>(na));
+                atomicAdd(acc + 2, static_cast<double>(gg));
+            }
+            if (++buf == 2) { buf = 0; acc_phase ^= 1; }
         }
     } else {
         // ------------------------------------------------- epilogue warps
@@ -1065,8 +1180,8 @@ k2_backproject(const __grid_constant__ K2Params p) {
 // Martinsson and Tropp, 2011 -- this library's choice of method, not the
 // paper's): out (M x N) = op(A) B with fp32 accumulation,
 // written in fp32 and/or bf16.  A is read K-major (stored M x K) or MN-major
-// (stored K x M), optionally as two planes A_hi + A_lo (two MMAs per k-step
-// keep ~16 significant bits of A, used for V); B is stored K x N (MN-major).
+// (stored K x M); A or B may come as two planes hi + lo (two MMAs per k-step
+// keep ~16 significant bits, used for V); B is stored K x N (MN-major).
 // Used for V^T Q, V Z, the Gram matrices X^T X and the triangular factor
 // products X R^-1.  Tile 256 x 256 (two 128-row accumulators in TMEM), BK =
 // 64, one tile per CTA: the contractions are long enough that the epilogue
@@ -1076,7 +1191,7 @@ k2_backproject(const __grid_constant__ K2Params p) {
 // ===========================================================================
 constexpr int KR_BM = 256, KR_BN = 256, KR_BK = 64;
 constexpr int KR_PLANE = KR_BM * KR_BK * 2;               // 32 KB: one A plane or the B tile
-template <bool LO> struct KrCfg {
+template <int LO> struct KrCfg {
     static constexpr int STAGES = LO ? 2 : 3;
     static constexpr int STAGE_BYTES = (LO ? 3 : 2) * KR_PLANE;
 };
@@ -1087,19 +1202,11 @@ constexpr int kKrGroup = 64;                              // problems per launch
 
 struct KrParams {
     CUtensorMap amap[kKrGroup];        // A_hi, box {64, 64}
-    CUtensorMap lmap[kKrGroup];        // A_lo (same geometry), unused without LO
+    CUtensorMap lmap[kKrGroup];        // A_lo or B_lo (the geometry of A or B), unused without LO
     CUtensorMap bmap[kKrGroup];        // B ({N, K}), box {64, 64}
     float* out[kKrGroup];              // M x N fp32 or null
     uint16_t* out_bf[kKrGroup];        // M x N bf16 or null
     uint16_t* out_lo[kKrGroup];        // M x N bf16 residual (out - bf16(out)) or null
-    // alignment reduction (ALIGN): element (j, i) of the product (al_tr) or
-    // element (i, j), weighted by the block norm mag[i][j / al_B], is dotted
-    // with G[i][j]; al_m is the number of valid product columns
-    const uint16_t* al_G[kKrGroup];
-    const float* al_mag[kKrGroup];
-    double* al_acc[kKrGroup];          // 3 doubles: <G, a>, <a, a>, <G, G>
-    int al_ld[kKrGroup], al_kb[kKrGroup], al_m[kKrGroup], al_tr[kKrGroup];
-    int al_B, al_log2B;                // block size (a power of two) and its log2
     int M[kKrGroup], N[kKrGroup], K[kKrGroup];
     int ktri[kKrGroup];
     int lower[kKrGroup];               // tiles above the diagonal are skipped
@@ -1112,7 +1219,8 @@ struct KrParams {
 
 static_assert(sizeof(KrParams) <= 32764, "KR's parameter block fits the kernel parameter space");
 
-template <bool KMAJOR, bool LO, bool ALIGN = false>
+// LO: 1 adds the MMA with A's residual plane, 2 with B's.
+template <bool KMAJOR, int LO>
 __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constant__ KrParams p) {
     constexpr int STAGES = KrCfg<LO>::STAGES;
     constexpr int STAGE_BYTES = KrCfg<LO>::STAGE_BYTES;
@@ -1164,7 +1272,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
             int stage = 0;
             uint32_t phase = 0;
             uint32_t issued = 0, last_par = 0;
-            const uint32_t bytes = (LO ? 2 : 1) * KR_PLANE + nch * 8192;
+            const uint32_t bytes = (LO == 1 ? 2 : 1) * KR_PLANE + (LO == 2 ? 2 : 1) * nch * 8192;
             for (int kb = 0; kb < nk; ++kb) {
                 if (!ptx::mbar_wait(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1, abort_flag, p.status,
                                     MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit))
@@ -1172,15 +1280,18 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
                 const uint32_t fb = ptx::smem_u32(&ctl->full[stage]);
                 ptx::mbar_arrive_expect_tx(fb, bytes);
                 const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
-                const uint32_t b = a + (LO ? 2 : 1) * KR_PLANE;
+                const uint32_t b = a + (LO == 1 ? 2 : 1) * KR_PLANE;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const int x = KMAJOR ? kb * KR_BK : i0 + 64 * c;
                     const int y = KMAJOR ? i0 + 64 * c : kb * KR_BK;
                     ptx::tma_load_2d(a + c * 8192, &p.amap[pi], fb, x, y);
-                    if (LO) ptx::tma_load_2d(a + KR_PLANE + c * 8192, &p.lmap[pi], fb, x, y);
+                    if (LO == 1) ptx::tma_load_2d(a + KR_PLANE + c * 8192, &p.lmap[pi], fb, x, y);
                 }
-                for (int c = 0; c < nch; ++c) ptx::tma_load_2d(b + c * 8192, &p.bmap[pi], fb, n0 + 64 * c, kb * KR_BK);
+                for (int c = 0; c < nch; ++c) {
+                    ptx::tma_load_2d(b + c * 8192, &p.bmap[pi], fb, n0 + 64 * c, kb * KR_BK);
+                    if (LO == 2) ptx::tma_load_2d(b + KR_PLANE + c * 8192, &p.lmap[pi], fb, n0 + 64 * c, kb * KR_BK);
+                }
                 issued |= 1u << stage;
                 last_par = (last_par & ~(1u << stage)) | (phase << stage);
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -1200,7 +1311,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
                                     MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit)) break;
                 ptx::tc_fence_after();
                 const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
-                const uint32_t b = a + (LO ? 2 : 1) * KR_PLANE;
+                const uint32_t b = a + (LO == 1 ? 2 : 1) * KR_PLANE;
                 for (int h = 0; h < halves; ++h) {
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
@@ -1209,11 +1320,14 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
                                                       : ptx::smem_desc_sw128(ao, 8192, 1024);
                         const uint64_t bdesc = ptx::smem_desc_sw128(b + kk * 2048, 8192, 1024);
                         ptx::mma_f16(tmem + h * 256, adesc, bdesc, idesc, (kb | kk) != 0);
-                        if (LO) {
+                        if (LO == 1) {
                             const uint32_t lo_addr = ao + KR_PLANE;
                             const uint64_t ldesc = KMAJOR ? ptx::smem_desc_sw128(lo_addr, 16, 1024)
                                                           : ptx::smem_desc_sw128(lo_addr, 8192, 1024);
                             ptx::mma_f16(tmem + h * 256, ldesc, bdesc, idesc, 1);
+                        } else if (LO == 2) {
+                            ptx::mma_f16(tmem + h * 256, adesc,
+                                         ptx::smem_desc_sw128(b + KR_PLANE + kk * 2048, 8192, 1024), idesc, 1);
                         }
                     }
                 }
@@ -1231,67 +1345,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
         const int h = ew >> 2;
         const bool got = ptx::mbar_wait(ptx::smem_u32(&ctl->accf[0]), 0, abort_flag, p.status,
                                         MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit);
-        if (ALIGN && __all_sync(0xffffffffu, got) && h < halves) {
-            // S(W, t) of §3.2: this thread's row of the product -- row j of
-            // (P P^T V)^T against column j of G, or row i of V Q Q^T against
-            // row i of G -- weighted by Rep_B(M)
-            ptx::tc_fence_after();
-            const int row = i0 + h * 128 + q * 32 + lane;
-            const uint16_t* const Gp = p.al_G[pi];
-            const float* const mg = p.al_mag[pi];
-            const int ldg = p.al_ld[pi], kbm = p.al_kb[pi], mm = p.al_m[pi];
-            const bool tr = p.al_tr[pi] != 0;
-            const int lgB = p.al_log2B;
-            const int jb = row >> lgB;
-            float dot = 0.0f, na = 0.0f, gg = 0.0f;
-            for (int c = 0; c < nch * 4; ++c) {
-                const int c0 = n0 + c * 16;
-                if (c0 >= mm) break;                      // warp-uniform
-                float v[16];
-                __syncwarp();
-                ptx::tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + h * 256 + c * 16, v);
-                if (row >= M) continue;
-                if (tr) {                                 // product entry (j, i): G[i][j], M[i][j / B]
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int ci = c0 + e;
-                        if (ci < mm) {
-                            const float g = __bfloat162float(__ushort_as_bfloat16(Gp[(long long)ci * ldg + row]));
-                            const float a = mg[(long long)ci * kbm + jb] * v[e];
-                            dot = fmaf(g, a, dot);
-                            na = fmaf(a, a, na);
-                            gg = fmaf(g, g, gg);
-                        }
-                    }
-                } else {                                  // product entry (i, j): G[i][j], M[i][j / B]
-                    const uint16_t* grow = Gp + (long long)row * ldg;
-                    const float* mrow = mg + (long long)row * kbm;
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int ci = c0 + e;
-                        if (ci < mm) {
-                            const float g = __bfloat162float(__ushort_as_bfloat16(grow[ci]));
-                            const float a = mrow[ci >> lgB] * v[e];
-                            dot = fmaf(g, a, dot);
-                            na = fmaf(a, a, na);
-                            gg = fmaf(g, g, gg);
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                na += __shfl_xor_sync(0xffffffffu, na, o);
-                gg += __shfl_xor_sync(0xffffffffu, gg, o);
-            }
-            if (lane == 0) {
-                double* acc = p.al_acc[pi];
-                atomicAdd(acc + 0, static_cast<double>(dot));
-                atomicAdd(acc + 1, static_cast<double>(na));
-                atomicAdd(acc + 2, static_cast<double>(gg));
-            }
-        } else if (!ALIGN && __all_sync(0xffffffffu, got) && h < halves) {
+        if (__all_sync(0xffffffffu, got) && h < halves) {
             ptx::tc_fence_after();
             const int row = i0 + h * 128 + q * 32 + lane;
             uint16_t* const ol = p.out_lo[pi];
@@ -1589,6 +1643,7 @@ int max_clusters(const void* fn, int threads, int smem, int cap) {
 template <int BLK>
 void set_smem_attrs() {
     cudaFuncSetAttribute(k2_backproject<BLK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_SMEM);
+    cudaFuncSetAttribute(k2_backproject<BLK, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_SMEM);
     if constexpr (BLK >= 32)
         cudaFuncSetAttribute(k2_backproject<BLK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, K2_SMEM);
 }
@@ -1728,6 +1783,9 @@ int tc_register(TcState* st, int id, const ModDev& md, const moara_hparams& hp) 
              encode_2d(st->encode, &mp[6], sdt, ses, md.exp_avg, md.r, md.m, scols, K1_BM) &&
              encode_2d(st->encode, &mp[7], sdt, ses, md.exp_avg_sq, md.r, md.m, scols, K1_BM);
     }
+    // residual plane of N for the alignment diagnostic, after its hi plane
+    ok = ok && (md.right ? encode_bf16_2d(st->encode, &mp[9], t.Nb + (size_t)md.m * md.r, md.r, md.m, 64, 128)
+                         : encode_bf16_2d(st->encode, &mp[9], t.Nb + (size_t)md.r * md.n, md.n, md.r, 64, 64));
     ok = ok && encode_2d(st->encode, &mp[3], sdt, ses, md.W, md.n, md.m, scols, K2_BM);
     if (!ok) {
         st->err = "cuTensorMapEncodeTiled failed";
@@ -1812,6 +1870,25 @@ static void lpt_assign(const std::vector<TcTile>& tiles, const std::vector<doubl
         for (int i : per[c]) out.push_back(tiles[i]);
     }
     start[grid] = static_cast<int>(out.size());
+}
+
+// Shared-memory limits of the step kernels and their resident grids.
+static void tc_init(TcState* st) {
+    if (!st->attrs_set) {
+        for (auto fn : {k1_project<true, false, false>, k1_project<false, false, false>, k1_project<true, true, false>,
+                        k1_project<false, true, false>, k1_project<true, false, true>, k1_project<false, false, true>,
+                        k1_project<true, true, true>, k1_project<false, true, true>})
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, K1_SMEM);
+        set_smem_attrs<8>(); set_smem_attrs<16>(); set_smem_attrs<32>(); set_smem_attrs<64>();
+        set_smem_attrs<128>();
+        // clusters of two that fit on the GPU at once (persistent grids)
+        st->k1_clusters = max_clusters(reinterpret_cast<const void*>(k1_project<false, false, false>), K1_THREADS,
+                                       K1_SMEM,
+                                       st->sms / 2);
+        st->k2_clusters = max_clusters(reinterpret_cast<const void*>(k2_backproject<128, false>), K2_THREADS, K2_SMEM,
+                                       st->sms / 2);
+        st->attrs_set = true;
+    }
 }
 
 // Work lists of one launch: K1 tiles (128-rank x 256-column) and K2 tiles
@@ -1968,21 +2045,7 @@ int tc_group_limit() { return kTcGroup; }
 int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, const void* const* G, float bc1,
             float bc2, float lr, int first_step, const float* clip, const TcClipFuse* fuse, cudaStream_t s,
             int64_t* launches, const TcProfile& prof) {
-    if (!st->attrs_set) {
-        for (auto fn : {k1_project<true, false, false>, k1_project<false, false, false>, k1_project<true, true, false>,
-                        k1_project<false, true, false>, k1_project<true, false, true>, k1_project<false, false, true>,
-                        k1_project<true, true, true>, k1_project<false, true, true>})
-            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, K1_SMEM);
-        set_smem_attrs<8>(); set_smem_attrs<16>(); set_smem_attrs<32>(); set_smem_attrs<64>();
-        set_smem_attrs<128>();
-        // clusters of two that fit on the GPU at once (persistent grids)
-        st->k1_clusters = max_clusters(reinterpret_cast<const void*>(k1_project<false, false, false>), K1_THREADS,
-                                       K1_SMEM,
-                                       st->sms / 2);
-        st->k2_clusters = max_clusters(reinterpret_cast<const void*>(k2_backproject<128, false>), K2_THREADS, K2_SMEM,
-                                       st->sms / 2);
-        st->attrs_set = true;
-    }
+    tc_init(st);
     int rc = tc_upload(st);
     if (rc != MOARA_OK) return rc;
     const bool dec = hp.decompose != 0;
@@ -2164,18 +2227,12 @@ void tc_set_wait_limit(TcState* st, long long cycles) {
     if (st != nullptr) st->wait_limit = cycles > 0 ? cycles : kWaitLimit;
 }
 
-// Grouped KR launches; with align_B > 0 the alignment epilogue (A K-major
-// with two planes only) replaces the stores.
-static int kr_launch(TcState* st, int a_kmajor, const TcGemmItem* items, int count, int align_B,
-                     const uint16_t* const* al_G, const float* const* al_mag, const int* al_ld, const int* al_kb,
-                     const int* al_m, double* const* al_acc, cudaStream_t s, int64_t* launches,
-                     const int* al_tr = nullptr) {
+int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, cudaStream_t s,
+                 int64_t* launches) {
     if (!st->kr_attrs) {
-        cudaFuncSetAttribute(kr_product<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
-        cudaFuncSetAttribute(kr_product<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
-        cudaFuncSetAttribute(kr_product<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
-        cudaFuncSetAttribute(kr_product<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
-        cudaFuncSetAttribute(kr_product<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
+        for (auto fn : {kr_product<true, 0>, kr_product<true, 1>, kr_product<true, 2>, kr_product<false, 0>,
+                        kr_product<false, 1>, kr_product<false, 2>})
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
         st->kr_attrs = true;
     }
     for (int i = 0; i < count; ++i) {
@@ -2185,16 +2242,13 @@ static int kr_launch(TcState* st, int a_kmajor, const TcGemmItem* items, int cou
             st->err = "tensor-core refresh GEMM: row pitches must be multiples of 16 bytes";
             return MOARA_ERR_UNSUPPORTED;
         }
-        if (align_B > 0 && (!a_kmajor || x.A_lo == nullptr)) {
-            st->err = "alignment product: A must be K-major with two planes";
-            return MOARA_ERR_UNSUPPORTED;
-        }
     }
-    // two sub-launches: items with and without the A_lo plane
-    for (int with_lo = 0; with_lo < 2; ++with_lo) {
+    // sub-launches: items without a residual plane, with A's, with B's
+    auto kind = [](const TcGemmItem& x) { return x.A_lo != nullptr ? 1 : x.B_lo != nullptr ? 2 : 0; };
+    for (int with_lo = 0; with_lo < 3; ++with_lo) {
         std::vector<int> sel;
         for (int i = 0; i < count; ++i)
-            if ((items[i].A_lo != nullptr) == (with_lo == 1)) sel.push_back(i);
+            if (kind(items[i]) == with_lo) sel.push_back(i);
         for (size_t c0 = 0; c0 < sel.size(); c0 += kKrGroup) {
             const int cnt = static_cast<int>(std::min<size_t>(kKrGroup, sel.size() - c0));
             KrParams& kp = st->pr;
@@ -2205,7 +2259,8 @@ static int kr_launch(TcState* st, int a_kmajor, const TcGemmItem* items, int cou
                 const TcGemmItem& x = items[it];
                 const uint64_t a_cols = a_kmajor ? x.K : x.M, a_rows = a_kmajor ? x.M : x.K;
                 bool ok = encode_bf16_2d(st->encode, &kp.amap[q], x.A, a_cols, a_rows, 64, 64);
-                if (with_lo) ok = ok && encode_bf16_2d(st->encode, &kp.lmap[q], x.A_lo, a_cols, a_rows, 64, 64);
+                if (with_lo == 1) ok = ok && encode_bf16_2d(st->encode, &kp.lmap[q], x.A_lo, a_cols, a_rows, 64, 64);
+                if (with_lo == 2) ok = ok && encode_bf16_2d(st->encode, &kp.lmap[q], x.B_lo, x.N, x.K, 64, 64);
                 ok = ok && encode_bf16_2d(st->encode, &kp.bmap[q], x.B, x.N, x.K, 64, 64);
                 if (!ok) {
                     st->err = "cuTensorMapEncodeTiled failed for a refresh operand";
@@ -2214,11 +2269,6 @@ static int kr_launch(TcState* st, int a_kmajor, const TcGemmItem* items, int cou
                 kp.out[q] = x.out;
                 kp.out_bf[q] = x.out_bf16;
                 kp.out_lo[q] = x.out_lo;
-                if (align_B > 0) {
-                    kp.al_G[q] = al_G[it]; kp.al_mag[q] = al_mag[it]; kp.al_acc[q] = al_acc[it];
-                    kp.al_ld[q] = al_ld[it]; kp.al_kb[q] = al_kb[it]; kp.al_m[q] = al_m[it];
-                    kp.al_tr[q] = al_tr != nullptr ? al_tr[it] : 1;
-                }
                 kp.M[q] = x.M; kp.N[q] = x.N; kp.K[q] = x.K;
                 kp.ktri[q] = x.ktri;
                 kp.lower[q] = x.lower;
@@ -2230,19 +2280,11 @@ static int kr_launch(TcState* st, int a_kmajor, const TcGemmItem* items, int cou
             kp.count = cnt;
             kp.status = st->d_status;
             kp.wait_limit = st->wait_limit;
-            kp.al_B = align_B;
-            kp.al_log2B = 0;
-            while ((1 << kp.al_log2B) < align_B) ++kp.al_log2B;
             if (total == 0) continue;
-            if (align_B > 0) {
-                kr_product<true, true, true><<<total, KR_THREADS, KR_SMEM, s>>>(kp);
-            } else if (!a_kmajor) {
-                if (with_lo) kr_product<false, true><<<total, KR_THREADS, KR_SMEM, s>>>(kp);
-                else kr_product<false, false><<<total, KR_THREADS, KR_SMEM, s>>>(kp);
-            } else {
-                if (with_lo) kr_product<true, true><<<total, KR_THREADS, KR_SMEM, s>>>(kp);
-                else kr_product<true, false><<<total, KR_THREADS, KR_SMEM, s>>>(kp);
-            }
+            auto fn = a_kmajor ? (with_lo == 0 ? kr_product<true, 0> : with_lo == 1 ? kr_product<true, 1> : kr_product<true, 2>)
+                               : (with_lo == 0 ? kr_product<false, 0>
+                                               : with_lo == 1 ? kr_product<false, 1> : kr_product<false, 2>);
+            fn<<<total, KR_THREADS, KR_SMEM, s>>>(kp);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) {
                 st->err = cudaGetErrorString(e);
@@ -2252,12 +2294,6 @@ static int kr_launch(TcState* st, int a_kmajor, const TcGemmItem* items, int cou
         }
     }
     return MOARA_OK;
-}
-
-int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, cudaStream_t s,
-                 int64_t* launches) {
-    return kr_launch(st, a_kmajor, items, count, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, s,
-                     launches);
 }
 
 // out (cols x ld_out, bf16) = in^T for in (rows x cols, bf16, row pitch
@@ -2312,12 +2348,8 @@ int tc_alignment(TcState* st, const moara_hparams& hp, int n_mod, const int* ids
             st->err = "alignment: module is not on the tensor-core path";
             return MOARA_ERR_UNSUPPORTED;
         }
-        const long long mp = (md->m + 7) / 8 * 8;
-        if ((long long)md->r * mp > 2LL * md->m * md->n) {
-            st->err = "alignment: workspace too small for the transposed projector";
-            return MOARA_ERR_UNSUPPORTED;
-        }
     }
+    tc_init(st);
     int rc = tc_upload(st);
     if (rc != MOARA_OK) return rc;
     // 1. block norms M (into the module's norm buffer) and V = V_hi + V_lo
@@ -2352,65 +2384,53 @@ int tc_alignment(TcState* st, const moara_hparams& hp, int n_mod, const int* ids
             return MOARA_ERR_CUDA;
         }
     }
-    // 2. left projector: R^T = V^T P (n x r); right projector: R = V Q
-    //    (m x r); as two bf16 planes in the module's N buffer
+    // 2. R = P^T V (r x n), or V Q (m x r) with a right projector, V in two
+    //    planes, as two bf16 planes in the module's N buffer
     std::vector<TcGemmItem> g1[2];
     for (int q = 0; q < n_mod; ++q) {
         const TcMod& md = st->mods[ids[q]];
-        if (!md.right)
-            g1[0].push_back(TcGemmItem{md.Vhi, md.Vlo, md.Pb, nullptr, md.Nb, md.n, md.r, md.m, 0,
-                                       md.Nb + (size_t)md.n * md.r});
-        else
+        if (!md.right) {
+            TcGemmItem g{md.Pb, nullptr, md.Vhi, nullptr, md.Nb, md.r, md.n, md.m, 0, md.Nb + (size_t)md.r * md.n};
+            g.B_lo = md.Vlo;
+            g1[0].push_back(g);
+        } else {
             g1[1].push_back(TcGemmItem{md.Vhi, md.Vlo, md.Pb, nullptr, md.Nb, md.m, md.r, md.n, 0,
                                        md.Nb + (size_t)md.m * md.r});
+        }
     }
     for (int side = 0; side < 2; ++side) {
         if (g1[side].empty()) continue;
-        rc = kr_launch(st, side, g1[side].data(), static_cast<int>(g1[side].size()), 0, nullptr, nullptr, nullptr,
-                       nullptr, nullptr, nullptr, s, launches);
+        rc = tc_gemm_bf16(st, side, g1[side].data(), static_cast<int>(g1[side].size()), s, launches);
         if (rc != MOARA_OK) return rc;
     }
-    // 3. left projector: P^T (r x mp, zero-padded columns) over the V planes,
-    //    now free (a right projector's Q^T is kept in the workspace)
-    for (int q = 0; q < n_mod; ++q) {
-        const TcMod& md = st->mods[ids[q]];
-        if (md.right) continue;
-        const int mp = (md.m + 7) / 8 * 8;
-        const int tiles = ((mp + 31) / 32) * ((md.r + 31) / 32);
-        k_transpose_pad_bf16<<<std::min(tiles, st->sms * 8), 256, 0, s>>>(md.Pb, md.Vhi, md.m, md.r, mp);
-        ++*launches;
-    }
+    // 3. P R, or R Q^T, reduced against G
     if (cudaMemsetAsync(acc, 0, sizeof(double) * 3 * (size_t)n_mod, s) != cudaSuccess) {
         st->err = "alignment accumulator reset failed";
         return MOARA_ERR_CUDA;
     }
-    // 4. left: (P R)^T = R^T P^T (n x mp); right: V Q Q^T = R Q^T (m x n);
-    //    reduced against G in the epilogue
-    std::vector<TcGemmItem> g2(n_mod);
-    std::vector<const uint16_t*> aG(n_mod);
-    std::vector<const float*> aM(n_mod);
-    std::vector<int> ald(n_mod), akb(n_mod), am(n_mod), atr(n_mod);
-    std::vector<double*> aacc(n_mod);
-    for (int q = 0; q < n_mod; ++q) {
-        const TcMod& md = st->mods[ids[q]];
-        if (!md.right) {
-            const int mp = (md.m + 7) / 8 * 8;
-            g2[q] = TcGemmItem{md.Nb, md.Nb + (size_t)md.n * md.r, md.Vhi, nullptr, nullptr, md.n, mp, md.r, 0, nullptr};
-            am[q] = md.m;
-            atr[q] = 1;
-        } else {
-            g2[q] = TcGemmItem{md.Nb, md.Nb + (size_t)md.m * md.r, md.Qt, nullptr, nullptr, md.m, md.n, md.r, 0, nullptr};
-            am[q] = md.n;
-            atr[q] = 0;
+    for (int c0 = 0; c0 < n_mod; c0 += kTcGroup) {
+        const int cnt = std::min(kTcGroup, n_mod - c0);
+        TcState::Tiles* tl = tc_tiles(st, std::vector<int>(ids + c0, ids + c0 + cnt));
+        if (tl == nullptr) { st->err = "tile list allocation failed"; return MOARA_ERR_CUDA; }
+        K2AlignParams p2{};
+        p2.cta_start = tl->k2_start; p2.tiles = tl->k2;
+        p2.mods = st->d_mods; p2.maps = st->d_maps; p2.status = st->d_status;
+        p2.acc = acc + 3 * (size_t)c0;
+        for (int q = 0; q < cnt; ++q) p2.G[q] = static_cast<const uint16_t*>(G[c0 + q]);
+        const int g2 = 2 * tl->g2;
+        switch (B) {
+            case 8: k2_backproject<8, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
+            case 16: k2_backproject<16, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
+            case 32: k2_backproject<32, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
+            case 64: k2_backproject<64, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
+            default: k2_backproject<128, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
         }
-        aG[q] = static_cast<const uint16_t*>(G[q]);
-        aM[q] = md.mag;
-        ald[q] = md.n; akb[q] = md.kb;
-        aacc[q] = acc + 3 * q;
+        ++*launches;
+        if (cudaGetLastError() != cudaSuccess) {
+            st->err = "alignment product launch failed";
+            return MOARA_ERR_CUDA;
+        }
     }
-    rc = kr_launch(st, 1, g2.data(), n_mod, B, aG.data(), aM.data(), ald.data(), akb.data(), am.data(),
-                   aacc.data(), s, launches, atr.data());
-    if (rc != MOARA_OK) return rc;
     k_align_finish<<<(n_mod + 127) / 128, 128, 0, s>>>(acc, S_out, n_mod);
     ++*launches;
     if (cudaGetLastError() != cudaSuccess) {

@@ -50,6 +50,7 @@ struct TcGemmItem {
     int ktri;              // B upper triangular: column j needs k <= j only
     uint16_t* out_lo;      // M x N row-major bf16 residual out - bf16(out), or null
     int lower;             // 1: only output tiles on or below the diagonal (M = N)
+    const uint16_t* B_lo;  // residual plane of B (with A_lo null), or null
 };
 
 // Grouped launch of TcGemmItems (A read K-major when a_kmajor, else
@@ -104,9 +105,10 @@ cudaError_t tc_transpose_bf16(const uint16_t* in, uint16_t* out, int rows, int c
 
 const char* tc_last_error(const TcState* st);
 
-// Clock cycles a bounded wait of the refresh / alignment product kernels (KR,
-// KS) spins before it gives up and records MOARA_ERR_DEVICE_TIMEOUT; <= 0
-// restores the default (~2 s).
+// Clock cycles a bounded wait of the refresh and alignment products on KR and
+// KS spins before it gives up and records MOARA_ERR_DEVICE_TIMEOUT; <= 0
+// restores the default (~2 s); the alignment's second product, on the step
+// kernels' CTA pairs, keeps the default.
 void tc_set_wait_limit(TcState* st, long long cycles);
 
 }  // namespace moara
