@@ -91,6 +91,7 @@ struct GemmProb {
     int lower_only;       // skip output tiles strictly above the diagonal
     int k_tri;            // triangular operand: the K range of an output tile shrinks (KTRI_*)
     uint16_t* c_bf16;     // EPI_STORE: also write C rounded to bf16 here (same layout), or null
+    int split;            // parts of the K range (set at launch)
 };
 
 template <int CAP>

@@ -411,7 +411,8 @@ __global__ void __launch_bounds__(256, 4) k_gemm_small(const __grid_constant__ G
     else if (p.k_tri == KTRI_B_LOWER) kbeg = min(p.K, n0);
     else if (p.k_tri == KTRI_A_LOWER) kend = min(p.K, m0 + SM_T);
     const int chunks = kend > kbeg ? (kend - kbeg + SM_K - 1) / SM_K : 0;
-    const int c0 = chunks * rank / S, c1 = chunks * (rank + 1) / S;
+    const int split = p.split;                        // <= S; the other ranks only help to store
+    const int c0 = rank < split ? chunks * rank / split : 0, c1 = rank < split ? chunks * (rank + 1) / split : 0;
     SliceLoader<ALAY == A_KCONTIG, ASC, ABF> la;
     SliceLoader<BLAY == B_KCONTIG, BSC, BBF> lb;
     auto load = [&](int c) {
@@ -451,7 +452,7 @@ __global__ void __launch_bounds__(256, 4) k_gemm_small(const __grid_constant__ G
         const int i = rank * R + e / SM_T, j = e % SM_T;
         float v = 0.0f;
         if (S > 1) {
-            for (int q = 0; q < S; ++q) v += *cl.map_shared_rank(&part[i][j], q);
+            for (int q = 0; q < split; ++q) v += *cl.map_shared_rank(&part[i][j], q);
         } else {
             v = part[i][j];
         }
@@ -462,6 +463,17 @@ __global__ void __launch_bounds__(256, 4) k_gemm_small(const __grid_constant__ G
 
 constexpr int kWideTiles = 304;       // two 128 x 128 tiles per SM
 constexpr int kSmallCtas = 608;       // four 64 x 64 CTAs per SM
+
+// Parts of a problem's K range: up to eight while the problem's own tiles leave
+// SMs idle and a part has a slice of its own.  From the problem alone, so that
+// its sums do not depend on what it is grouped with (both kernels add the
+// terms of a part in the order of k).
+static int k_split(const GemmProb& p) {
+    const int tiles = (p.M + SM_T - 1) / SM_T * ((p.N + SM_T - 1) / SM_T);
+    int split = 1;
+    while (split < 8 && 2 * split * tiles <= kSmallCtas && p.K >= 2 * split * SM_K) split *= 2;
+    return split;
+}
 
 template <int CAP, int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
 static cudaError_t launch_small(const GemmBatch& b, int total, int split, cudaStream_t s) {
@@ -496,13 +508,7 @@ static cudaError_t launch_small(const GemmBatch& b, int total, int split, cudaSt
 }
 
 template <int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
-static cudaError_t launch_one(GemmBatch& b, cudaStream_t s, int64_t* launches) {
-    b.log2B = -1;
-    if (b.B > 0 && (b.B & (b.B - 1)) == 0) {
-        int lg = 0;
-        while ((1 << lg) < b.B) ++lg;
-        b.log2B = lg;
-    }
+static cudaError_t launch_part(GemmBatch& b, cudaStream_t s, int64_t* launches) {
     auto enumerate = [&](int tm_, int tn_) {
         int total = 0;
         for (int i = 0; i < b.count; ++i) {
@@ -516,23 +522,47 @@ static cudaError_t launch_one(GemmBatch& b, cudaStream_t s, int64_t* launches) {
         b.tile_start[b.count] = total;
         return total;
     };
+    int split = 1;
+    for (int i = 0; i < b.count; ++i) split = b.p[i].split > split ? b.p[i].split : split;
     int total = enumerate(TM, TN);
     if (total == 0) return cudaSuccess;
     ++*launches;
-    if (total >= kWideTiles) {
+    if (split == 1 && total >= kWideTiles) {
         // enough 128 x 128 tiles for every SM: half the shared-memory reads
         // per FMA of the small kernel
         k_gemm<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI><<<total, 256, 0, s>>>(b);
         return cudaGetLastError();
     }
     total = enumerate(SM_T, SM_T);
-    int kmax = 0;
-    for (int i = 0; i < b.count; ++i) kmax = b.p[i].K > kmax ? b.p[i].K : kmax;
-    int split = 1;
-    while (split < 8 && 2 * split * total <= kSmallCtas && kmax >= 2 * split * SM_K) split *= 2;
     if (b.count <= kFewGroup)
         return launch_small<kFewGroup, ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(b, total, split, s);
     return launch_small<kMaxGroup, ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(b, total, split, s);
+}
+
+template <int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
+static cudaError_t launch_one(GemmBatch& b, cudaStream_t s, int64_t* launches) {
+    b.log2B = -1;
+    if (b.B > 0 && (b.B & (b.B - 1)) == 0) {
+        int lg = 0;
+        while ((1 << lg) < b.B) ++lg;
+        b.log2B = lg;
+    }
+    int whole = 0;
+    for (int i = 0; i < b.count; ++i) {
+        b.p[i].split = k_split(b.p[i]);
+        whole += b.p[i].split == 1;
+    }
+    if (whole == 0 || whole == b.count) return launch_part<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(b, s, launches);
+    // split problems (clusters) and whole ones in launches of their own
+    for (int part = 0; part < 2; ++part) {
+        GemmBatch c = b;
+        c.count = 0;
+        for (int i = 0; i < b.count; ++i)
+            if ((b.p[i].split == 1) == (part == 1)) c.p[c.count++] = b.p[i];
+        const cudaError_t e = launch_part<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(c, s, launches);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Dispatch over the operand/epilogue combinations the library uses.
