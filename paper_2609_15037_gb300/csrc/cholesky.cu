@@ -34,6 +34,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "launch.cuh"
 
 namespace moara {
 
@@ -484,6 +485,7 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ CholBatch b) {
+    pdl_begin();
     extern __shared__ __align__(16) float smem[];
     float (*const buf0)[LD] = reinterpret_cast<float (*)[LD]>(smem);
     float (*const buf1)[LD] = reinterpret_cast<float (*)[LD]>(smem + NB * LD);
@@ -801,20 +803,8 @@ cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches) {
         b.tile_start[b.count] = total;
         b.step = step;
         const int C = b.count <= kCritModules ? kCritCtas : 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(C * b.count + (total + C - 1) / C * C);
-        cfg.blockDim = dim3(NT);
-        cfg.dynamicSmemBytes = CHOL_SMEM;
-        cfg.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = C;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
         ++*launches;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_chol_step, b);
+        const cudaError_t e = launch(k_chol_step, dim3(C * b.count + (total + C - 1) / C * C), NT, CHOL_SMEM, s, C, b);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "launch.cuh"
 
 namespace moara {
 
@@ -43,6 +44,7 @@ __device__ __forceinline__ float u01(uint32_t x) {
 }
 
 __global__ void k_philox_gaussian(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     const int pi = blockIdx.y;
     float* out = b.a[pi];
     uint16_t* hout = b.h[pi];
@@ -80,13 +82,13 @@ cudaError_t launch_philox_gaussian(const SmallBatch& b, cudaStream_t s, int64_t*
     long long most = 1;
     for (int q = 0; q < b.count; ++q) most = std::max(most, ((long long)b.rows[q] * b.l[q] + 4095) / 4096);
     dim3 grid(static_cast<unsigned>(std::min(2048LL, most)), b.count);
-    k_philox_gaussian<<<grid, 256, 0, s>>>(b);
     ++*launches;
-    return cudaGetLastError();
+    return launch(k_philox_gaussian, grid, 256, 0, s, 1, b);
 }
 
 // c <- a and h <- a rounded to bf16 (rows x l entries each).
 __global__ void __launch_bounds__(256) k_copy_bf16(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     const int pi = blockIdx.y;
     const float* src = b.a[pi];
     float* dst = b.c[pi];
@@ -113,9 +115,8 @@ cudaError_t launch_copy_bf16(const SmallBatch& b, cudaStream_t s, int64_t* launc
     if (b.count <= 0) return cudaSuccess;
     long long most = 1;
     for (int q = 0; q < b.count; ++q) most = std::max(most, ((long long)b.rows[q] * b.l[q] + 4095) / 4096);
-    k_copy_bf16<<<dim3(static_cast<unsigned>(std::min(2048LL, most)), b.count), 256, 0, s>>>(b);
     ++*launches;
-    return cudaGetLastError();
+    return launch(k_copy_bf16, dim3(static_cast<unsigned>(std::min(2048LL, most)), b.count), 256, 0, s, 1, b);
 }
 
 constexpr int kSmallThreads = 1024;
@@ -142,6 +143,7 @@ __device__ float block_sum(float v, float* red) {
 // h <- a^T rounded to bf16 (l x l): 32 x 32 tiles through shared memory.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_transpose_bf16(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     __shared__ float t[32][33];
     const int pi = blockIdx.z;
     const int l = b.l[pi];
@@ -172,9 +174,8 @@ cudaError_t launch_transpose_bf16(const SmallBatch& b, cudaStream_t s, int64_t* 
     int lmax = 1;
     for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
     const int tiles = (lmax + 31) / 32;
-    k_transpose_bf16<<<dim3(std::min(1024, tiles * tiles), 1, b.count), 256, 0, s>>>(b);
     ++*launches;
-    return cudaGetLastError();
+    return launch(k_transpose_bf16, dim3(std::min(1024, tiles * tiles), 1, b.count), 256, 0, s, 1, b);
 }
 
 // ---------------------------------------------------------------------------
@@ -185,6 +186,7 @@ cudaError_t launch_transpose_bf16(const SmallBatch& b, cudaStream_t s, int64_t* 
 // shared memory keep both sides coalesced.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_split3(const __grid_constant__ SmallBatch b, int transpose) {
+    pdl_begin();
     __shared__ float t[32][33];
     const int pi = blockIdx.z;
     const int rows = b.rows[pi], cols = b.l[pi];
@@ -255,15 +257,15 @@ cudaError_t launch_split3(const SmallBatch& b, int transpose, cudaStream_t s, in
     long long tiles = 1;
     for (int q = 0; q < b.count; ++q)
         tiles = std::max(tiles, (long long)((b.rows[q] + 31) / 32) * ((b.l[q] + 31) / 32));
-    k_split3<<<dim3(static_cast<unsigned>(std::min(256LL, tiles)), 1, b.count), 256, 0, s>>>(b, transpose);
     ++*launches;
-    return cudaGetLastError();
+    return launch(k_split3, dim3(static_cast<unsigned>(std::min(256LL, tiles)), 1, b.count), 256, 0, s, 1, b, transpose);
 }
 
 // ---------------------------------------------------------------------------
 // a <- I (l x l)
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_set_identity(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     const int pi = blockIdx.y;
     const int l = b.l[pi];
     for (int i = blockIdx.x; i < l; i += gridDim.x) {
@@ -276,9 +278,8 @@ cudaError_t launch_set_identity(const SmallBatch& b, cudaStream_t s, int64_t* la
     if (b.count <= 0) return cudaSuccess;
     int lmax = 1;
     for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
-    k_set_identity<<<dim3(std::min(1024, lmax), b.count), 256, 0, s>>>(b);
     ++*launches;
-    return cudaGetLastError();
+    return launch(k_set_identity, dim3(std::min(1024, lmax), b.count), 256, 0, s, 1, b);
 }
 
 // ---------------------------------------------------------------------------
@@ -288,6 +289,7 @@ cudaError_t launch_set_identity(const SmallBatch& b, cudaStream_t s, int64_t* la
 // launches together take 0.05 ms.)
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kSmallThreads) k_ritz_values(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     __shared__ float s_acc[32][33], s_nrm[32][33];
     const int pi = blockIdx.y;
     const int l = b.l[pi];
@@ -322,6 +324,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_ritz_values(const __grid_cons
 // The descending order of the Ritz values (c): iaux[rank] = j,
 // rank_j = #{i : d_i > d_j, or d_i == d_j and i < j}.
 __global__ void __launch_bounds__(256) k_ritz_order(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     __shared__ float d[1024];
     const int pi = blockIdx.y;
     const int l = b.l[pi];
@@ -363,6 +366,7 @@ constexpr int kLeadW = 64;
 __host__ __device__ inline int lead_slabs(int l) { return l < 2 * kLeadW ? 1 : l / kLeadW; }
 
 __global__ void __launch_bounds__(256) k_lead_gram(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     __shared__ __align__(16) float xs[32][kLeadW], ws[32][kLeadW];
     const int pi = blockIdx.y;
     const int l = b.l[pi];
@@ -405,6 +409,7 @@ constexpr int kJacThreads = 512;
 constexpr int kJacPairs = kLeadW / 2;
 
 __global__ void __launch_bounds__(kJacThreads) k_lead_jacobi(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     __shared__ float H[kLeadW][kLeadW + 1];
     __shared__ float J[kLeadW][kLeadW + 1];
     __shared__ float rc[kJacPairs], rs_[kJacPairs];
@@ -506,6 +511,7 @@ __global__ void __launch_bounds__(kJacThreads) k_lead_jacobi(const __grid_consta
 
 // X_w <- X_w J, W_w <- W_w J: 32 rows of one of the two per CTA.
 __global__ void __launch_bounds__(256) k_lead_rotate(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     __shared__ float js[kLeadW][kLeadW], xs[32][kLeadW];
     const int pi = blockIdx.y;
     const int l = b.l[pi];
@@ -533,27 +539,28 @@ cudaError_t launch_lead_ritz(const SmallBatch& b, cudaStream_t s, int64_t* launc
     if (b.count <= 0) return cudaSuccess;
     int lmax = 1;
     for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
-    k_lead_gram<<<dim3(lead_slabs(lmax), b.count), 256, 0, s>>>(b);
-    k_lead_jacobi<<<b.count, kJacThreads, 0, s>>>(b);
-    k_lead_rotate<<<dim3((lmax + 31) / 32, b.count, 2), 256, 0, s>>>(b);
     *launches += 3;
-    return cudaGetLastError();
+    cudaError_t e = launch(k_lead_gram, dim3(lead_slabs(lmax), b.count), 256, 0, s, 1, b);
+    if (e == cudaSuccess) e = launch(k_lead_jacobi, b.count, kJacThreads, 0, s, 1, b);
+    if (e == cudaSuccess) e = launch(k_lead_rotate, dim3((lmax + 31) / 32, b.count, 2), 256, 0, s, 1, b);
+    return e;
 }
 
 cudaError_t launch_ritz_sort(const SmallBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
     int lmax = 1;
     for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
-    k_ritz_values<<<dim3((lmax + 31) / 32, b.count), kSmallThreads, 0, s>>>(b);
-    k_ritz_order<<<dim3((lmax + 255) / 256, b.count), 256, 0, s>>>(b);
     *launches += 2;
-    return cudaGetLastError();
+    cudaError_t e = launch(k_ritz_values, dim3((lmax + 31) / 32, b.count), kSmallThreads, 0, s, 1, b);
+    if (e == cudaSuccess) e = launch(k_ritz_order, dim3((lmax + 255) / 256, b.count), 256, 0, s, 1, b);
+    return e;
 }
 
 // ---------------------------------------------------------------------------
 // c[:, q] = a[:, iaux[q]] for q < rows (a is l x l, c is l x rows).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_gather_cols(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     const int pi = blockIdx.y;
     const int l = b.l[pi], r = b.rows[pi];
     const int* perm = b.iaux[pi];
@@ -568,9 +575,8 @@ cudaError_t launch_gather_cols(const SmallBatch& b, cudaStream_t s, int64_t* lau
     if (b.count <= 0) return cudaSuccess;
     int lmax = 1;
     for (int q = 0; q < b.count; ++q) lmax = std::max(lmax, b.l[q]);
-    k_gather_cols<<<dim3(std::min(1024, lmax), b.count), 256, 0, s>>>(b);
     ++*launches;
-    return cudaGetLastError();
+    return launch(k_gather_cols, dim3(std::min(1024, lmax), b.count), 256, 0, s, 1, b);
 }
 
 // ---------------------------------------------------------------------------
@@ -588,6 +594,7 @@ cudaError_t launch_gather_cols(const SmallBatch& b, cudaStream_t s, int64_t* lau
 constexpr int kSignCtas = 8;
 
 __global__ void __launch_bounds__(256) k_sign_fix_store(const __grid_constant__ SmallBatch b) {
+    pdl_begin();
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ float s_best[8][32];
@@ -670,19 +677,8 @@ cudaError_t launch_sign_fix_store(const SmallBatch& b, cudaStream_t s, int64_t* 
     if (b.count <= 0) return cudaSuccess;
     int rmax = 1;
     for (int q = 0; q < b.count; ++q) rmax = std::max(rmax, b.l[q]);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((rmax + 31) / 32 * kSignCtas, b.count);
-    cfg.blockDim = dim3(256);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kSignCtas;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
     ++*launches;
-    return cudaLaunchKernelEx(&cfg, k_sign_fix_store, b);
+    return launch(k_sign_fix_store, dim3((rmax + 31) / 32 * kSignCtas, b.count), 256, 0, s, kSignCtas, b);
 }
 
 }  // namespace moara

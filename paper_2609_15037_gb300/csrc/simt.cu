@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "launch.cuh"
 
 namespace moara {
 
@@ -56,6 +57,7 @@ __device__ __forceinline__ void finish_item(const DecompBatch& b, const DecompIt
 
 // One thread per (row, block): used for B <= 32.
 __global__ void __launch_bounds__(256) k_decompose_thread(const __grid_constant__ DecompBatch b) {
+    pdl_begin();
     const long long total = b.item_start[b.count];
     for (long long item = blockIdx.x * (long long)blockDim.x + threadIdx.x; item < total;
          item += (long long)gridDim.x * blockDim.x) {
@@ -79,6 +81,7 @@ __global__ void __launch_bounds__(256) k_decompose_thread(const __grid_constant_
 
 // One warp per (row, block): used for B > 32.
 __global__ void __launch_bounds__(256) k_decompose_warp(const __grid_constant__ DecompBatch b) {
+    pdl_begin();
     const long long total = b.item_start[b.count];
     const int lane = threadIdx.x & 31;
     const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
@@ -111,14 +114,14 @@ cudaError_t launch_decompose(const DecompBatch& b, cudaStream_t s, int64_t* laun
     if (b.B > 32) {
         long long blocks = (total * 32 + threads - 1) / threads;
         if (blocks > 152LL * 64) blocks = 152LL * 64;
-        k_decompose_warp<<<static_cast<unsigned>(blocks), threads, 0, s>>>(b);
+        ++*launches;
+        return launch(k_decompose_warp, static_cast<unsigned>(blocks), threads, 0, s, 1, b);
     } else {
         long long blocks = (total + threads - 1) / threads;
         if (blocks > 152LL * 64) blocks = 152LL * 64;
-        k_decompose_thread<<<static_cast<unsigned>(blocks), threads, 0, s>>>(b);
+        ++*launches;
+        return launch(k_decompose_thread, static_cast<unsigned>(blocks), threads, 0, s, 1, b);
     }
-    ++*launches;
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -223,6 +226,7 @@ __device__ __forceinline__ void epilogue(const GemmBatchT<CAP>& b, const GemmPro
 
 template <int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
 __global__ void __launch_bounds__(256, 2) k_gemm(const __grid_constant__ GemmBatch b) {
+    pdl_begin();
     __shared__ __align__(16) float As[2][TK][TM + TPAD];
     __shared__ __align__(16) float Bs[2][TK][TN + TPAD];
 
@@ -386,6 +390,7 @@ struct SliceLoader {
 
 template <int CAP, int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
 __global__ void __launch_bounds__(256, 4) k_gemm_small(const __grid_constant__ GemmBatchT<CAP> b) {
+    pdl_begin();
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ __align__(16) float As[2][SM_K][SM_LD];
@@ -477,20 +482,9 @@ static int k_split(const GemmProb& p) {
 
 template <int CAP, int ALAY, bool ASC, bool ABF, int BLAY, bool BSC, bool BBF, int EPI>
 static cudaError_t launch_small(const GemmBatch& b, int total, int split, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(total * split);
-    cfg.blockDim = dim3(256);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = split;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
     auto fn = k_gemm_small<CAP, ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>;
     if constexpr (CAP == kMaxGroup) {
-        return cudaLaunchKernelEx(&cfg, fn, b);
+        return launch(fn, total * split, 256, 0, s, split, b);
     } else {
         GemmBatchT<CAP> f;
         f.count = b.count; f.B = b.B; f.log2B = b.log2B;
@@ -503,7 +497,7 @@ static cudaError_t launch_small(const GemmBatch& b, int total, int split, cudaSt
             f.p[i] = b.p[i];
         }
         f.tile_start[b.count] = b.tile_start[b.count];
-        return cudaLaunchKernelEx(&cfg, fn, f);
+        return launch(fn, total * split, 256, 0, s, split, f);
     }
 }
 
@@ -530,8 +524,7 @@ static cudaError_t launch_part(GemmBatch& b, cudaStream_t s, int64_t* launches) 
     if (split == 1 && total >= kWideTiles) {
         // enough 128 x 128 tiles for every SM: half the shared-memory reads
         // per FMA of the small kernel
-        k_gemm<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI><<<total, 256, 0, s>>>(b);
-        return cudaGetLastError();
+        return launch(k_gemm<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>, total, 256, 0, s, 1, b);
     }
     total = enumerate(SM_T, SM_T);
     if (b.count <= kFewGroup)

@@ -29,6 +29,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "launch.cuh"
 #include "tc.h"
 #include "tc_ptx.cuh"
 
@@ -234,6 +235,7 @@ __device__ __forceinline__ float mag_adam(const K0Params& p, float mag, float ol
 // from 81.5 to 75.8 us.
 template <int BLK, bool ADAM>
 __global__ void __launch_bounds__(256, 3) k0_decompose(const __grid_constant__ K0Params p) {
+    pdl_begin();
     constexpr int LPB = BLK / 8;                       // lanes per block (1..16)
     constexpr int SUBB = 256 / BLK;                    // blocks of a sub-segment
     static_assert(!ADAM || 4 * SUBB <= 32, "a lane per block of the item");
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(256, 3) k0_decompose(const __grid_constant__ K
 // for blocks below 32 columns, and where the clipping coefficient needs every
 // norm first.
 __global__ void __launch_bounds__(256) k0_mag_adam(const __grid_constant__ K0Params p) {
+    pdl_begin();
     const long long total = p.mstart[p.count];
     // a clipped gradient c G has block norms c M and the same direction V
     const float cf = p.clip != nullptr ? *p.clip : 1.0f;
@@ -439,6 +442,7 @@ k1_project(const __grid_constant__ K1Params p) {
     ptx::tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
     const int t_begin = p.cta_start[cluster], t_end = p.cta_start[cluster + 1];
+    pdl_begin();
 
     if (warp == 0) {
         // ------------------------------------------------------ TMA producer
@@ -812,6 +816,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
     ptx::tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
     const int t_begin = p.cta_start[cluster], t_end = p.cta_start[cluster + 1];
+    pdl_begin();
 
     if (warp == 0) {
         // ------------------------------------------------ operand TMA producer
@@ -1307,6 +1312,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
+    pdl_begin();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -1535,6 +1541,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) ks_product(const __grid_constan
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
+    pdl_begin();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -1996,6 +2003,15 @@ static TcState::Tiles* tc_tiles(TcState* st, const std::vector<int>& ids) {
     return &(st->tiles[ids] = t);
 }
 
+// The decomposition without Optimizer_M for block size B.
+static auto k0_plain(int B) {
+    return B == 8    ? k0_decompose<8, false>
+           : B == 16 ? k0_decompose<16, false>
+           : B == 32 ? k0_decompose<32, false>
+           : B == 64 ? k0_decompose<64, false>
+                     : k0_decompose<128, false>;
+}
+
 // K0 and Optimizer_M of one module part.  `background`: a grid of short
 // CTAs (about four row segments per warp) that fills the room K1 / K2 leave
 // on each SM instead of a persistent grid that would hold SMs they need.
@@ -2008,41 +2024,37 @@ static cudaError_t launch_k0(TcState* st, const K0Params& p0, bool background, c
     const int g0 = background ? static_cast<int>(std::max<long long>(1, std::min<long long>((items + 31) / 32, 1 << 30)))
                               : st->sms * 3;
     bool pass = mag_adam;                              // Optimizer_M as a pass of its own
+    cudaError_t e = cudaSuccess;
     if constexpr (BLK >= 32) {
-        if (mag_adam) k0_decompose<BLK, true><<<g0, 256, 0, s>>>(p0);
+        if (mag_adam) e = launch_if(!background, k0_decompose<BLK, true>, g0, 256, 0, s, 1, p0);
         pass = false;
     }
-    if (BLK < 32 || !mag_adam) k0_decompose<BLK, false><<<g0, 256, 0, s>>>(p0);
-    if (pass) k0_mag_adam<<<background ? st->sms : st->sms * 4, 256, 0, s>>>(p0);
+    if (BLK < 32 || !mag_adam) e = launch_if(!background, k0_decompose<BLK, false>, g0, 256, 0, s, 1, p0);
+    if (pass && e == cudaSuccess) e = launch_if(!background, k0_mag_adam, background ? st->sms : st->sms * 4, 256, 0, s, 1, p0);
     if (prof.on) prof.mark(prof.ctx, phase, s, false);
     *launches += pass ? 2 : 1;
-    return cudaGetLastError();
+    return e;
 }
 
-// which: 1 = K1 only, 2 = K2 only, 3 = both
+// which: 1 = K1, 2 = K2, 4 = K1 directly behind its decomposition on the stream
 template <int BLK, bool SB>
 static cudaError_t launch_k12(TcState* st, const K1Params& p1, const K2Params& p2, int g1, int g2, bool hilo,
                               cudaStream_t s, int64_t* launches, const TcProfile& prof, int which, bool rt) {
     cudaError_t e;
     if (which & 1) {
         if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_PROJECT, s, true);
-        if (rt) {
-            if (hilo) k1_project<true, SB, true><<<2 * g1, K1_THREADS, K1_SMEM, s>>>(p1);
-            else k1_project<false, SB, true><<<2 * g1, K1_THREADS, K1_SMEM, s>>>(p1);
-        } else {
-            if (hilo) k1_project<true, SB, false><<<2 * g1, K1_THREADS, K1_SMEM, s>>>(p1);
-            else k1_project<false, SB, false><<<2 * g1, K1_THREADS, K1_SMEM, s>>>(p1);
-        }
+        auto fn = rt ? (hilo ? k1_project<true, SB, true> : k1_project<false, SB, true>)
+                     : (hilo ? k1_project<true, SB, false> : k1_project<false, SB, false>);
+        // of several parts, K1 waits for its part's decomposition on the other stream
+        e = launch_if((which & 4) != 0 && !prof.on, fn, 2 * g1, K1_THREADS, K1_SMEM, s, 1, p1);
         if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_PROJECT, s, false);
-        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         ++*launches;
     }
     if (!(which & 2)) return cudaSuccess;
     if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_BACKPROJECT, s, true);
-    k2_backproject<BLK, SB><<<2 * g2, K2_THREADS, K2_SMEM, s>>>(p2);
+    e = launch_if(!prof.on, k2_backproject<BLK, SB>, 2 * g2, K2_THREADS, K2_SMEM, s, 1, p2);
     if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_BACKPROJECT, s, false);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     ++*launches;
     return cudaSuccess;
@@ -2061,7 +2073,7 @@ static cudaError_t launch_k0_any(int B, TcState* st, const K0Params& p0, bool ba
 
 static cudaError_t launch_k12_any(int B, bool sb, TcState* st, const K1Params& p1, const K2Params& p2, int g1,
                                   int g2, bool hilo, cudaStream_t s, int64_t* launches, const TcProfile& prof,
-                                  int which = 3, bool rt = false) {
+                                  int which, bool rt = false) {
     if (sb) {   // bf16 states: B >= 32 (tc_supported)
         switch (B) {
             case 32: return launch_k12<32, true>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
@@ -2212,7 +2224,7 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
             // left a gap after each K1 and was slower.)
             const bool bg = dec && q + 1 < np;
             if (bg && cudaEventRecord(st->ev_k1[q], s) != cudaSuccess) return fail("part event");
-            cudaError_t e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->g2, hilo, s, launches, prof, 1, rt);
+            cudaError_t e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->g2, hilo, s, launches, prof, np == 1 ? 5 : 1, rt);
             if (e != cudaSuccess) {
                 st->err = cudaGetErrorString(e);
                 return MOARA_ERR_CUDA;
@@ -2330,8 +2342,7 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
             auto fn = a_kmajor ? (with_lo == 0 ? kr_product<true, 0> : with_lo == 1 ? kr_product<true, 1> : kr_product<true, 2>)
                                : (with_lo == 0 ? kr_product<false, 0>
                                                : with_lo == 1 ? kr_product<false, 1> : kr_product<false, 2>);
-            fn<<<total, KR_THREADS, KR_SMEM, s>>>(kp);
-            const cudaError_t e = cudaGetLastError();
+            const cudaError_t e = launch(fn, total, KR_THREADS, KR_SMEM, s, 1, kp);
             if (e != cudaSuccess) {
                 st->err = cudaGetErrorString(e);
                 return MOARA_ERR_CUDA;
@@ -2417,15 +2428,9 @@ int tc_alignment(TcState* st, const moara_hparams& hp, int n_mod, const int* ids
             acc_items += static_cast<long long>(md.m) * segs;
         }
         p0.start[cnt] = acc_items;
-        switch (B) {
-            case 8: k0_decompose<8, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            case 16: k0_decompose<16, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            case 32: k0_decompose<32, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            case 64: k0_decompose<64, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            default: k0_decompose<128, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-        }
+        const cudaError_t e = launch(k0_plain(B), st->sms * 3, 256, 0, s, 1, p0);
         ++*launches;
-        if (cudaGetLastError() != cudaSuccess) {
+        if (e != cudaSuccess) {
             st->err = "alignment decomposition launch failed";
             return MOARA_ERR_CUDA;
         }
@@ -2463,16 +2468,14 @@ int tc_alignment(TcState* st, const moara_hparams& hp, int n_mod, const int* ids
         p2.mods = st->d_mods; p2.maps = st->d_maps; p2.status = st->d_status;
         p2.acc = acc + 3 * (size_t)c0;
         for (int q = 0; q < cnt; ++q) p2.G[q] = static_cast<const uint16_t*>(G[c0 + q]);
-        const int g2 = 2 * tl->g2;
-        switch (B) {
-            case 8: k2_backproject<8, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
-            case 16: k2_backproject<16, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
-            case 32: k2_backproject<32, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
-            case 64: k2_backproject<64, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
-            default: k2_backproject<128, false, true><<<g2, K2_THREADS, K2_SMEM, s>>>(p2); break;
-        }
+        auto fn = B == 8    ? k2_backproject<8, false, true>
+                  : B == 16 ? k2_backproject<16, false, true>
+                  : B == 32 ? k2_backproject<32, false, true>
+                  : B == 64 ? k2_backproject<64, false, true>
+                            : k2_backproject<128, false, true>;
+        const cudaError_t e = launch(fn, 2 * tl->g2, K2_THREADS, K2_SMEM, s, 1, p2);
         ++*launches;
-        if (cudaGetLastError() != cudaSuccess) {
+        if (e != cudaSuccess) {
             st->err = "alignment product launch failed";
             return MOARA_ERR_CUDA;
         }
@@ -2506,15 +2509,11 @@ int tc_split_v(TcState* st, const TcSplitItem* items, int count, int B, float de
             acc += static_cast<long long>(x.m) * segs;
         }
         p0.start[cnt] = acc;
-        switch (B) {
-            case 8: k0_decompose<8, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            case 16: k0_decompose<16, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            case 32: k0_decompose<32, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            case 64: k0_decompose<64, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            case 128: k0_decompose<128, false><<<st->sms * 3, 256, 0, s>>>(p0); break;
-            default: st->err = "block size not supported on the tensor-core path"; return MOARA_ERR_UNSUPPORTED;
+        if (!(B == 8 || B == 16 || B == 32 || B == 64 || B == 128)) {
+            st->err = "block size not supported on the tensor-core path";
+            return MOARA_ERR_UNSUPPORTED;
         }
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch(k0_plain(B), st->sms * 3, 256, 0, s, 1, p0);
         if (e != cudaSuccess) {
             st->err = cudaGetErrorString(e);
             return MOARA_ERR_CUDA;
@@ -2578,9 +2577,7 @@ int tc_gemm_split3(TcState* st, const TcSplitGemmItem* items, int count, int pla
         kp.status = st->d_status;
         kp.wait_limit = st->wait_limit;
         if (total == 0) continue;
-        if (planes == 3) ks_product<3><<<total, KR_THREADS, KS_SMEM, s>>>(kp);
-        else ks_product<2><<<total, KR_THREADS, KS_SMEM, s>>>(kp);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch(planes == 3 ? ks_product<3> : ks_product<2>, total, KR_THREADS, KS_SMEM, s, 1, kp);
         if (e != cudaSuccess) {
             st->err = cudaGetErrorString(e);
             return MOARA_ERR_CUDA;
