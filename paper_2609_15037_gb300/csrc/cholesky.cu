@@ -67,7 +67,8 @@ __host__ __device__ inline CholTiles chol_tiles(int l, int s) {
     if (s < 0 || s >= nb) return t;
     t.slab = imax(0, nb - (s + 2));
     t.islab = s - s / kTriSuper * kTriSuper;
-    t.zero = (l + ZCOLS - 1) / ZCOLS;
+    // nothing to clear in the last row block of a matrix of one superblock
+    t.zero = s == nb - 1 && s < kTriSuper ? 0 : (l + ZCOLS - 1) / ZCOLS;
     if (s >= 1) {
         const int q = (nb - (s + 1) + 1) / 2;          // pairs of blocks from s + 1 on
         t.bulk = q > 0 ? q * (q + 1) / 2 : 0;
@@ -802,6 +803,7 @@ cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches) {
         }
         b.tile_start[b.count] = total;
         b.step = step;
+        if (total == 0 && step == nbmax - 1) break;           // no module has anything left
         const int C = b.count <= kCritModules ? kCritCtas : 1;
         ++*launches;
         const cudaError_t e = launch(k_chol_step, dim3(C * b.count + (total + C - 1) / C * C), NT, CHOL_SMEM, s, C, b);

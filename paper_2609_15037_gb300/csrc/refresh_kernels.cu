@@ -412,8 +412,8 @@ __global__ void __launch_bounds__(kJacThreads) k_lead_jacobi(const __grid_consta
     pdl_begin();
     __shared__ float H[kLeadW][kLeadW + 1];
     __shared__ float J[kLeadW][kLeadW + 1];
-    __shared__ float rc[kJacPairs], rs_[kJacPairs];
-    __shared__ int rp[kJacPairs], rq[kJacPairs];
+    __shared__ float rc[2][kJacPairs], rs_[2][kJacPairs];     // rotations of this round and the last one
+    __shared__ int rp[2][kJacPairs], rq[2][kJacPairs];
     __shared__ float red[33];
     const int pi = blockIdx.x;
     const int l = b.l[pi];
@@ -442,6 +442,20 @@ __global__ void __launch_bounds__(kJacThreads) k_lead_jacobi(const __grid_consta
     __syncthreads();
     const int npairs = wp / 2;
     const int lane = t & 31, warp = t >> 5;
+    constexpr int WARPS = kJacThreads / 32;
+    // J <- J G for the rotations in buffer k, rows dealt to warps first, first + 1, ..
+    auto turn_j = [&](int k, int first) {
+        if (lane >= npairs || rq[k][lane] >= w) return;
+        const int p2 = rp[k][lane], q2 = rq[k][lane];
+        const float c2 = rc[k][lane], s2 = rs_[k][lane];
+#pragma unroll 4
+        for (int row = warp - first; row < w; row += WARPS - first) {
+            const float jp = J[row][p2], jq = J[row][q2];
+            J[row][p2] = c2 * jp - s2 * jq;
+            J[row][q2] = s2 * jp + c2 * jq;
+        }
+    };
+    int done = 0;                                  // rounds so far; J is one behind
     for (int sweep = 0; sweep < 20; ++sweep) {
         // stop once the off-diagonal mass is below fp32 resolution of the diagonal
         float off = 0.0f, dia = 0.0f;
@@ -453,59 +467,71 @@ __global__ void __launch_bounds__(kJacThreads) k_lead_jacobi(const __grid_consta
         off = block_sum(off, red);
         dia = block_sum(dia, red);
         if (!(off > 1e-14f * dia)) break;          // also ends on a non-finite H
-        for (int round = 0; round < wp - 1; ++round) {
-            if (t < npairs) {
-                // tournament: player 0 fixed, the others rotate by one each round
-                auto player = [&](int pos) {
-                    int k = pos - 1 + round;
-                    if (k >= wp - 1) k -= wp - 1;
-                    return pos == 0 ? 0 : 1 + k;
-                };
-                int p = player(t), q = player(wp - 1 - t);
-                if (p > q) { const int x = p; p = q; q = x; }
-                float c = 1.0f, sn = 0.0f;
-                if (q < w) {
-                    const float hpq = H[p][q];
-                    if (fabsf(hpq) > 1e-30f) {
-                        const float tau = (H[q][q] - H[p][p]) / (2.0f * hpq);
-                        const float tt = (tau >= 0.0f ? 1.0f : -1.0f) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
-                        c = 1.0f / sqrtf(1.0f + tt * tt);
-                        sn = tt * c;
+        for (int round = 0; round < wp - 1; ++round, ++done) {
+            const int k = done & 1;
+            if (warp == 0) {
+                if (t < npairs) {
+                    // tournament: player 0 fixed, the others rotate by one each round
+                    auto player = [&](int pos) {
+                        int x = pos - 1 + round;
+                        if (x >= wp - 1) x -= wp - 1;
+                        return pos == 0 ? 0 : 1 + x;
+                    };
+                    int p = player(t), q = player(wp - 1 - t);
+                    if (p > q) { const int x = p; p = q; q = x; }
+                    float c = 1.0f, sn = 0.0f;
+                    if (q < w) {
+                        const float hpq = H[p][q];
+                        if (fabsf(hpq) > 1e-30f) {
+                            // the angle to a few ulp (approximate division and
+                            // square root), the rotation orthonormal to
+                            // rounding: c from the tangent that sn uses, by
+                            // rsqrtf and one step of Newton's iteration
+                            const float tau = __fdividef(H[q][q] - H[p][p], 2.0f * hpq);
+                            const float at = fabsf(tau);
+                            // |tau| past 1e15: tan = 1 / (2 tau), below it (tau^2 does not overflow)
+                            const float tt = copysignf(at < 1e15f ? __fdividef(1.0f, at + __fsqrt_rn(fmaf(tau, tau, 1.0f)))
+                                                                  : __fdividef(0.5f, at), tau);
+                            const float d = fmaf(tt, tt, 1.0f);
+                            const float r = rsqrtf(d);
+                            c = fmaf(0.5f * r, fmaf(-d * r, r, 1.0f), r);
+                            sn = tt * c;
+                        }
                     }
+                    rp[k][t] = p; rq[k][t] = q; rc[k][t] = c; rs_[k][t] = sn;
                 }
-                rp[t] = p; rq[t] = q; rc[t] = c; rs_[t] = sn;
+            } else if (done > 0) {
+                turn_j(k ^ 1, 1);
             }
             __syncthreads();
             // H <- G^T H G by 2 x 2 blocks: the block of pairs (k1, k2) is read
-            // and written by one thread (lane = k2, a warp takes two k1); the
-            // columns of J turn by G as well
+            // and written by one thread (lane = k2, a warp takes two k1)
             if (lane < npairs) {
-                const int p2 = rp[lane], q2 = rq[lane];
-                const float c2 = rc[lane], s2 = rs_[lane];
+                const int p2 = rp[k][lane], q2 = rq[k][lane];
+                const float c2 = rc[k][lane], s2 = rs_[k][lane];
                 const bool two = q2 < w;
-                for (int k1 = warp; k1 < npairs; k1 += kJacThreads / 32) {
-                    const int p1 = rp[k1], q1 = rq[k1];
-                    const float c1 = rc[k1], s1 = rs_[k1];
+#pragma unroll
+                for (int u = 0; u < kJacPairs / WARPS; ++u) {
+                    const int k1 = warp + u * WARPS;
+                    if (k1 >= npairs) break;
+                    const int p1 = rp[k][k1], q1 = rq[k][k1];
+                    const float c1 = rc[k][k1], s1 = rs_[k][k1];
                     const float a = H[p1][p2], d = q1 < w && two ? H[q1][q2] : 0.0f;
-                    const float u = two ? H[p1][q2] : 0.0f, v = q1 < w ? H[q1][p2] : 0.0f;
+                    const float h = two ? H[p1][q2] : 0.0f, v = q1 < w ? H[q1][p2] : 0.0f;
                     // columns, then rows
-                    const float a1 = c2 * a - s2 * u, u1 = s2 * a + c2 * u;
+                    const float a1 = c2 * a - s2 * h, u1 = s2 * a + c2 * h;
                     const float v1 = c2 * v - s2 * d, d1 = s2 * v + c2 * d;
                     H[p1][p2] = c1 * a1 - s1 * v1;
                     if (two) H[p1][q2] = c1 * u1 - s1 * d1;
                     if (q1 < w) H[q1][p2] = s1 * a1 + c1 * v1;
                     if (two && q1 < w) H[q1][q2] = s1 * u1 + c1 * d1;
                 }
-                if (two)
-                    for (int row = warp; row < w; row += kJacThreads / 32) {
-                        const float jp = J[row][p2], jq = J[row][q2];
-                        J[row][p2] = c2 * jp - s2 * jq;
-                        J[row][q2] = s2 * jp + c2 * jq;
-                    }
             }
             __syncthreads();
         }
     }
+    if (done > 0) turn_j((done - 1) & 1, 0);
+    __syncthreads();
     for (int e = t; e < w * w; e += kJacThreads) part[e] = J[e / w][e % w];
 }
 
