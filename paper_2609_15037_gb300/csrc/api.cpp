@@ -523,12 +523,14 @@ struct RefreshRunner {
 
     // out = A B (l x l) from three-plane operands (A stored K x M, B K x N)
     void ks_gemm(const std::vector<uint16_t*>& A, const std::vector<uint16_t*>& B, const std::vector<float*>& out,
-                 int ktri, int planes) {
+                 int ktri, int planes, int lower = 0) {
         std::vector<moara::TcSplitGemmItem> g;
         for (size_t i = 0; i < it.size(); ++i) {
             const int l = it[i].l;
             const size_t pl = (size_t)l * l;
-            g.push_back({A[i], B[i], pl, pl, out[i], l, l, l, ktri});
+            moara::TcSplitGemmItem item{A[i], B[i], pl, pl, out[i], l, l, l, ktri};
+            item.lower = lower;
+            g.push_back(item);
         }
         ks_run(g, planes);
     }
@@ -553,7 +555,9 @@ struct RefreshRunner {
         for (size_t i = 0; i < n_it; ++i) {
             const int l = it[i].l;
             const size_t pm = (size_t)rows[i] * l;
-            g.push_back({pl[i], pl[i], pm, pm, it[i].Cg, l, l, rows[i], 0});
+            moara::TcSplitGemmItem item{pl[i], pl[i], pm, pm, it[i].Cg, l, l, rows[i], 0};
+            item.lower = 1;                 // the Cholesky reads the lower triangle only
+            g.push_back(item);
         }
         ks_run(g, planes);                  // Gram X^T X
         cholesky(rows, shift_rel);
@@ -581,7 +585,7 @@ struct RefreshRunner {
         std::vector<float*> cg(it.size());
         for (size_t i = 0; i < it.size(); ++i) cg[i] = it[i].Cg;
         split3(Win, p1, 0);                 // W (as A = W^T, MN-major, and as B)
-        ks_gemm(p1, p1, cg, 0, planes);     // Gram W^T W
+        ks_gemm(p1, p1, cg, 0, planes, 1);  // Gram W^T W (the lower triangle)
         cholesky(rows_l, shift_rel);
         tri_inverse();
         std::vector<float*> linv(it.size());

@@ -182,13 +182,100 @@ cudaError_t launch_transpose_bf16(const SmallBatch& b, cudaStream_t s, int64_t* 
 // Three bf16 planes of an fp32 matrix (rows x l, row-major, row pitch ld or
 // l): hi = bf16(x), mid = bf16(x - hi), lo = bf16(x - hi - mid), so
 // hi + mid + lo carries 24 significant bits.  With `transpose` the planes hold the l x rows transpose.
-// Planes are consecutive at h, each rows * l elements.  32 x 32 tiles through
-// shared memory keep both sides coalesced.
+// Planes are consecutive at h, each rows * l elements.  Bound by HBM / L2
+// bytes (4 read, 6 written per entry): 64 x 64 tiles, 16-byte loads and
+// stores, through shared memory for the transpose (as 32 x 32 tiles with
+// 4-byte stores on a 256-CTA grid per matrix, 45 M entries took 167 us, now
+// 63 us = 7.1 TB/s); 32 x 32 tiles where a pitch or an address is not a
+// multiple of 16 bytes.
 // ---------------------------------------------------------------------------
+// the three bf16 parts of eight values, as 16-byte units
+__device__ __forceinline__ void split8(const float (&x)[8], uint4 (&p)[3]) {
+    uint32_t w[3][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float a = x[2 * k], b = x[2 * k + 1];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+            w[q][k] = *reinterpret_cast<const uint32_t*>(&h);
+            a -= __low2float(h);
+            b -= __high2float(h);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) p[q] = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+}
+
+// Whether both kernels' 16-byte accesses are aligned for item pi.
+__device__ __forceinline__ bool split_wide(const SmallBatch& b, int pi) {
+    const int lds = b.ld[pi] > 0 ? b.ld[pi] : b.l[pi];
+    return ((b.rows[pi] | b.l[pi]) & 7) == 0 && (lds & 3) == 0 &&
+           ((reinterpret_cast<uintptr_t>(b.a[pi]) | reinterpret_cast<uintptr_t>(b.h[pi])) & 15) == 0;
+}
+
+__global__ void __launch_bounds__(256) k_split3_wide(const __grid_constant__ SmallBatch b, int transpose) {
+    pdl_begin();
+    __shared__ float t[64][65];
+    const int pi = blockIdx.z;
+    if (!split_wide(b, pi)) return;
+    const int rows = b.rows[pi], cols = b.l[pi];
+    const long long lds = b.ld[pi] > 0 ? b.ld[pi] : cols;
+    const float* src = b.a[pi];
+    uint16_t* dst = b.h[pi];
+    const long long plane = (long long)rows * cols;
+    const int tr = (rows + 63) / 64, tc = (cols + 63) / 64;
+    const int tid = threadIdx.x;
+    for (int tile = blockIdx.x; tile < tr * tc; tile += gridDim.x) {
+        const int i0 = tile / tc * 64, j0 = (tile - tile / tc * tc) * 64;
+        if (!transpose) {
+            // thread: rows tid / 8 and 32 further, eight columns
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int i = i0 + (tid >> 3) + 32 * u, j = j0 + 8 * (tid & 7);
+                if (i >= rows || j >= cols) continue;
+                const float4* s4 = reinterpret_cast<const float4*>(src + i * lds + j);
+                const float4 v = s4[0], w = s4[1];
+                const float x[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
+                uint4 p[3];
+                split8(x, p);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4*>(dst + q * plane + (long long)i * cols + j) = p[q];
+            }
+            continue;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = (tid >> 4) + 16 * u, c = 4 * (tid & 15);
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (i0 + r < rows && j0 + c < cols) v = *reinterpret_cast<const float4*>(src + (i0 + r) * lds + j0 + c);
+            t[r][c] = v.x; t[r][c + 1] = v.y; t[r][c + 2] = v.z; t[r][c + 3] = v.w;
+        }
+        __syncthreads();
+        // output row j0 + (tid / 8) and 32 further, eight columns of it
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = (tid >> 3) + 32 * u, r = 8 * (tid & 7);
+            if (j0 + c < cols && i0 + r < rows) {
+                float x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) x[k] = t[r + k][c];
+                uint4 p[3];
+                split8(x, p);
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    *reinterpret_cast<uint4*>(dst + q * plane + (long long)(j0 + c) * rows + i0 + r) = p[q];
+            }
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void __launch_bounds__(256) k_split3(const __grid_constant__ SmallBatch b, int transpose) {
     pdl_begin();
     __shared__ float t[32][33];
     const int pi = blockIdx.z;
+    if (split_wide(b, pi)) return;
     const int rows = b.rows[pi], cols = b.l[pi];
     const long long lds = b.ld[pi] > 0 ? b.ld[pi] : cols;
     const float* src = b.a[pi];
@@ -253,12 +340,26 @@ __global__ void __launch_bounds__(256) k_split3(const __grid_constant__ SmallBat
 
 cudaError_t launch_split3(const SmallBatch& b, int transpose, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    // as many blocks per item as the largest item has 32 x 32 tiles (at most 256)
-    long long tiles = 1;
-    for (int q = 0; q < b.count; ++q)
-        tiles = std::max(tiles, (long long)((b.rows[q] + 31) / 32) * ((b.l[q] + 31) / 32));
-    ++*launches;
-    return launch(k_split3, dim3(static_cast<unsigned>(std::min(256LL, tiles)), 1, b.count), 256, 0, s, 1, b, transpose);
+    // as many blocks per item as the largest item has tiles
+    long long wide = 0, narrow = 0;
+    for (int q = 0; q < b.count; ++q) {
+        const int lds = b.ld[q] > 0 ? b.ld[q] : b.l[q];
+        if (((b.rows[q] | b.l[q]) & 7) == 0 && (lds & 3) == 0 &&
+            ((reinterpret_cast<uintptr_t>(b.a[q]) | reinterpret_cast<uintptr_t>(b.h[q])) & 15) == 0)
+            wide = std::max(wide, (long long)((b.rows[q] + 63) / 64) * ((b.l[q] + 63) / 64));
+        else
+            narrow = std::max(narrow, (long long)((b.rows[q] + 31) / 32) * ((b.l[q] + 31) / 32));
+    }
+    cudaError_t e = cudaSuccess;
+    if (wide > 0) {
+        e = launch(k_split3_wide, dim3(static_cast<unsigned>(std::min(2048LL, wide)), 1, b.count), 256, 0, s, 1, b, transpose);
+        ++*launches;
+    }
+    if (narrow > 0 && e == cudaSuccess) {
+        e = launch(k_split3, dim3(static_cast<unsigned>(std::min(256LL, narrow)), 1, b.count), 256, 0, s, 1, b, transpose);
+        ++*launches;
+    }
+    return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -357,7 +458,7 @@ __global__ void __launch_bounds__(256) k_ritz_order(const __grid_constant__ Smal
 // Three launches: partial Gram blocks over slabs of rows, one CTA per module
 // for the Jacobi sweeps, and the rotation over slabs of rows.  As one CTA per
 // module the whole took 0.32 / 0.63 / 1.20 ms at l = 64 / 288 / 2080, now
-// 0.26 / 0.45 / 0.48 ms; what is left is the chain of the sweeps.  h: scratch of
+// 0.22 / 0.36 / 0.37 ms; what is left is the chain of the sweeps.  h: scratch of
 // l x l floats, the partial Gram blocks and then J.
 // ---------------------------------------------------------------------------
 constexpr int kLeadW = 64;

@@ -1462,8 +1462,9 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
 // bits); six MMAs per k-step (hi.hi, hi.mid, mid.hi, hi.lo, mid.mid, lo.hi)
 // leave out terms of relative size 2^-24 and below.  out (M x N, fp32) =
 // A B with A stored K x M and B stored K x N (both MN-major), tile 256 x 256
-// (two 128-row accumulators in TMEM), BK = 32, two stages of 96 KB; `ktri`
-// stops the K loop of column tile n0 at n0 + 256 (B upper triangular).
+// (two 128-row accumulators in TMEM) or 128 x 256, BK = 32, two stages of
+// 96 KB; `ktri` stops the K loop of column tile n0 at n0 + 256 (B upper
+// triangular).
 // ===========================================================================
 constexpr int KS_BM = 256, KS_BN = 256, KS_BK = 32;
 constexpr int KS_PLANE = KS_BM * KS_BK * 2;               // 16 KB: one plane of A (or B)
@@ -1491,6 +1492,7 @@ struct KsParams {
     int tiles_n[kKsGroup];
     int tile_start[kKsGroup + 1];
     int count;
+    int bm;                            // tile rows: 256 or 128
     int* status;
     long long wait_limit;              // clock cycles of a bounded wait before it gives up
 };
@@ -1515,11 +1517,11 @@ __global__ void __launch_bounds__(KR_THREADS, 1) ks_product(const __grid_constan
     const int pi = lo;
     const int local = tile - p.tile_start[pi];
     const int M = p.M[pi], N = p.N[pi], K = p.K[pi];
-    const int i0 = (local / p.tiles_n[pi]) * KS_BM;
+    const int i0 = (local / p.tiles_n[pi]) * p.bm;
     const int n0 = (local % p.tiles_n[pi]) * KS_BN;
-    if (p.lower[pi] && n0 >= i0 + KS_BM) return;     // whole CTA, before any barrier or TMEM
+    if (p.lower[pi] && n0 >= i0 + p.bm) return;      // whole CTA, before any barrier or TMEM
     const int nch = min(4, (N - n0 + 63) / 64);
-    const int halves = (M - i0) > 128 ? 2 : 1;
+    const int halves = p.bm > 128 && (M - i0) > 128 ? 2 : 1;
     const int kend = p.ktri[pi] ? min(K, n0 + KS_BN) : K;
     const int nk = (kend + KS_BK - 1) / KS_BK;
 
@@ -1548,7 +1550,8 @@ __global__ void __launch_bounds__(KR_THREADS, 1) ks_product(const __grid_constan
             int stage = 0;
             uint32_t phase = 0;
             uint32_t issued = 0, last_par = 0;
-            const uint32_t bytes = NP * KS_PLANE + NP * nch * 4096;
+            const int ach = p.bm / 64;                     // 64-row chunks of A
+            const uint32_t bytes = NP * (ach + nch) * 4096;
             for (int kb = 0; kb < nk; ++kb) {
                 if (!ptx::mbar_wait(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1, abort_flag, p.status,
                                     MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit))
@@ -1561,7 +1564,8 @@ __global__ void __launch_bounds__(KR_THREADS, 1) ks_product(const __grid_constan
                 for (int q = 0; q < NP; ++q) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        ptx::tma_load_2d(a + q * KS_PLANE + c * 4096, &p.amap[pi][q], fb, i0 + 64 * c, kb * KS_BK);
+                        if (c < ach)
+                            ptx::tma_load_2d(a + q * KS_PLANE + c * 4096, &p.amap[pi][q], fb, i0 + 64 * c, kb * KS_BK);
                     for (int c = 0; c < nch; ++c)
                         ptx::tma_load_2d(b + q * KS_PLANE + c * 4096, &p.bmap[pi][q], fb, n0 + 64 * c, kb * KS_BK);
                 }
@@ -1610,16 +1614,17 @@ __global__ void __launch_bounds__(KR_THREADS, 1) ks_product(const __grid_constan
     } else {
         const int ew = warp - 2;
         const int q = warp & 3;
-        const int h = ew >> 2;
+        // row half of the tile, or with one half every other 16-column chunk
+        const int h = halves == 2 ? ew >> 2 : 0, cfirst = halves == 2 ? 0 : ew >> 2, cstep = halves == 2 ? 1 : 2;
         const bool got = ptx::mbar_wait(ptx::smem_u32(&ctl->accf[0]), 0, abort_flag, p.status,
                                         MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit);
-        if (__all_sync(0xffffffffu, got) && h < halves) {
+        if (__all_sync(0xffffffffu, got)) {
             ptx::tc_fence_after();
             const int row = i0 + h * 128 + q * 32 + lane;
             float* const of = p.out[pi];
             const long long ro = (long long)row * p.ldo[pi];
             const bool sub = p.sub[pi] != 0;
-            for (int c = 0; c < nch * 4; ++c) {
+            for (int c = cfirst; c < nch * 4; c += cstep) {
                 const int j0 = n0 + c * 16;
                 if (j0 >= N) break;                       // warp-uniform
                 float v[16];
@@ -2546,13 +2551,35 @@ int tc_gemm_split3(TcState* st, const TcSplitGemmItem* items, int count, int pla
             return MOARA_ERR_UNSUPPORTED;
         }
     }
+    // longest K first, so that the last CTAs to start are short ones
+    std::vector<int> order(count);
+    for (int i = 0; i < count; ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return items[a].K > items[b].K; });
     for (int c0 = 0; c0 < count; c0 += kKsGroup) {
         const int cnt = std::min(kKsGroup, count - c0);
+        // Tiles of 128 rows where the longest 256-row tile (its K) lasts longer
+        // than all of them take on every SM: few tiles, or a tall Gram matrix
+        // among short ones.  A 128-row tile costs about 5/8 of a 256-row one
+        // (its operands are 3/4 of the bytes).  Seven tall three-plane Gram
+        // matrices (132 tiles, K up to 11008) take 418 us instead of 572, a group of
+        // l = 160 / 288 products 33 us instead of 48; 830 tiles 389 us with 128 rows,
+        // 357 with 256.
+        double longest = 0.0, total256 = 0.0, total128 = 0.0;
+        for (int q = 0; q < cnt; ++q) {
+            const TcSplitGemmItem& x = items[order[c0 + q]];
+            longest = std::max(longest, 1.0 * x.K);
+            for (int i0 = 0; i0 < x.M; i0 += 128) {
+                const int c128 = x.lower ? std::min(x.N, i0 + 128) : x.N;
+                total128 += 0.625 * x.K * ((c128 + KS_BN - 1) / KS_BN);
+                if (i0 % 256 == 0) total256 += 1.0 * x.K * (((x.lower ? std::min(x.N, i0 + 256) : x.N) + KS_BN - 1) / KS_BN);
+            }
+        }
+        const int bm = std::max(0.625 * longest, total128 / st->sms) < std::max(longest, total256 / st->sms) ? 128 : 256;
         KsParams& kp = st->ps;
         std::memset(&kp, 0, sizeof(kp));
         int total = 0;
         for (int q = 0; q < cnt; ++q) {
-            const TcSplitGemmItem& x = items[c0 + q];
+            const TcSplitGemmItem& x = items[order[c0 + q]];
             bool ok = true;
             for (int pl = 0; pl < 3; ++pl) {
                 ok = ok && encode_bf16_2d(st->encode, &kp.amap[q][pl], x.A + (size_t)pl * x.a_plane, x.M, x.K, 64, 32);
@@ -2570,10 +2597,11 @@ int tc_gemm_split3(TcState* st, const TcSplitGemmItem* items, int count, int pla
             kp.lower[q] = x.lower;
             kp.tiles_n[q] = (x.N + KS_BN - 1) / KS_BN;
             kp.tile_start[q] = total;
-            total += ((x.M + KS_BM - 1) / KS_BM) * kp.tiles_n[q];
+            total += ((x.M + bm - 1) / bm) * kp.tiles_n[q];
         }
         kp.tile_start[cnt] = total;
         kp.count = cnt;
+        kp.bm = bm;
         kp.status = st->d_status;
         kp.wait_limit = st->wait_limit;
         if (total == 0) continue;
