@@ -1265,6 +1265,50 @@ struct KrParams {
 
 static_assert(sizeof(KrParams) <= 32764, "KR's parameter block fits the kernel parameter space");
 
+// Columns j0 .. j0 + 15 of one output row (offset ro) in fp32, bf16 and / or as
+// a bf16 residual.
+__device__ __forceinline__ void kr_store16(float* of, uint16_t* ob, uint16_t* ol, long long ro, int j0, int N,
+                                           const float (&v)[16]) {
+    if (j0 + 16 <= N) {                       // N % 8 == 0: 16-byte aligned rows
+        if (of != nullptr) {
+            float4* o4 = reinterpret_cast<float4*>(of + ro + j0);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                o4[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+        }
+        if (ob != nullptr) {
+            uint4* b4 = reinterpret_cast<uint4*>(ob + ro + j0);
+            b4[0] = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]),
+                               pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+            b4[1] = make_uint4(pack_bf16x2(v[8], v[9]), pack_bf16x2(v[10], v[11]),
+                               pack_bf16x2(v[12], v[13]), pack_bf16x2(v[14], v[15]));
+        }
+        if (ol != nullptr) {
+            float rl[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+                rl[e] = v[e] - __bfloat162float(__float2bfloat16_rn(v[e]));
+            uint4* l4 = reinterpret_cast<uint4*>(ol + ro + j0);
+            l4[0] = make_uint4(pack_bf16x2(rl[0], rl[1]), pack_bf16x2(rl[2], rl[3]),
+                               pack_bf16x2(rl[4], rl[5]), pack_bf16x2(rl[6], rl[7]));
+            l4[1] = make_uint4(pack_bf16x2(rl[8], rl[9]), pack_bf16x2(rl[10], rl[11]),
+                               pack_bf16x2(rl[12], rl[13]), pack_bf16x2(rl[14], rl[15]));
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            if (j0 + e >= N) continue;
+            if (of != nullptr) of[ro + j0 + e] = v[e];
+            const __nv_bfloat16 hb = __float2bfloat16_rn(v[e]);
+            if (ob != nullptr) ob[ro + j0 + e] = *reinterpret_cast<const uint16_t*>(&hb);
+            if (ol != nullptr) {
+                const __nv_bfloat16 lb = __float2bfloat16_rn(v[e] - __bfloat162float(hb));
+                ol[ro + j0 + e] = *reinterpret_cast<const uint16_t*>(&lb);
+            }
+        }
+    }
+}
+
 // LO: 1 adds the MMA with A's residual plane, 2 with B's.
 template <bool KMAJOR, int LO>
 __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constant__ KrParams p) {
@@ -1405,45 +1449,7 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
                 float v[16];
                 __syncwarp();
                 ptx::tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + h * 256 + c * 16, v);
-                if (row >= M) continue;
-                if (j0 + 16 <= N) {                       // N % 8 == 0: 16-byte aligned rows
-                    if (of != nullptr) {
-                        float4* o4 = reinterpret_cast<float4*>(of + ro + j0);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            o4[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-                    }
-                    if (ob != nullptr) {
-                        uint4* b4 = reinterpret_cast<uint4*>(ob + ro + j0);
-                        b4[0] = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]),
-                                           pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
-                        b4[1] = make_uint4(pack_bf16x2(v[8], v[9]), pack_bf16x2(v[10], v[11]),
-                                           pack_bf16x2(v[12], v[13]), pack_bf16x2(v[14], v[15]));
-                    }
-                    if (ol != nullptr) {
-                        float rl[16];
-#pragma unroll
-                        for (int e = 0; e < 16; ++e)
-                            rl[e] = v[e] - __bfloat162float(__float2bfloat16_rn(v[e]));
-                        uint4* l4 = reinterpret_cast<uint4*>(ol + ro + j0);
-                        l4[0] = make_uint4(pack_bf16x2(rl[0], rl[1]), pack_bf16x2(rl[2], rl[3]),
-                                           pack_bf16x2(rl[4], rl[5]), pack_bf16x2(rl[6], rl[7]));
-                        l4[1] = make_uint4(pack_bf16x2(rl[8], rl[9]), pack_bf16x2(rl[10], rl[11]),
-                                           pack_bf16x2(rl[12], rl[13]), pack_bf16x2(rl[14], rl[15]));
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        if (j0 + e >= N) continue;
-                        if (of != nullptr) of[ro + j0 + e] = v[e];
-                        const __nv_bfloat16 hb = __float2bfloat16_rn(v[e]);
-                        if (ob != nullptr) ob[ro + j0 + e] = *reinterpret_cast<const uint16_t*>(&hb);
-                        if (ol != nullptr) {
-                            const __nv_bfloat16 lb = __float2bfloat16_rn(v[e] - __bfloat162float(hb));
-                            ol[ro + j0 + e] = *reinterpret_cast<const uint16_t*>(&lb);
-                        }
-                    }
-                }
+                if (row < M) kr_store16(of, ob, ol, ro, j0, N, v);
             }
         }
     }
@@ -1453,6 +1459,169 @@ __global__ void __launch_bounds__(KR_THREADS, 1) kr_product(const __grid_constan
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, 512);
+    }
+}
+
+// The same product on 2-CTA pairs: an output tile of 256 x 256 with 128 rows and
+// half of B's columns per CTA, so that a k-step takes half as long and each
+// operand is fetched once per pair.  For launches that one tile's K outlasts
+// (few tiles): 199 Gram tiles of seven modules (K up to 11008) take 81 us
+// instead of 110, the products of a 1024 / 2816 layer 25 and 14 instead of 40
+// and 21.
+// With more tiles than SMs the fixed costs per tile (barriers, TMEM, an
+// epilogue that overlaps no MMAs) weigh twice and the single CTA is as fast.
+template <int LO> struct KpCfg {
+    static constexpr int STAGE_BYTES = (LO ? 3 : 2) * (KR_PLANE / 2);
+    static constexpr int STAGES = 6 * KR_PLANE / STAGE_BYTES;
+};
+
+template <bool KMAJOR, int LO>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KR_THREADS, 1) kr_pair(const __grid_constant__ KrParams p) {
+    constexpr int STAGES = KpCfg<LO>::STAGES, STAGE_BYTES = KpCfg<LO>::STAGE_BYTES;
+    constexpr int PLANE = KR_PLANE / 2;                      // 128 rows of A, or 128 columns of B
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = align1024(smem_raw);
+    SmemCtl* ctl = reinterpret_cast<SmemCtl*>(smem + 6 * KR_PLANE);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int crank = static_cast<int>(ptx::cluster_ctarank());
+    volatile int* abort_flag = &ctl->abort;
+
+    const int tile = blockIdx.x >> 1;
+    int lo = 0, hi = p.count - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (p.tile_start[mid] <= tile) lo = mid; else hi = mid - 1;
+    }
+    const int pi = lo;
+    const int local = tile - p.tile_start[pi];
+    const int M = p.M[pi], N = p.N[pi], K = p.K[pi];
+    const int i0 = (local / p.tiles_n[pi]) * KR_BM;
+    const int n0 = (local % p.tiles_n[pi]) * KR_BN;
+    if (p.lower[pi] && n0 >= i0 + KR_BM) return;     // the whole pair, before any barrier or TMEM
+    const int r0 = i0 + 128 * crank;
+    const int nb = N - n0 > 128 ? 2 : 1;             // 64-column chunks of B per CTA
+    const int kend = p.ktri[pi] ? min(K, n0 + KR_BN) : K;
+    const int nk = (kend + KR_BK - 1) / KR_BK;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            ptx::mbar_init(ptx::smem_u32(&ctl->full[s]), 1);
+            ptx::mbar_init(ptx::smem_u32(&ctl->empty[s]), 1);
+        }
+        ptx::mbar_init(ptx::smem_u32(&ctl->accf[0]), 1);
+        ptx::mbar_init(ptx::smem_u32(&ctl->drain), 1);
+        ctl->abort = 0;
+        ptx::fence_barrier_init();
+    }
+    if (warp == 1) {                // collective: one warp of each CTA of the pair
+        ptx::tmem_alloc2(ptx::smem_u32(&ctl->tmem_base), 256);
+        ptx::tmem_relinquish2();
+    }
+    ptx::tc_fence_before();
+    __syncwarp();
+    ptx::cluster_sync();            // barriers of both CTAs initialised before any remote signal
+    ptx::tc_fence_after();
+    const uint32_t tmem = ctl->tmem_base;
+    pdl_begin();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            uint32_t issued = 0, last_par = 0;
+            bool ok = true;
+            const uint32_t bytes = (LO == 1 ? 2 : 1) * PLANE + (LO == 2 ? 2 : 1) * nb * 8192;
+            for (int kb = 0; kb < nk; ++kb) {
+                if (!ptx::mbar_wait(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1, abort_flag, p.status,
+                                    MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
+                const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
+                const uint32_t fb = ptx::mapa(own, 0);
+                if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * bytes);
+                const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
+                const uint32_t b = a + (LO == 1 ? 2 : 1) * PLANE;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const int x = KMAJOR ? kb * KR_BK : r0 + 64 * c;
+                    const int y = KMAJOR ? r0 + 64 * c : kb * KR_BK;
+                    ptx::tma_load_2d_pair(a + c * 8192, &p.amap[pi], fb, x, y);
+                    if (LO == 1) ptx::tma_load_2d_pair(a + PLANE + c * 8192, &p.lmap[pi], fb, x, y);
+                }
+                for (int c = 0; c < nb; ++c) {
+                    const int x = n0 + 64 * (nb * crank + c);
+                    ptx::tma_load_2d_pair(b + c * 8192, &p.bmap[pi], fb, x, kb * KR_BK);
+                    if (LO == 2) ptx::tma_load_2d_pair(b + PLANE + c * 8192, &p.lmap[pi], fb, x, kb * KR_BK);
+                }
+                issued |= 1u << stage;
+                last_par = (last_par & ~(1u << stage)) | (phase << stage);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+            if (!ok && crank == 0) {   // let the copies already in flight land before the CTA exits
+                for (int s = 0; s < STAGES; ++s)
+                    if (issued & (1u << s)) wait_drain(ptx::smem_u32(&ctl->full[s]), (last_par >> s) & 1);
+            }
+        }
+    } else if (warp == 1) {
+        if (crank == 0 && lane == 0) {
+            const uint32_t idesc = ptx::idesc_bf16(256, nb * 128, KMAJOR ? 0 : 1, 1);
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = 0; kb < nk; ++kb) {
+                if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag, p.status,
+                                            MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) break;
+                ptx::tc_fence_after();
+                const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
+                const uint32_t b = a + (LO == 1 ? 2 : 1) * PLANE;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint32_t ao = a + (KMAJOR ? kk * 32 : kk * 2048);
+                    const uint64_t adesc = KMAJOR ? ptx::smem_desc_sw128(ao, 16, 1024)
+                                                  : ptx::smem_desc_sw128(ao, 8192, 1024);
+                    const uint64_t bdesc = ptx::smem_desc_sw128(b + kk * 2048, 8192, 1024);
+                    ptx::mma2_f16(tmem, adesc, bdesc, idesc, (kb | kk) != 0);
+                    if (LO == 1) {
+                        const uint64_t ldesc = KMAJOR ? ptx::smem_desc_sw128(ao + PLANE, 16, 1024)
+                                                      : ptx::smem_desc_sw128(ao + PLANE, 8192, 1024);
+                        ptx::mma2_f16(tmem, ldesc, bdesc, idesc, 1);
+                    } else if (LO == 2) {
+                        ptx::mma2_f16(tmem, adesc, ptx::smem_desc_sw128(b + PLANE + kk * 2048, 8192, 1024), idesc, 1);
+                    }
+                }
+                ptx::mma2_commit_mc(ptx::smem_u32(&ctl->empty[stage]), 0x3);
+                if (++stage == STAGES) { stage = 0; phase ^= 1; }
+            }
+            ptx::mma2_commit_mc(ptx::smem_u32(&ctl->accf[0]), 0x3);
+            ptx::mma2_commit_mc(ptx::smem_u32(&ctl->drain), 0x1);
+            wait_drain(ptx::smem_u32(&ctl->drain), 0);
+        }
+    } else {
+        // 8 epilogue warps: lane quarter q = warp % 4, every other 16-column chunk
+        const int q = warp & 3;
+        const bool got = ptx::mbar_wait(ptx::smem_u32(&ctl->accf[0]), 0, abort_flag, p.status,
+                                        MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit);
+        if (__all_sync(0xffffffffu, got)) {
+            ptx::tc_fence_after();
+            const int row = r0 + q * 32 + lane;
+            uint16_t* const ol = p.out_lo[pi];
+            float* const of = p.out[pi];
+            uint16_t* const ob = p.out_bf[pi];
+            const long long ro = (long long)row * N;
+            for (int c = (warp - 2) >> 2; c < nb * 8; c += 2) {
+                const int j0 = n0 + c * 16;
+                if (j0 >= N) break;                       // warp-uniform
+                float v[16];
+                __syncwarp();
+                ptx::tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + c * 16, v);
+                if (row < M) kr_store16(of, ob, ol, ro, j0, N, v);
+            }
+        }
+    }
+
+    ptx::tc_fence_before();
+    __syncwarp();
+    ptx::cluster_sync();            // no CTA leaves while its peer may still signal or fill it
+    if (warp == 1) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc2(tmem, 256);
     }
 }
 
@@ -2296,6 +2465,9 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
         for (auto fn : {kr_product<true, 0>, kr_product<true, 1>, kr_product<true, 2>, kr_product<false, 0>,
                         kr_product<false, 1>, kr_product<false, 2>})
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
+        for (auto fn : {kr_pair<true, 0>, kr_pair<true, 1>, kr_pair<true, 2>, kr_pair<false, 0>, kr_pair<false, 1>,
+                        kr_pair<false, 2>})
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
         st->kr_attrs = true;
     }
     for (int i = 0; i < count; ++i) {
@@ -2312,6 +2484,8 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
         std::vector<int> sel;
         for (int i = 0; i < count; ++i)
             if (kind(items[i]) == with_lo) sel.push_back(i);
+        // longest K first, so that the last CTAs to start are short ones
+        std::stable_sort(sel.begin(), sel.end(), [&](int a, int b) { return items[a].K > items[b].K; });
         for (size_t c0 = 0; c0 < sel.size(); c0 += kKrGroup) {
             const int cnt = static_cast<int>(std::min<size_t>(kKrGroup, sel.size() - c0));
             KrParams& kp = st->pr;
@@ -2344,10 +2518,26 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
             kp.status = st->d_status;
             kp.wait_limit = st->wait_limit;
             if (total == 0) continue;
-            auto fn = a_kmajor ? (with_lo == 0 ? kr_product<true, 0> : with_lo == 1 ? kr_product<true, 1> : kr_product<true, 2>)
+            // CTA pairs where one tile's K outlasts what all tiles take on every
+            // SM (a pair works it off in half the time); the waits of a pair
+            // keep the default bound
+            double longest = 0.0, work = 0.0;
+            for (int q = 0; q < cnt; ++q) {
+                const TcGemmItem& x = items[sel[c0 + q]];
+                longest = std::max(longest, 1.0 * x.K);
+                for (int i0 = 0; i0 < x.M; i0 += KR_BM)
+                    work += 1.0 * x.K * (((x.lower ? std::min(x.N, i0 + KR_BM) : x.N) + KR_BN - 1) / KR_BN);
+            }
+            work /= st->sms;
+            const bool pair = st->wait_limit == kWaitLimit && std::max(0.5 * longest, 1.1 * work) < 0.95 * std::max(longest, work);
+            auto fn = pair ? (a_kmajor ? (with_lo == 0 ? kr_pair<true, 0> : with_lo == 1 ? kr_pair<true, 1> : kr_pair<true, 2>)
+                                       : (with_lo == 0 ? kr_pair<false, 0>
+                                                       : with_lo == 1 ? kr_pair<false, 1> : kr_pair<false, 2>))
+                    : a_kmajor ? (with_lo == 0 ? kr_product<true, 0> : with_lo == 1 ? kr_product<true, 1> : kr_product<true, 2>)
                                : (with_lo == 0 ? kr_product<false, 0>
                                                : with_lo == 1 ? kr_product<false, 1> : kr_product<false, 2>);
-            const cudaError_t e = launch(fn, total, KR_THREADS, KR_SMEM, s, 1, kp);
+            // (the pairs' cluster shape is the kernel's own)
+            const cudaError_t e = launch(fn, pair ? 2 * total : total, KR_THREADS, KR_SMEM, s, 1, kp);
             if (e != cudaSuccess) {
                 st->err = cudaGetErrorString(e);
                 return MOARA_ERR_CUDA;

@@ -45,3 +45,40 @@ def test_refresh_sketch_widths(bf16, l):
     U = top_subspace(G, r)[0]
     if l >= 8:      # a one- or two-column sketch holds a mixture of close directions
         assert np.min(np.abs(np.sum(P * U, axis=0))) >= 0.9999
+
+
+@pytest.mark.parametrize("shapes", [
+    [(264, 2048, 40)],                        # two row tiles, the second of 8 rows; one column tile of 72
+    [(130, 1304, 24), (2312, 136, 96)],       # mixed K, column tiles of 56 and of 128
+    [(1304, 1032, 232), (1032, 1304, 264)],   # l = 264 and 296: a second column tile of 8 and 40
+])
+def test_refresh_product_tiles(shapes):
+    """Refreshes whose products have few tiles and a long K (2-CTA pairs), at
+    row and column tiles with remainders, V and G read both ways.  Energy slack
+    5e-3: with sketches this close to the full width the three Ritz iterations
+    leave 2.2e-3 to 3.5e-3 more than an exact eigensolve, on single-CTA
+    products just so."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_15037_gb300 as M
+    from gpu_helpers import check_refresh
+    from oracle import moara_ref as o
+    from oracle import rsi_ref as R
+    B = 64
+    for rule in (M.MOARA_PROJ_LEFT, M.MOARA_PROJ_SMALLER):
+        g = M.MoaraGroup(block_size=B, proj_rule=rule)
+        gs, Xs = [], []
+        for i, (m, n, r) in enumerate(shapes):
+            G = synth.to_bf16_exact(synth.lowrank_grad(m, n, 16, 10.0, 0.05, 1, seed=2, module=i, noise_rel=True))
+            g.add(m, n, r, "bf16")
+            gs.append(torch.tensor(G, dtype=torch.float32).to(torch.bfloat16).cuda())
+            Xs.append(o.decompose(G, B)[1])
+        g.refresh(gs)
+        torch.cuda.synchronize()
+        assert g.status() == 0
+        for mid, (m, n, r), X in zip(g.ids, shapes, Xs):
+            right = rule == M.MOARA_PROJ_SMALLER and m > n
+            P = g.modules[mid].P.double().cpu().numpy()
+            check_refresh(P, X.T if right else X, r, g.hp.oversample, g.hp.power_iters, R.sketch_key(g.hp.seed, mid, 0),
+                          rsi_slack=5e-3)
+        g.close()
