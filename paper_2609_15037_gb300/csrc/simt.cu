@@ -196,8 +196,24 @@ struct TileLoader {
     }
 };
 
+// What the epilogue of entry (i, j) reads: the moments (EPI_ADAM), or W and dM
+// (EPI_UPDATE).
+struct Old {
+    float x, y;
+};
+
 template <int EPI, int CAP>
-__device__ __forceinline__ void epilogue(const GemmBatchT<CAP>& b, const GemmProb& p, int i, int j, float acc) {
+__device__ __forceinline__ Old epilogue_old(const GemmBatchT<CAP>& b, const GemmProb& p, int i, int j) {
+    const long long o = (long long)i * p.ldc + j;
+    if (EPI == EPI_ADAM) return Old{p.aux0[o], p.aux1[o]};
+    if (EPI == EPI_UPDATE)
+        return Old{p.aux0[o], p.aux2 != nullptr ? p.aux2[(long long)i * p.kb + block_of(j, b.B, b.log2B)] : 1.0f};
+    return Old{0.0f, 0.0f};
+}
+
+template <int EPI, int CAP>
+__device__ __forceinline__ void epilogue(const GemmBatchT<CAP>& b, const GemmProb& p, int i, int j, float acc,
+                                         const Old& old) {
     const long long o = (long long)i * p.ldc + j;
     if (EPI == EPI_STORE) {
         p.C[o] = acc;
@@ -211,16 +227,16 @@ __device__ __forceinline__ void epilogue(const GemmBatchT<CAP>& b, const GemmPro
         // Optimizer_V (Algorithm 1): Adam on the projected direction R = acc
         // (of the clipped gradient when a clipping coefficient is given).
         if (b.clip != nullptr) acc *= *b.clip;
-        float ea = b.beta1 * p.aux0[o] + (1.0f - b.beta1) * acc;
-        float eas = b.beta2 * p.aux1[o] + (1.0f - b.beta2) * acc * acc;
+        float ea = b.beta1 * old.x + (1.0f - b.beta1) * acc;
+        float eas = b.beta2 * old.y + (1.0f - b.beta2) * acc * acc;
         p.aux0[o] = ea;
         p.aux1[o] = eas;
         p.C[o] = (ea / b.bc1) / (sqrtf(eas / b.bc2) + b.adam_eps);
     } else {
         // W <- W - lr*alpha*(Rep_B(dM) (.) dV)  (Algorithm 1; Rep_B of §3.1).
         float u = acc;
-        if (p.aux2 != nullptr) u *= p.aux2[(long long)i * p.kb + block_of(j, b.B, b.log2B)];
-        p.aux0[o] = p.aux0[o] - b.step_scale * u;
+        if (p.aux2 != nullptr) u *= old.y;
+        p.aux0[o] = old.x - b.step_scale * u;
     }
 }
 
@@ -319,7 +335,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm(const __grid_constant__ GemmBat
                     } else {
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
-                            if (j + c < p.N) epilogue<EPI>(b, p, i, j + c, acc[a][4 * h + c]);
+                            if (j + c < p.N) epilogue<EPI>(b, p, i, j + c, acc[a][4 * h + c], epilogue_old<EPI>(b, p, i, j + c));
                     }
                 }
             }
@@ -333,7 +349,7 @@ __global__ void __launch_bounds__(256, 2) k_gemm(const __grid_constant__ GemmBat
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int j = n0 + (c < 4 ? tx * 4 + c : 64 + tx * 4 + (c - 4));
-            if (j < p.N) epilogue<EPI>(b, p, i, j, acc[a][c]);
+            if (j < p.N) epilogue<EPI>(b, p, i, j, acc[a][c], epilogue_old<EPI>(b, p, i, j));
         }
     }
 }
@@ -450,18 +466,38 @@ __global__ void __launch_bounds__(256, 4) k_gemm_small(const __grid_constant__ G
 #pragma unroll
     for (int i = 0; i < 4; ++i)
         *reinterpret_cast<float4*>(&part[4 * ty + i][4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    // entries of the CTA's rows, two a thread at a time: what the epilogue reads
+    // is fetched first, for the first two before the barrier
+    const int R = SM_T / S;
+    Old old[2];
+    auto fetch = [&](int e0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int e = e0 + threadIdx.x + 256 * u, i = m0 + rank * R + e / SM_T, j = n0 + e % SM_T;
+            if (e < R * SM_T && i < p.M && j < p.N) old[u] = epilogue_old<EPI>(b, p, i, j);
+        }
+    };
+    fetch(0);
     if (S > 1) cl.sync();
     else __syncthreads();
-    const int R = SM_T / S;
-    for (int e = threadIdx.x; e < R * SM_T; e += 256) {
-        const int i = rank * R + e / SM_T, j = e % SM_T;
-        float v = 0.0f;
-        if (S > 1) {
-            for (int q = 0; q < split; ++q) v += *cl.map_shared_rank(&part[i][j], q);
-        } else {
-            v = part[i][j];
+    auto total = [&](int i, int j) {
+        if (S == 1) return part[i][j];
+        float x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) x[q] = q < split ? *cl.map_shared_rank(&part[i][j], q) : 0.0f;
+        float v = x[0];
+#pragma unroll
+        for (int q = 1; q < 8; ++q)
+            if (q < split) v += x[q];
+        return v;
+    };
+    for (int e0 = 0; e0 < R * SM_T; e0 += 512) {
+        if (e0 > 0) fetch(e0);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int e = e0 + threadIdx.x + 256 * u, i = rank * R + e / SM_T, j = e % SM_T;
+            if (e < R * SM_T && m0 + i < p.M && n0 + j < p.N) epilogue<EPI>(b, p, m0 + i, n0 + j, total(i, j), old[u]);
         }
-        if (m0 + i < p.M && n0 + j < p.N) epilogue<EPI>(b, p, m0 + i, n0 + j, v);
     }
     if (S > 1) cl.sync();       // no CTA leaves while a peer may still read its partial tile
 }
@@ -540,13 +576,18 @@ static cudaError_t launch_one(GemmBatch& b, cudaStream_t s, int64_t* launches) {
         while ((1 << lg) < b.B) ++lg;
         b.log2B = lg;
     }
-    int whole = 0;
+    int whole = 0, tiles = 0, split = 1;
     for (int i = 0; i < b.count; ++i) {
-        b.p[i].split = k_split(b.p[i]);
-        whole += b.p[i].split == 1;
+        const GemmProb& p = b.p[i];
+        b.p[i].split = k_split(p);
+        whole += p.split == 1;
+        split = p.split > split ? p.split : split;
+        tiles += (p.M + SM_T - 1) / SM_T * ((p.N + SM_T - 1) / SM_T);
     }
-    if (whole == 0 || whole == b.count) return launch_part<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(b, s, launches);
-    // split problems (clusters) and whole ones in launches of their own
+    if (whole == 0 || whole == b.count || tiles * split <= kSmallCtas)
+        return launch_part<ALAY, ASC, ABF, BLAY, BSC, BBF, EPI>(b, s, launches);
+    // split problems and whole ones in launches of their own, where the whole
+    // ones' idle CTAs would not fit beside the others
     for (int part = 0; part < 2; ++part) {
         GemmBatch c = b;
         c.count = 0;
