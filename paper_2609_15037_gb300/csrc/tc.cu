@@ -88,6 +88,12 @@ struct K0Params {
 
 // ------------------------------------------------------------------- K1
 constexpr int K1_BM = 128, K1_BN = 256, K1_BK = 64;
+// Columns of a pair tile where the launch's tiles of 256 would leave half of
+// the pairs idle: half the MMAs and half the epilogue per tile.  Above that a
+// tile of 128 columns is the slower one: it fetches the projector's rows twice
+// as often.  A 1024 / 2816 layer (35 tiles of 256, 76 pairs): 27 us instead of
+// 31, its step 66.4 instead of 70.7.
+constexpr int K1_BN_NARROW = 128;
 constexpr int K1_A_BYTES = K1_BM * K1_BK * 2;           // 16 KB: two 64-rank chunks of P^T (MN-major)
 constexpr int K1_B_BYTES = K1_BK * (K1_BN / 2) * 2;     // 16 KB: this CTA's two 64-column chunks of V
 // The Adam moments stream through a ring of slots, each one 32-column chunk
@@ -397,11 +403,13 @@ __global__ void __launch_bounds__(256) k0_mag_sq(const __grid_constant__ K0Param
 // ===========================================================================
 // RT: the launch may hold modules with a right projector (per-tile operand
 // roles); without it those branches are compiled out.
-template <bool HILO, bool SB, bool RT>
+template <bool HILO, bool SB, bool RT, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(K1_THREADS, 1)
 k1_project(const __grid_constant__ K1Params p) {
     constexpr int MC = StateCols<SB>::N;              // moment columns per chunk
     constexpr int HC = MC / 2;                        // columns per epilogue thread and chunk
+    constexpr int BCH = BN / 128;                     // 64-column chunks of V per CTA
+    constexpr int LOADED = K1_A_BYTES + (HILO ? 2 : 1) * BCH * 8192;   // bytes of a stage that are filled (left projector)
     constexpr int STAGES = K1Cfg<HILO>::STAGES;
     constexpr int STAGE_BYTES = K1Cfg<HILO>::STAGE_BYTES;
     constexpr int MSLOTS = K1Cfg<HILO>::MSLOTS;
@@ -461,7 +469,7 @@ k1_project(const __grid_constant__ K1Params p) {
                 const CUtensorMap* pmap = &p.maps[tl.mod * kMaps + 0];
                 const CUtensorMap* vmap = p.decompose ? &p.maps[tl.mod * kMaps + 4] : &p.gmap[tl.slot];
                 const CUtensorMap* lmap = &p.maps[tl.mod * kMaps + 5];
-                const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * K1_BN;
+                const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * BN;
                 const bool right = RT && md.right != 0;
                 const int nk = ((right ? md.n : md.m) + K1_BK - 1) / K1_BK;
                 for (int kb = 0; kb < nk; ++kb) {
@@ -469,15 +477,17 @@ k1_project(const __grid_constant__ K1Params p) {
                                         MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
                     const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
                     const uint32_t fb = ptx::mapa(own, 0);
-                    if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * STAGE_BYTES);
+                    // a right projector's V_lo is as long as its V (128 rows)
+                    if (crank == 0)
+                        ptx::mbar_arrive_expect_tx(own, 2 * (right ? K1_A_BYTES * (HILO ? 2 : 1) + BCH * 8192 : LOADED));
                     const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
                     const uint32_t b = a + K1_A_BYTES;
                     if (!right) {
 #pragma unroll
                         for (int c = 0; c < 2; ++c) ptx::tma_load_2d_pair(a + c * 8192, pmap, fb, r0 + 64 * c, kb * K1_BK);
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int c = 2 * crank + h;
+                        for (int h = 0; h < BCH; ++h) {
+                            const int c = BCH * crank + h;
                             ptx::tma_load_2d_pair(b + h * 8192, vmap, fb, n0 + 64 * c, kb * K1_BK);
                             if (HILO) ptx::tma_load_2d_pair(b + K1_B_BYTES + h * 8192, lmap, fb, n0 + 64 * c, kb * K1_BK);
                         }
@@ -488,8 +498,8 @@ k1_project(const __grid_constant__ K1Params p) {
                         ptx::tma_load_2d_pair(a, vmap, fb, kb * K1_BK, r0);
                         if (HILO) ptx::tma_load_2d_pair(b + K1_B_BYTES, lmap, fb, kb * K1_BK, r0);
 #pragma unroll
-                        for (int h = 0; h < 2; ++h)
-                            ptx::tma_load_2d_pair(b + h * 8192, pmap, fb, n0 + 64 * (2 * crank + h), kb * K1_BK);
+                        for (int h = 0; h < BCH; ++h)
+                            ptx::tma_load_2d_pair(b + h * 8192, pmap, fb, n0 + 64 * (BCH * crank + h), kb * K1_BK);
                     }
                     issued |= 1u << stage;
                     last_par = (last_par & ~(1u << stage)) | (phase << stage);
@@ -507,8 +517,8 @@ k1_project(const __grid_constant__ K1Params p) {
             // M = 256 (both CTAs' rank tiles), N = 256, K = 16 per MMA; the
             // full barrier of a stage counts both CTAs' copies
             if (lane == 0) {
-                constexpr uint32_t idesc_l = ptx::idesc_bf16(256, K1_BN, 1, 1);   // A MN-major (P^T)
-                constexpr uint32_t idesc_r = ptx::idesc_bf16(256, K1_BN, 0, 1);   // A K-major (V rows)
+                constexpr uint32_t idesc_l = ptx::idesc_bf16(256, BN, 1, 1);   // A MN-major (P^T)
+                constexpr uint32_t idesc_r = ptx::idesc_bf16(256, BN, 0, 1);   // A K-major (V rows)
                 int stage = 0;
                 uint32_t phase = 0;
                 int buf = 0;
@@ -572,9 +582,9 @@ k1_project(const __grid_constant__ K1Params p) {
                 const TcMod& md = p.mods[tl.mod];
                 const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 6];
                 const CUtensorMap* smap = &p.maps[tl.mod * kMaps + 7];
-                const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * K1_BN;
+                const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * BN;
                 const int cols = (RT && md.right) ? md.r : md.n;    // R is r x n, or m x r (right projector)
-                const int nc = min(K1_BN / MC, (cols - n0 + MC - 1) / MC);
+                const int nc = min(BN / MC, (cols - n0 + MC - 1) / MC);
                 for (int c = 0; c < nc; ++c, ++g) {
                     const int b = g % MSLOTS;
                     const uint32_t ph = (g / MSLOTS) & 1;
@@ -604,9 +614,9 @@ k1_project(const __grid_constant__ K1Params p) {
                 const TcMod& md = p.mods[tl.mod];
                 const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 6];
                 const CUtensorMap* smap = &p.maps[tl.mod * kMaps + 7];
-                const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * K1_BN;
+                const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * BN;
                 const int cols = (RT && md.right) ? md.r : md.n;    // R is r x n, or m x r (right projector)
-                const int nc = min(K1_BN / MC, (cols - n0 + MC - 1) / MC);
+                const int nc = min(BN / MC, (cols - n0 + MC - 1) / MC);
                 for (int c = 0; c < nc; ++c, ++g) {
                     const int b = g % MSLOTS;
                     const uint32_t ph = (g / MSLOTS) & 1;
@@ -644,10 +654,10 @@ k1_project(const __grid_constant__ K1Params p) {
             // R (and the moments, N) is r x n, or m x r with a right projector
             const int rr = (RT && md.right) ? md.m : md.r, nn = (RT && md.right) ? md.r : md.n;
             uint16_t* const nb_p = md.Nb;
-            const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * K1_BN;
+            const int r0 = (2 * tl.t0 + crank) * K1_BM, n0 = tl.t1 * BN;
             const int a = r0 + il;
             const bool row_ok = a < rr;
-            const int nc = min(K1_BN / MC, (nn - n0 + MC - 1) / MC);
+            const int nc = min(BN / MC, (nn - n0 + MC - 1) / MC);
             const bool got = ptx::mbar_wait(ptx::smem_u32(&ctl->accf[buf]), acc_phase, abort_flag, p.status,
                                             MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit);
             if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
@@ -1887,7 +1897,7 @@ struct TcState {
     // Per-CTA work lists of one launch (CSR: start offsets, then tiles).
     struct Tiles {
         void* mem = nullptr;
-        const int* k1_start = nullptr; const TcTile* k1 = nullptr; int g1 = 0;
+        const int* k1_start = nullptr; const TcTile* k1 = nullptr; int g1 = 0; int bn1 = K1_BN;
         const int* k2_start = nullptr; const TcTile* k2 = nullptr; int g2 = 0;
     };
     std::map<std::vector<int>, Tiles> tiles;
@@ -2097,14 +2107,20 @@ static void lpt_assign(const std::vector<TcTile>& tiles, const std::vector<doubl
 // Shared-memory limits of the step kernels and their resident grids.
 static void tc_init(TcState* st) {
     if (!st->attrs_set) {
-        for (auto fn : {k1_project<true, false, false>, k1_project<false, false, false>, k1_project<true, true, false>,
-                        k1_project<false, true, false>, k1_project<true, false, true>, k1_project<false, false, true>,
-                        k1_project<true, true, true>, k1_project<false, true, true>})
+        constexpr int W = K1_BN, N = K1_BN_NARROW;
+        for (auto fn : {k1_project<true, false, false, W>, k1_project<false, false, false, W>,
+                        k1_project<true, true, false, W>, k1_project<false, true, false, W>,
+                        k1_project<true, false, true, W>, k1_project<false, false, true, W>,
+                        k1_project<true, true, true, W>, k1_project<false, true, true, W>,
+                        k1_project<true, false, false, N>, k1_project<false, false, false, N>,
+                        k1_project<true, true, false, N>, k1_project<false, true, false, N>,
+                        k1_project<true, false, true, N>, k1_project<false, false, true, N>,
+                        k1_project<true, true, true, N>, k1_project<false, true, true, N>})
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, K1_SMEM);
         set_smem_attrs<8>(); set_smem_attrs<16>(); set_smem_attrs<32>(); set_smem_attrs<64>();
         set_smem_attrs<128>();
         // clusters of two that fit on the GPU at once (persistent grids)
-        st->k1_clusters = max_clusters(reinterpret_cast<const void*>(k1_project<false, false, false>), K1_THREADS,
+        st->k1_clusters = max_clusters(reinterpret_cast<const void*>(k1_project<false, false, false, K1_BN>), K1_THREADS,
                                        K1_SMEM,
                                        st->sms / 2);
         st->k2_clusters = max_clusters(reinterpret_cast<const void*>(k2_backproject<128, false>), K2_THREADS, K2_SMEM,
@@ -2125,18 +2141,26 @@ static TcState::Tiles* tc_tiles(TcState* st, const std::vector<int>& ids) {
     // row (K2) tiles 2 t0 and 2 t0 + 1 of the same column tile t1.
     std::vector<TcTile> k1, k2;
     std::vector<double> c1, c2;
+    // columns of a K1 tile (see K1_BN_NARROW)
+    int wide = 0;
+    for (int id : ids) {
+        const TcMod& md = st->mods[id];
+        const int rows = md.right ? md.m : md.r, cols = md.right ? md.r : md.n;
+        wide += (rows + 2 * K1_BM - 1) / (2 * K1_BM) * ((cols + K1_BN - 1) / K1_BN);
+    }
+    const int bn = 2 * wide <= st->k1_clusters ? K1_BN_NARROW : K1_BN;
     for (size_t slot = 0; slot < ids.size(); ++slot) {
         const TcMod& md = st->mods[ids[slot]];
         // column tiles outer, rank pairs inner: clusters that start together
         // share the V panel of one column tile in L2
         // R: r x n (K = m), or m x r (K = n) with a right projector
         const int Rr = md.right ? md.m : md.r, Rc = md.right ? md.r : md.n, Rk = md.right ? md.n : md.m;
-        const int nt = (Rc + K1_BN - 1) / K1_BN, rt = (Rr + K1_BM - 1) / K1_BM;
+        const int nt = (Rc + bn - 1) / bn, rt = (Rr + K1_BM - 1) / K1_BM;
         for (int j = 0; j < nt; ++j)
             for (int i = 0; i < (rt + 1) / 2; ++i) {
                 const int rows = std::min(K1_BM, Rr - 2 * i * K1_BM);
-                const double mma = 8.0 * Rk;
-                const double epi = 0.66 * rows * std::min(K1_BN, Rc - j * K1_BN);
+                const double mma = 8.0 * Rk * bn / K1_BN;
+                const double epi = 0.66 * rows * std::min(bn, Rc - j * bn);
                 k1.push_back({ids[slot], static_cast<int>(slot), i, j});
                 c1.push_back(std::max(mma, epi));
             }
@@ -2150,6 +2174,7 @@ static TcState::Tiles* tc_tiles(TcState* st, const std::vector<int>& ids) {
             }
     }
     TcState::Tiles t;
+    t.bn1 = bn;
     t.g1 = std::max(1, std::min(static_cast<int>(k1.size()), st->k1_clusters));   // clusters
     t.g2 = std::max(1, std::min(static_cast<int>(k2.size()), st->k2_clusters));
     std::vector<int> s1, s2;
@@ -2212,13 +2237,16 @@ static cudaError_t launch_k0(TcState* st, const K0Params& p0, bool background, c
 
 // which: 1 = K1, 2 = K2, 4 = K1 directly behind its decomposition on the stream
 template <int BLK, bool SB>
-static cudaError_t launch_k12(TcState* st, const K1Params& p1, const K2Params& p2, int g1, int g2, bool hilo,
+static cudaError_t launch_k12(TcState* st, const K1Params& p1, const K2Params& p2, int g1, int bn, int g2, bool hilo,
                               cudaStream_t s, int64_t* launches, const TcProfile& prof, int which, bool rt) {
     cudaError_t e;
     if (which & 1) {
         if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_PROJECT, s, true);
-        auto fn = rt ? (hilo ? k1_project<true, SB, true> : k1_project<false, SB, true>)
-                     : (hilo ? k1_project<true, SB, false> : k1_project<false, SB, false>);
+        constexpr int W = K1_BN, N = K1_BN_NARROW;
+        auto fn = bn == W ? (rt ? (hilo ? k1_project<true, SB, true, W> : k1_project<false, SB, true, W>)
+                                : (hilo ? k1_project<true, SB, false, W> : k1_project<false, SB, false, W>))
+                          : (rt ? (hilo ? k1_project<true, SB, true, N> : k1_project<false, SB, true, N>)
+                                : (hilo ? k1_project<true, SB, false, N> : k1_project<false, SB, false, N>));
         // of several parts, K1 waits for its part's decomposition on the other stream
         e = launch_if((which & 4) != 0 && !prof.on, fn, 2 * g1, K1_THREADS, K1_SMEM, s, 1, p1);
         if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_PROJECT, s, false);
@@ -2246,21 +2274,21 @@ static cudaError_t launch_k0_any(int B, TcState* st, const K0Params& p0, bool ba
 }
 
 static cudaError_t launch_k12_any(int B, bool sb, TcState* st, const K1Params& p1, const K2Params& p2, int g1,
-                                  int g2, bool hilo, cudaStream_t s, int64_t* launches, const TcProfile& prof,
+                                  int bn, int g2, bool hilo, cudaStream_t s, int64_t* launches, const TcProfile& prof,
                                   int which, bool rt = false) {
     if (sb) {   // bf16 states: B >= 32 (tc_supported)
         switch (B) {
-            case 32: return launch_k12<32, true>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
-            case 64: return launch_k12<64, true>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
-            default: return launch_k12<128, true>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
+            case 32: return launch_k12<32, true>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
+            case 64: return launch_k12<64, true>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
+            default: return launch_k12<128, true>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
         }
     }
     switch (B) {
-        case 8: return launch_k12<8, false>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
-        case 16: return launch_k12<16, false>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
-        case 32: return launch_k12<32, false>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
-        case 64: return launch_k12<64, false>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
-        default: return launch_k12<128, false>(st, p1, p2, g1, g2, hilo, s, launches, prof, which, rt);
+        case 8: return launch_k12<8, false>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
+        case 16: return launch_k12<16, false>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
+        case 32: return launch_k12<32, false>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
+        case 64: return launch_k12<64, false>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
+        default: return launch_k12<128, false>(st, p1, p2, g1, bn, g2, hilo, s, launches, prof, which, rt);
     }
 }
 
@@ -2398,7 +2426,7 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
             // left a gap after each K1 and was slower.)
             const bool bg = dec && q + 1 < np;
             if (bg && cudaEventRecord(st->ev_k1[q], s) != cudaSuccess) return fail("part event");
-            cudaError_t e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->g2, hilo, s, launches, prof, np == 1 ? 5 : 1, rt);
+            cudaError_t e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->bn1, tl->g2, hilo, s, launches, prof, np == 1 ? 5 : 1, rt);
             if (e != cudaSuccess) {
                 st->err = cudaGetErrorString(e);
                 return MOARA_ERR_CUDA;
@@ -2411,7 +2439,7 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
                     return fail("background decomposition launch failed");
             }
             if (!fused) {
-                e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->g2, hilo, s, launches, prof, 2, rt);
+                e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->bn1, tl->g2, hilo, s, launches, prof, 2, rt);
                 if (e != cudaSuccess) {
                     st->err = cudaGetErrorString(e);
                     return MOARA_ERR_CUDA;
@@ -2442,7 +2470,7 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
             p2.mods = st->d_mods; p2.maps = st->d_maps; p2.status = st->d_status;
             p2.step_scale = lr * hp.scale;
             p2.decompose = hp.decompose;
-            const cudaError_t e = launch_k12_any(B, hp.state_dtype == MOARA_DTYPE_BF16, st, st->p1, p2, tl->g1, tl->g2,
+            const cudaError_t e = launch_k12_any(B, hp.state_dtype == MOARA_DTYPE_BF16, st, st->p1, p2, tl->g1, tl->bn1, tl->g2,
                                                  hilo, s, launches, prof, 2);
             if (e != cudaSuccess) {
                 st->err = cudaGetErrorString(e);
