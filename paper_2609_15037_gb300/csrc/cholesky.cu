@@ -25,10 +25,11 @@
 // spent two barriers per pivot (43 us a launch), a panel solve (11 us) and a
 // trailing update (14 us) as launches of their own, a 64-column step took
 // 68 us, and the inverse's levels up to 256 another 36 us each; here a step
-// takes 16 us (seven modules, l = 160 / 288) to 21 us (l = 544 to 2080, mean
-// over the steps) and the levels up to 256 are inside it.  A refresh plus
-// alignment of the 1024 / 2816 layer went from 10.33 to 4.71 ms, of the 4096 /
-// 11008 layer from 68.0 to 39.8 ms.
+// takes 14 us (seven modules, l = 160 / 288) to 21 us (l = 544 to 2080, mean
+// over the steps; up to 33 us where the updates of seven modules fill the GPU
+// more than once) and the whole inverse is inside it.  The first form of this
+// kernel took a refresh plus alignment of the 1024 / 2816 layer from 10.33 to
+// 4.71 ms, of the 4096 / 11008 layer from 68.0 to 39.8 ms.
 #include <algorithm>
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -84,6 +85,11 @@ struct Block {
     float4 v[4];
     __device__ __forceinline__ void load(const float* src, long long l, int nr, int nc, bool vec) {
         const int i = threadIdx.x >> 2, k0 = (threadIdx.x & 3) * 4;
+        if (vec && nr >= NB && nc >= NB) {            // the same for every thread: four loads, no branches
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) v[kk] = *reinterpret_cast<const float4*>(src + i * l + kk * 16 + k0);
+            return;
+        }
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
             const int k = kk * 16 + k0;
@@ -459,24 +465,41 @@ __device__ __forceinline__ void wide_update(const float (*As)[LDW], const float 
 #pragma unroll
             for (int q = 0; q < 8; ++q) acc[p][q] = fmaf(av[p], bv[q], acc[p][q]);
     }
+    // A column half's entries of C are all fetched before the first is stored:
+    // read and written one after the other, sixteen L2 latencies stood in a row
+    // and a step with l = 2080 alone took 24 us instead of 16, with the seven
+    // modules of a 4096 / 11008 layer up to 43 instead of 32 (its refresh and
+    // alignment 24.4 ms instead of 22.4).
 #pragma unroll
-    for (int p = 0; p < 8; ++p) {
-        const int i = (p >> 2) * NB + 4 * ty + (p & 3);
-        if (i >= nr) continue;
+    for (int h = 0; h < 2; ++h) {
+        const int j = h * NB + 4 * tx;
+        if (j >= nc) continue;
+        const bool z = h == 0 ? zero0 : zero1;
+        const int i0 = 4 * ty, li = static_cast<int>(l);
+        float* const c = C + (i0 * li + j);
+        auto at = [&](int p) { return ((p >> 2) * NB + (p & 3)) * li; };
+        auto mine = [&](int p) { return i0 + (p >> 2) * NB + (p & 3) < nr && !(skip && h == 0 && p < 4); };
+        if (vec && j + 3 < nc) {
+            float4 o[8];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int j = h * NB + 4 * tx;
-            if (j >= nc || (skip && h == 0 && p < 4)) continue;
-            const bool z = h == 0 ? zero0 : zero1;
-            float* c = C + i * l + j;
-            const float* x = &acc[p][4 * h];
-            if (vec && j + 3 < nc) {
-                const float4 o = z ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : *reinterpret_cast<const float4*>(c);
-                *reinterpret_cast<float4*>(c) = make_float4(o.x - x[0], o.y - x[1], o.z - x[2], o.w - x[3]);
-            } else {
+            for (int p = 0; p < 8; ++p) {
+                o[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (!z && mine(p)) o[p] = *reinterpret_cast<const float4*>(c + at(p));
+            }
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                const float* x = &acc[p][4 * h];
+                if (mine(p))
+                    *reinterpret_cast<float4*>(c + at(p)) =
+                        make_float4(o[p].x - x[0], o[p].y - x[1], o[p].z - x[2], o[p].w - x[3]);
+            }
+        } else {
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                if (!mine(p)) continue;
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (j + q < nc) c[q] = (z ? 0.0f : c[q]) - x[q];
+                    if (j + q < nc) c[at(p) + q] = (z ? 0.0f : c[at(p) + q]) - acc[p][4 * h + q];
             }
         }
     }
