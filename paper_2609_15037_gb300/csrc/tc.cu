@@ -2292,12 +2292,19 @@ static cudaError_t launch_k12_any(int B, bool sb, TcState* st, const K1Params& p
     }
 }
 
-// Modules per launch group are split into this many parts (consecutive
-// modules, about equal gradient bytes) when the group has at least
-// kOverlapMin modules: the decomposition of part q + 1 runs on an auxiliary
-// stream while K1 / K2 of part q run.
+// A launch group is split into parts (consecutive modules, about equal
+// gradient bytes): the decomposition of part q + 1 runs on an auxiliary stream
+// while K1 / K2 of part q run.  A part carries at least kPartBytes of
+// gradients, two 4096 / 11008 layers: every part boundary ends two persistent
+// grids and starts two, which costs more than the hidden decomposition gives
+// where a part holds less.  Measured, us per step with 1 / 2 / 4 / 8 / 16 parts:
+//   24 layers of 1024 / 2816 (0.6 GB)     1008   1023   1074   1132   1385
+//    4 layers of 4096 / 11008 (1.6 GB)    3501   3465   3487   3599   3795
+//    5 layers (2.0 GB)                    4405   4320   4336   4433   4627
+//    8 layers (3.2 GB)                    7080   6863   6968   6902   7185
+//   12 layers (4.9 GB)                   10755  10411  10428  10350  10536
 constexpr int kOverlapParts = 16;
-constexpr int kOverlapMin = 32;
+constexpr double kPartBytes = 0.8e9;
 static_assert(kOverlapParts <= 32, "one event per part");
 
 int tc_group_limit() { return kTcGroup; }
@@ -2325,11 +2332,11 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
     for (int c0 = 0; c0 < n_mod; c0 += kTcGroup) {
         const int cnt = std::min(kTcGroup, n_mod - c0);
         // parts of the group (consecutive modules, about equal G bytes)
-        const int nparts = (dec && cnt >= kOverlapMin) ? kOverlapParts : 1;
+        double tot = 0.0;
+        for (int q = 0; q < cnt; ++q) tot += (double)st->mods[ids[c0 + q]].m * st->mods[ids[c0 + q]].n;
+        const int nparts = dec ? std::max(1, static_cast<int>(std::min<double>(kOverlapParts, 2.0 * tot / kPartBytes))) : 1;
         std::vector<int> pstart{0};
         if (nparts > 1) {
-            double tot = 0.0;
-            for (int q = 0; q < cnt; ++q) tot += (double)st->mods[ids[c0 + q]].m * st->mods[ids[c0 + q]].n;
             double acc = 0.0;
             for (int q = 0; q < cnt; ++q) {
                 acc += (double)st->mods[ids[c0 + q]].m * st->mods[ids[c0 + q]].n;
