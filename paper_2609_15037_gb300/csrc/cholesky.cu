@@ -49,6 +49,15 @@ constexpr int kCritCtas = 4;          // CTAs of the chain per module (a cluster
 constexpr int kCritModules = 38;      // modules up to which they fit beside each other, one per SM
 constexpr int CHOL_SMEM = 5 * NB * LD * sizeof(float);
 static_assert(5 * LD >= 2 * LDW, "two 128-wide operand tiles fit the chain's five buffers");
+// A launch of at most two CTAs per SM whose chain runs on clusters asks for so
+// much shared memory that a CTA has its SM to itself: an update tile beside the
+// chain slows every link of it (refresh and alignment of a 1024 / 2816 layer
+// 3.04 -> 2.79 ms, of a 4096 / 11008 layer 22.6 -> 21.6).  Larger launches are
+// bound by their tiles and lose by it: the refresh of five 4096 / 11008 layers
+// 72.1 -> 79.4 ms with every launch so, 71.9 with this line; lines of 228, 400
+// and 500 CTAs give the same within 1%.
+constexpr int kAloneCtas = 304;
+constexpr int CHOL_SMEM_ALONE = 120 * 1024;
 constexpr int SP = 8;                 // pivots per sub-panel of the diagonal block
 
 // Tile counts of one module at step s; the same on the host and the device.
@@ -814,7 +823,7 @@ __global__ void __launch_bounds__(NT, 2) k_chol_step(const __grid_constant__ Cho
 
 cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches) {
     if (b.count <= 0) return cudaSuccess;
-    const cudaError_t ea = cudaFuncSetAttribute(k_chol_step, cudaFuncAttributeMaxDynamicSharedMemorySize, CHOL_SMEM);
+    const cudaError_t ea = cudaFuncSetAttribute(k_chol_step, cudaFuncAttributeMaxDynamicSharedMemorySize, CHOL_SMEM_ALONE);
     if (ea != cudaSuccess) return ea;
     int nbmax = 0;
     for (int i = 0; i < b.count; ++i) nbmax = std::max(nbmax, (b.p[i].l + NB - 1) / NB);
@@ -828,8 +837,10 @@ cudaError_t launch_cholesky(CholBatch& b, cudaStream_t s, int64_t* launches) {
         b.step = step;
         if (total == 0 && step == nbmax - 1) break;           // no module has anything left
         const int C = b.count <= kCritModules ? kCritCtas : 1;
+        const int ctas = C * b.count + (total + C - 1) / C * C;
         ++*launches;
-        const cudaError_t e = launch(k_chol_step, dim3(C * b.count + (total + C - 1) / C * C), NT, CHOL_SMEM, s, C, b);
+        const cudaError_t e = launch(k_chol_step, dim3(ctas), NT, C > 1 && ctas <= kAloneCtas ? CHOL_SMEM_ALONE : CHOL_SMEM,
+                                     s, C, b);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
