@@ -2216,7 +2216,7 @@ static auto k0_plain(int B) {
 // on each SM instead of a persistent grid that would hold SMs they need.
 template <int BLK>
 static cudaError_t launch_k0(TcState* st, const K0Params& p0, bool background, cudaStream_t s,
-                             int64_t* launches, const TcProfile& prof, bool mag_adam = true) {
+                             int64_t* launches, const TcProfile& prof, bool early, bool mag_adam) {
     const int phase = background ? MOARA_PHASE_TC_DECOMPOSE_OVERLAP : MOARA_PHASE_TC_DECOMPOSE;
     if (prof.on) prof.mark(prof.ctx, phase, s, true);
     const long long items = p0.start[p0.count];
@@ -2225,17 +2225,17 @@ static cudaError_t launch_k0(TcState* st, const K0Params& p0, bool background, c
     bool pass = mag_adam;                              // Optimizer_M as a pass of its own
     cudaError_t e = cudaSuccess;
     if constexpr (BLK >= 32) {
-        if (mag_adam) e = launch_if(!background, k0_decompose<BLK, true>, g0, 256, 0, s, 1, p0);
+        if (mag_adam) e = launch_if(early && !background, k0_decompose<BLK, true>, g0, 256, 0, s, 1, p0);
         pass = false;
     }
-    if (BLK < 32 || !mag_adam) e = launch_if(!background, k0_decompose<BLK, false>, g0, 256, 0, s, 1, p0);
-    if (pass && e == cudaSuccess) e = launch_if(!background, k0_mag_adam, background ? st->sms : st->sms * 4, 256, 0, s, 1, p0);
+    if (BLK < 32 || !mag_adam) e = launch_if(early && !background, k0_decompose<BLK, false>, g0, 256, 0, s, 1, p0);
+    if (pass && e == cudaSuccess) e = launch_if(early && !background, k0_mag_adam, background ? st->sms : st->sms * 4, 256, 0, s, 1, p0);
     if (prof.on) prof.mark(prof.ctx, phase, s, false);
     *launches += pass ? 2 : 1;
     return e;
 }
 
-// which: 1 = K1, 2 = K2, 4 = K1 directly behind its decomposition on the stream
+// which: 1 = K1, 2 = K2, 4 = early launches (of K1 only directly behind its decomposition on the stream)
 template <int BLK, bool SB>
 static cudaError_t launch_k12(TcState* st, const K1Params& p1, const K2Params& p2, int g1, int bn, int g2, bool hilo,
                               cudaStream_t s, int64_t* launches, const TcProfile& prof, int which, bool rt) {
@@ -2255,7 +2255,7 @@ static cudaError_t launch_k12(TcState* st, const K1Params& p1, const K2Params& p
     }
     if (!(which & 2)) return cudaSuccess;
     if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_BACKPROJECT, s, true);
-    e = launch_if(!prof.on, k2_backproject<BLK, SB>, 2 * g2, K2_THREADS, K2_SMEM, s, 1, p2);
+    e = launch_if((which & 4) != 0 && !prof.on, k2_backproject<BLK, SB>, 2 * g2, K2_THREADS, K2_SMEM, s, 1, p2);
     if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_BACKPROJECT, s, false);
     if (e != cudaSuccess) return e;
     ++*launches;
@@ -2263,13 +2263,13 @@ static cudaError_t launch_k12(TcState* st, const K1Params& p1, const K2Params& p
 }
 
 static cudaError_t launch_k0_any(int B, TcState* st, const K0Params& p0, bool background, cudaStream_t s,
-                                 int64_t* launches, const TcProfile& prof, bool mag_adam = true) {
+                                 int64_t* launches, const TcProfile& prof, bool early, bool mag_adam) {
     switch (B) {
-        case 8: return launch_k0<8>(st, p0, background, s, launches, prof, mag_adam);
-        case 16: return launch_k0<16>(st, p0, background, s, launches, prof, mag_adam);
-        case 32: return launch_k0<32>(st, p0, background, s, launches, prof, mag_adam);
-        case 64: return launch_k0<64>(st, p0, background, s, launches, prof, mag_adam);
-        default: return launch_k0<128>(st, p0, background, s, launches, prof, mag_adam);
+        case 8: return launch_k0<8>(st, p0, background, s, launches, prof, early, mag_adam);
+        case 16: return launch_k0<16>(st, p0, background, s, launches, prof, early, mag_adam);
+        case 32: return launch_k0<32>(st, p0, background, s, launches, prof, early, mag_adam);
+        case 64: return launch_k0<64>(st, p0, background, s, launches, prof, early, mag_adam);
+        default: return launch_k0<128>(st, p0, background, s, launches, prof, early, mag_adam);
     }
 }
 
@@ -2305,6 +2305,14 @@ static cudaError_t launch_k12_any(int B, bool sb, TcState* st, const K1Params& p
 //   12 layers (4.9 GB)                   10755  10411  10428  10350  10536
 constexpr int kOverlapParts = 16;
 constexpr double kPartBytes = 0.8e9;
+// Groups of up to so many gradient bytes, and every group without a
+// decomposition, launch each kernel beside the end of the one in front.
+// Larger decomposed groups lose by it when steps follow one another (us per
+// step with / without: one layer of 1024 / 2816, 25 MB, 66.0 / 71.6; two 108.9 /
+// 112.8; four 194.3 / 193.8; eight 361.8 / 352.1; thirty ragged weights of 0.63
+// GB 1053 / 1011; a 4096 / 11008 layer 872 / 862; a layer without decomposition
+// 730 / 742).
+constexpr double kEarlyBytes = 6.4e7;
 static_assert(kOverlapParts <= 32, "one event per part");
 
 int tc_group_limit() { return kTcGroup; }
@@ -2335,6 +2343,7 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
         double tot = 0.0;
         for (int q = 0; q < cnt; ++q) tot += (double)st->mods[ids[c0 + q]].m * st->mods[ids[c0 + q]].n;
         const int nparts = dec ? std::max(1, static_cast<int>(std::min<double>(kOverlapParts, 2.0 * tot / kPartBytes))) : 1;
+        const bool early = !dec || 2.0 * tot <= kEarlyBytes;
         std::vector<int> pstart{0};
         if (nparts > 1) {
             double acc = 0.0;
@@ -2389,7 +2398,7 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
         // decomposition: part 0 on s with the full grid; part q + 1 in the
         // background on the auxiliary stream, launched after K1 / K2 of part q
         // so that their persistent CTAs are placed first
-        if (dec && launch_k0_any(B, st, *build_p0(pstart[0], pstart[1]), false, s, launches, prof, !fused) !=
+        if (dec && launch_k0_any(B, st, *build_p0(pstart[0], pstart[1]), false, s, launches, prof, early, !fused) !=
                        cudaSuccess)
             return fail("decomposition launch failed");
         for (int q = 0; q < np; ++q) {
@@ -2433,7 +2442,8 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
             // left a gap after each K1 and was slower.)
             const bool bg = dec && q + 1 < np;
             if (bg && cudaEventRecord(st->ev_k1[q], s) != cudaSuccess) return fail("part event");
-            cudaError_t e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->bn1, tl->g2, hilo, s, launches, prof, np == 1 ? 5 : 1, rt);
+            cudaError_t e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->bn1, tl->g2, hilo, s, launches, prof,
+                                           np == 1 && early ? 5 : 1, rt);
             if (e != cudaSuccess) {
                 st->err = cudaGetErrorString(e);
                 return MOARA_ERR_CUDA;
@@ -2441,12 +2451,12 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
             if (bg) {
                 if (cudaStreamWaitEvent(st->aux, st->ev_k1[q], 0) != cudaSuccess ||
                     launch_k0_any(B, st, *build_p0(pstart[q + 1], pstart[q + 2]), true, st->aux, launches, prof,
-                                  !fused) != cudaSuccess ||
+                                  false, !fused) != cudaSuccess ||
                     cudaEventRecord(st->ev_part[q + 1], st->aux) != cudaSuccess)
                     return fail("background decomposition launch failed");
             }
             if (!fused) {
-                e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->bn1, tl->g2, hilo, s, launches, prof, 2, rt);
+                e = launch_k12_any(B, sb, st, p1, p2, tl->g1, tl->bn1, tl->g2, hilo, s, launches, prof, early ? 6 : 2, rt);
                 if (e != cudaSuccess) {
                     st->err = cudaGetErrorString(e);
                     return MOARA_ERR_CUDA;
