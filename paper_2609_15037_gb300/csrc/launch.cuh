@@ -42,7 +42,10 @@ cudaError_t launch_if(bool overlap, void (*fn)(P...), dim3 grid, dim3 block, siz
     cfg.attrs = at;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     void* ptrs[] = {const_cast<void*>(static_cast<const void*>(&args))...};
-    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(fn), ptrs);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(fn), ptrs);
+    // reported here: a later call that asks for the runtime's last error must not meet it again
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 template <class... P, class... A>

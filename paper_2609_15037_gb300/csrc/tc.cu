@@ -2476,7 +2476,8 @@ int tc_step(TcState* st, const moara_hparams& hp, int n_mod, const int* ids, con
                 return fail("clipping coefficient launch failed");
             if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_CLIP_NORM, s, false);
             if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_DECOMPOSE, s, true);
-            k0_mag_adam<<<st->sms * 4, 256, 0, s>>>(*pall);
+            if (launch_if(false, k0_mag_adam, st->sms * 4, 256, 0, s, 1, *pall) != cudaSuccess)
+                return fail("clipped magnitude launch failed");
             ++*launches;
             if (prof.on) prof.mark(prof.ctx, MOARA_PHASE_TC_DECOMPOSE, s, false);
             std::vector<int> all(ids + c0, ids + c0 + cnt);
