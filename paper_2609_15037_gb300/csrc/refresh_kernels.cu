@@ -8,6 +8,7 @@
 
 #include "internal.h"
 #include "launch.cuh"
+#include "ritz.h"
 
 namespace moara {
 
@@ -419,11 +420,11 @@ __global__ void __launch_bounds__(kSmallThreads) k_ritz_values(const __grid_cons
         acc += __shfl_xor_sync(0xffffffffu, acc, o);
         nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
     }
-    if (lane == 0 && j0 + warp < l) b.c[pi][j0 + warp] = nrm > 0.0f ? acc / nrm : 0.0f;
+    if (lane == 0 && j0 + warp < l) b.c[pi][j0 + warp] = ritz_value(acc, nrm);
 }
 
 // The descending order of the Ritz values (c): iaux[rank] = j,
-// rank_j = #{i : d_i > d_j, or d_i == d_j and i < j}.
+// rank_j = #{i : d_i before d_j}.
 __global__ void __launch_bounds__(256) k_ritz_order(const __grid_constant__ SmallBatch b) {
     pdl_begin();
     __shared__ float d[1024];
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(256) k_ritz_order(const __grid_constant__ Smal
         __syncthreads();
         for (int i = threadIdx.x; i < cnt; i += 256) d[i] = b.c[pi][i0 + i];
         __syncthreads();
-        for (int i = 0; i < cnt; ++i) rank += (d[i] > dj || (d[i] == dj && i0 + i < j)) ? 1 : 0;
+        for (int i = 0; i < cnt; ++i) rank += ritz_before(d[i], i0 + i, dj, j) ? 1 : 0;
     }
     if (j < l) b.iaux[pi][rank] = j;
 }
