@@ -169,10 +169,21 @@ struct K2Params {
     int decompose;
 };
 
+// The diagnostic's tiles are numbered in the parameter block, modules in
+// descending K, and cluster c takes tiles c, c + clusters, ...: within one tile
+// of the longest-first assignment of the step's work lists, without a list in
+// device memory (the call may be recorded in a graph for modules that no call
+// had together before, and scoring many subsets keeps nothing).
 struct K2AlignParams : K2Params {
     const uint16_t* G[kTcGroup];       // gradient of each launch slot (m x n)
-    double* acc;                       // three sums per launch slot: <G, a>, <a, a>, <G, G>
+    double* acc;                       // three sums per module of the call: <G, a>, <a, a>, <G, G>
+    int count;
+    int mod[kTcGroup];                 // module of the slot
+    int call_idx[kTcGroup];            // its place in the call
+    int col_tiles[kTcGroup];
+    int start[kTcGroup + 1];           // first tile of the slot
 };
+static_assert(sizeof(K2AlignParams) <= 32764, "the diagnostic's parameter block fits the kernel parameter space");
 
 struct SmemCtl {
     uint64_t full[8];
@@ -825,7 +836,26 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
     ptx::cluster_sync();            // barriers of both CTAs initialised before any remote signal
     ptx::tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
-    const int t_begin = p.cta_start[cluster], t_end = p.cta_start[cluster + 1];
+    int t_begin, t_end, t_step = 1;
+    if constexpr (ALIGN) {
+        t_begin = cluster;
+        t_end = p.start[p.count];
+        t_step = static_cast<int>(gridDim.x >> 1);
+    } else {
+        t_begin = p.cta_start[cluster];
+        t_end = p.cta_start[cluster + 1];
+    }
+    // tile t of the list; slot: where the last one lay (tiles are taken in order)
+    auto tile_of = [&](int t, int& slot) {
+        if constexpr (ALIGN) {
+            while (t >= p.start[slot + 1]) ++slot;
+            const int local = t - p.start[slot], nt = p.col_tiles[slot];
+            return TcTile{p.mod[slot], slot, local / nt, local % nt};
+        } else {
+            return p.tiles[t];
+        }
+    };
+    int slot = 0;
     pdl_begin();
 
     if (warp == 0) {
@@ -837,8 +867,8 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
             uint32_t phase = 0;
             uint32_t issued = 0, last_par = 0;
             bool ok = true;
-            for (int t = t_begin; t < t_end && ok; ++t) {
-                const TcTile tl = p.tiles[t];
+            for (int t = t_begin; t < t_end && ok; t += t_step) {
+                const TcTile tl = tile_of(t, slot);
                 const TcMod& md = p.mods[tl.mod];
                 const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 1];
                 const CUtensorMap* bmap = &p.maps[tl.mod * kMaps + 2];
@@ -883,8 +913,8 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
             int buf = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
-            for (int t = t_begin; t < t_end && ok; ++t) {
-                const TcTile tl = p.tiles[t];
+            for (int t = t_begin; t < t_end && ok; t += t_step) {
+                const TcTile tl = tile_of(t, slot);
                 const TcMod& md = p.mods[tl.mod];
                 const int nk = (md.r + K2_BK - 1) / K2_BK;
                 const bool right = ALIGN && md.right != 0;
@@ -988,8 +1018,8 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
         const int il = q * 32 + lane;
         int buf = 0;
         uint32_t acc_phase = 0;
-        for (int t = t_begin; t < t_end; ++t) {
-            const TcTile tl = p.tiles[t];
+        for (int t = t_begin; t < t_end; t += t_step) {
+            const TcTile tl = tile_of(t, slot);
             const TcMod& md = p.mods[tl.mod];
             const int nn = md.n, mkb = md.kb;
             const int i = (2 * tl.t0 + crank) * K2_BM + il, c0 = tl.t1 * K2_BN + ch * (K2_BN / 2);
@@ -1056,7 +1086,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
                 gg += __shfl_xor_sync(0xffffffffu, gg, o);
             }
             if (lane == 0) {
-                double* acc = p.acc + 3 * tl.slot;
+                double* acc = p.acc + 3 * p.call_idx[tl.slot];
                 atomicAdd(acc + 0, static_cast<double>(dot));
                 atomicAdd(acc + 1, static_cast<double>(na));
                 atomicAdd(acc + 2, static_cast<double>(gg));
@@ -2702,19 +2732,32 @@ int tc_alignment(TcState* st, const moara_hparams& hp, int n_mod, const int* ids
     }
     for (int c0 = 0; c0 < n_mod; c0 += kTcGroup) {
         const int cnt = std::min(kTcGroup, n_mod - c0);
-        TcState::Tiles* tl = tc_tiles(st, std::vector<int>(ids + c0, ids + c0 + cnt));
-        if (tl == nullptr) { st->err = "tile list allocation failed"; return MOARA_ERR_CUDA; }
+        std::vector<int> order(cnt);
+        for (int q = 0; q < cnt; ++q) order[q] = q;
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int a, int b) { return st->mods[ids[c0 + a]].r > st->mods[ids[c0 + b]].r; });
         K2AlignParams p2{};
-        p2.cta_start = tl->k2_start; p2.tiles = tl->k2;
         p2.mods = st->d_mods; p2.maps = st->d_maps; p2.status = st->d_status;
         p2.acc = acc + 3 * (size_t)c0;
-        for (int q = 0; q < cnt; ++q) p2.G[q] = static_cast<const uint16_t*>(G[c0 + q]);
+        p2.count = cnt;
+        int tiles = 0;
+        for (int q = 0; q < cnt; ++q) {
+            const TcMod& md = st->mods[ids[c0 + order[q]]];
+            p2.G[q] = static_cast<const uint16_t*>(G[c0 + order[q]]);
+            p2.mod[q] = ids[c0 + order[q]];
+            p2.call_idx[q] = order[q];
+            p2.col_tiles[q] = (md.n + K2_BN - 1) / K2_BN;
+            p2.start[q] = tiles;
+            tiles += (md.m + 2 * K2_BM - 1) / (2 * K2_BM) * p2.col_tiles[q];
+        }
+        p2.start[cnt] = tiles;
+        const int clusters = std::min(tiles, st->k2_clusters);
         auto fn = B == 8    ? k2_backproject<8, false, true>
                   : B == 16 ? k2_backproject<16, false, true>
                   : B == 32 ? k2_backproject<32, false, true>
                   : B == 64 ? k2_backproject<64, false, true>
                             : k2_backproject<128, false, true>;
-        const cudaError_t e = launch(fn, 2 * tl->g2, K2_THREADS, K2_SMEM, s, 1, p2);
+        const cudaError_t e = launch(fn, 2 * clusters, K2_THREADS, K2_SMEM, s, 1, p2);
         ++*launches;
         if (e != cudaSuccess) {
             st->err = "alignment product launch failed";
