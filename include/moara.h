@@ -296,7 +296,9 @@ int moara_flatten_shape(int ndim, const int64_t* shape, int* m, int* n);
  * Scratch: each module's workspace (its contents are rewritten by the next
  * step anyway) and three doubles per module owned by the context (allocated
  * on first use or when a call has more modules than before; growing them
- * waits for `stream`).
+ * waits for `stream`), and a work list for each of the first 64 lists of
+ * modules (allocated and copied by the first call on it).  A call that is
+ * recorded in a graph makes no list and needs none.
  * Errors: MOARA_ERR_UNSUPPORTED (nothing launched) when a module is not on
  * the tensor-core path (bf16 gradient, n and r multiples of 8, B in {8, 16,
  * 32, 64, 128}); the usual argument errors otherwise. */

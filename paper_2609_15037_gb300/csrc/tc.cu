@@ -169,15 +169,20 @@ struct K2Params {
     int decompose;
 };
 
-// The diagnostic's tiles are numbered in the parameter block, modules in
-// descending K, and cluster c takes tiles c, c + clusters, ...: within one tile
-// of the longest-first assignment of the step's work lists, without a list in
-// device memory (the call may be recorded in a graph for modules that no call
-// had together before, and scoring many subsets keeps nothing).
+// The diagnostic takes the step's work list of its modules where there is one or
+// one can be made.  Otherwise (count > 0: a graph is being recorded, which allows
+// no allocation, or the context keeps kAlignLists of them already)
+// the tiles are numbered through the modules, in descending K, and dealt to the
+// clusters in turn, back and forth.  Without lists at all, four weights of 288 to
+// 7264 columns (312 tiles) took 129 us instead of 126: a few tiles per cluster
+// need the longest-first assignment, and the first touch of each line of the
+// parameter block is a miss.  (The lists in the parameter block, 30 KB of it: one
+// 500 x 1744 weight 35.6 us instead of 33.5.)
+constexpr int kAlignLists = 64;
 struct K2AlignParams : K2Params {
     const uint16_t* G[kTcGroup];       // gradient of each launch slot (m x n)
     double* acc;                       // three sums per module of the call: <G, a>, <a, a>, <G, G>
-    int count;
+    int count;                         // 0: tiles and slots (places in the call) from the list
     int mod[kTcGroup];                 // module of the slot
     int call_idx[kTcGroup];            // its place in the call
     int col_tiles[kTcGroup];
@@ -836,24 +841,29 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
     ptx::cluster_sync();            // barriers of both CTAs initialised before any remote signal
     ptx::tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
-    int t_begin, t_end, t_step = 1;
-    if constexpr (ALIGN) {
-        t_begin = cluster;
-        t_end = p.start[p.count];
-        t_step = static_cast<int>(gridDim.x >> 1);
-    } else {
+    int t_begin = 0, t_end = 0;
+    bool in_turn = false;
+    if constexpr (ALIGN) in_turn = p.count > 0;
+    if (!in_turn) {
         t_begin = p.cta_start[cluster];
         t_end = p.cta_start[cluster + 1];
+    } else if constexpr (ALIGN) {
+        const int total = p.start[p.count], g = static_cast<int>(gridDim.x >> 1);
+        t_end = total / g;
+        t_end += t_end * g + (t_end & 1 ? g - 1 - cluster : cluster) < total;
     }
-    // tile t of the list; slot: where the last one lay (tiles are taken in order)
+    // the cluster's tile t; slot: where the last one lay (in turn they go up)
     auto tile_of = [&](int t, int& slot) {
         if constexpr (ALIGN) {
-            while (t >= p.start[slot + 1]) ++slot;
-            const int local = t - p.start[slot], nt = p.col_tiles[slot];
-            return TcTile{p.mod[slot], slot, local / nt, local % nt};
-        } else {
-            return p.tiles[t];
+            if (in_turn) {
+                const int g = static_cast<int>(gridDim.x >> 1);
+                const int e = t * g + (t & 1 ? g - 1 - cluster : cluster);
+                while (e >= p.start[slot + 1]) ++slot;
+                const int local = e - p.start[slot], nt = p.col_tiles[slot];
+                return TcTile{p.mod[slot], slot, local / nt, local % nt};
+            }
         }
+        return p.tiles[t];
     };
     int slot = 0;
     pdl_begin();
@@ -867,7 +877,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
             uint32_t phase = 0;
             uint32_t issued = 0, last_par = 0;
             bool ok = true;
-            for (int t = t_begin; t < t_end && ok; t += t_step) {
+            for (int t = t_begin; t < t_end && ok; ++t) {
                 const TcTile tl = tile_of(t, slot);
                 const TcMod& md = p.mods[tl.mod];
                 const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 1];
@@ -913,7 +923,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
             int buf = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
-            for (int t = t_begin; t < t_end && ok; t += t_step) {
+            for (int t = t_begin; t < t_end && ok; ++t) {
                 const TcTile tl = tile_of(t, slot);
                 const TcMod& md = p.mods[tl.mod];
                 const int nk = (md.r + K2_BK - 1) / K2_BK;
@@ -1018,7 +1028,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
         const int il = q * 32 + lane;
         int buf = 0;
         uint32_t acc_phase = 0;
-        for (int t = t_begin; t < t_end; t += t_step) {
+        for (int t = t_begin; t < t_end; ++t) {
             const TcTile tl = tile_of(t, slot);
             const TcMod& md = p.mods[tl.mod];
             const int nn = md.n, mkb = md.kb;
@@ -1086,7 +1096,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
                 gg += __shfl_xor_sync(0xffffffffu, gg, o);
             }
             if (lane == 0) {
-                double* acc = p.acc + 3 * p.call_idx[tl.slot];
+                double* acc = p.acc + 3 * (in_turn ? p.call_idx[tl.slot] : tl.slot);
                 atomicAdd(acc + 0, static_cast<double>(dot));
                 atomicAdd(acc + 1, static_cast<double>(na));
                 atomicAdd(acc + 2, static_cast<double>(gg));
@@ -1931,6 +1941,7 @@ struct TcState {
         const int* k2_start = nullptr; const TcTile* k2 = nullptr; int g2 = 0;
     };
     std::map<std::vector<int>, Tiles> tiles;
+    int align_lists = 0;                   // of them, made by alignment calls
     bool attrs_set = false;
     int k1_clusters = 1, k2_clusters = 1;  // co-resident 2-CTA clusters of K1 / K2
     K1Params p1;                           // parameter block of the next K1 launch
@@ -2732,26 +2743,44 @@ int tc_alignment(TcState* st, const moara_hparams& hp, int n_mod, const int* ids
     }
     for (int c0 = 0; c0 < n_mod; c0 += kTcGroup) {
         const int cnt = std::min(kTcGroup, n_mod - c0);
-        std::vector<int> order(cnt);
-        for (int q = 0; q < cnt; ++q) order[q] = q;
-        std::stable_sort(order.begin(), order.end(),
-                         [&](int a, int b) { return st->mods[ids[c0 + a]].r > st->mods[ids[c0 + b]].r; });
+        const std::vector<int> chunk(ids + c0, ids + c0 + cnt);
         K2AlignParams p2{};
         p2.mods = st->d_mods; p2.maps = st->d_maps; p2.status = st->d_status;
         p2.acc = acc + 3 * (size_t)c0;
-        p2.count = cnt;
-        int tiles = 0;
-        for (int q = 0; q < cnt; ++q) {
-            const TcMod& md = st->mods[ids[c0 + order[q]]];
-            p2.G[q] = static_cast<const uint16_t*>(G[c0 + order[q]]);
-            p2.mod[q] = ids[c0 + order[q]];
-            p2.call_idx[q] = order[q];
-            p2.col_tiles[q] = (md.n + K2_BN - 1) / K2_BN;
-            p2.start[q] = tiles;
-            tiles += (md.m + 2 * K2_BM - 1) / (2 * K2_BM) * p2.col_tiles[q];
+        int clusters = 0;
+        TcState::Tiles* tl = nullptr;
+        if (st->tiles.count(chunk) > 0) {
+            tl = tc_tiles(st, chunk);
+        } else if (st->align_lists < kAlignLists) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+            if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+                tl = tc_tiles(st, chunk);
+            if (tl != nullptr) ++st->align_lists;
+            else cudaGetLastError();            // not to be had now (another thread records a graph): in turn
         }
-        p2.start[cnt] = tiles;
-        const int clusters = std::min(tiles, st->k2_clusters);
+        if (tl != nullptr) {
+            p2.cta_start = tl->k2_start; p2.tiles = tl->k2;
+            clusters = tl->g2;
+            for (int q = 0; q < cnt; ++q) p2.G[q] = static_cast<const uint16_t*>(G[c0 + q]);
+        } else {
+            std::vector<int> order(cnt);
+            for (int q = 0; q < cnt; ++q) order[q] = q;
+            std::stable_sort(order.begin(), order.end(),
+                             [&](int a, int b) { return st->mods[chunk[a]].r > st->mods[chunk[b]].r; });
+            p2.count = cnt;
+            int tiles = 0;
+            for (int q = 0; q < cnt; ++q) {
+                const TcMod& md = st->mods[chunk[order[q]]];
+                p2.G[q] = static_cast<const uint16_t*>(G[c0 + order[q]]);
+                p2.mod[q] = chunk[order[q]];
+                p2.call_idx[q] = order[q];
+                p2.col_tiles[q] = (md.n + K2_BN - 1) / K2_BN;
+                p2.start[q] = tiles;
+                tiles += (md.m + 2 * K2_BM - 1) / (2 * K2_BM) * p2.col_tiles[q];
+            }
+            p2.start[cnt] = tiles;
+            clusters = std::min(tiles, st->k2_clusters);
+        }
         auto fn = B == 8    ? k2_backproject<8, false, true>
                   : B == 16 ? k2_backproject<16, false, true>
                   : B == 32 ? k2_backproject<32, false, true>

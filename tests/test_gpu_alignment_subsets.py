@@ -1,5 +1,6 @@
 """The alignment diagnostic on subsets of a context's modules: recorded in a graph
-without a call on the same subset before, in any order of the modules, and with
+without a call on the same subset before, with and without a work list (more
+subsets than the context keeps lists of), in any order of the modules, and with
 more modules than one launch carries.  The scores of a subset are those of the
 calls on one module each; 1e-6 apart for the order of the atomic additions (each
 sum is of fp32 partial sums added in fp64)."""
@@ -59,12 +60,21 @@ def test_first_call_on_a_subset_is_capturable():
 @pytest.mark.parametrize("shapes", [
     [(512, 512, 8), (1030, 776, 264), (257, 264, 72), (2304, 1288, 8), (8, 8, 8), (300, 2056, 136)],   # ranks out of order
     [(40 + i % 90, 8 * (1 + i % 40), 8 * (1 + i % 3) if i % 40 > 2 else 8) for i in range(230)],       # two launches
+    [(2600, 9000, 8), (264, 520, 72)],                # several rounds of tiles per cluster, the last one partial
 ])
 def test_modules_of_one_call(shapes):
     M = _cuda()
     g, Gs = _group(M, shapes)
-    S = g.alignment(Gs)
+    S = g.alignment(Gs)                               # a list is made
     ref = _one_by_one(g, Gs)
+    assert (S - ref).abs().max() <= 1e-6
+    few = g.ids[:2]
+    for k in range(70):                               # as many lists as a context keeps, and more
+        m = g.add(8 + k, 16, 8, "bf16")
+        g.load_projector(m, torch.eye(8 + k, 8, device="cuda"))
+        g.alignment([Gs[0], Gs[1], torch.ones(8 + k, 16, device="cuda", dtype=torch.bfloat16)], ids=few + [m])
+    ids = g.ids[:len(shapes)][::-1]                   # a new list of modules: dealt out in turn
+    S = g.alignment(Gs[::-1], ids=ids).flip(0)
     torch.cuda.synchronize()
     assert g.status() == 0
     assert (S - ref).abs().max() <= 1e-6
