@@ -326,13 +326,13 @@ int64_t moara_launch_count(const moara_ctx* ctx);
  * word, waits (with the default bound) for its own copies and tensor-core
  * work in flight, frees its tensor memory and returns, leaving the context
  * usable.  This call sets the bound, in SM clock cycles, of the waits of the
- * tensor-core products of the projector refresh and of moara_alignment's
- * projection (the single-CTA kernels) for launches enqueued afterwards; cycles <= 0 restores
+ * tensor-core products of the projector refresh and of moara_alignment for
+ * launches enqueued afterwards; cycles <= 0 restores
  * the default (2^32 cycles, about 2 s).  A bound shorter than the kernels'
  * own latency (a few hundred cycles) makes them give up on purpose, which is
  * how the failure path is tested; their outputs are then undefined until the
- * next call with the default bound.  The two-CTA pairs (the step kernels and
- * moara_alignment's second product) keep the default bound.  Returns MOARA_ERR_UNSUPPORTED without tensor-core state. */
+ * next call with the default bound.  The step kernels keep the default bound.
+ * Returns MOARA_ERR_UNSUPPORTED without tensor-core state. */
 int moara_set_wait_limit(moara_ctx* ctx, int64_t cycles);
 
 /* Per-kernel timing with CUDA events recorded on the launching stream around

@@ -187,6 +187,7 @@ struct K2AlignParams : K2Params {
     int call_idx[kTcGroup];            // its place in the call
     int col_tiles[kTcGroup];
     int start[kTcGroup + 1];           // first tile of the slot
+    long long wait_limit;              // clock cycles of a bounded wait before it gives up
 };
 static_assert(sizeof(K2AlignParams) <= 32764, "the diagnostic's parameter block fits the kernel parameter space");
 
@@ -201,6 +202,7 @@ struct SmemCtl {
     uint64_t wempty[8];
     uint32_t tmem_base;
     int abort;
+    uint32_t steps;      // stages that this CTA's producer filled (kernels that settle a pair)
 };
 static_assert(sizeof(SmemCtl) <= kCtlBytes, "the barrier block fits the space K1 and K2 reserve for it");
 // K1 and K2 leave room beside them for one K0 CTA (no shared memory of its
@@ -218,6 +220,31 @@ __device__ __forceinline__ bool wait_drain(uint32_t bar, uint32_t parity) {
         if (clock64() - t0 > kWaitLimit) return false;
     }
     return true;
+}
+
+// A pair whose waits may run out while copies are in flight (a wait limit below
+// a copy's latency).  A copy of either CTA completes on the even CTA's barrier,
+// and a stage's phase ends when both CTAs' copies have landed; the two producers
+// may have given up a different number of stages in.
+//
+// pair_abort, by every warp before the last cluster barrier: if its CTA gave up,
+// the peer knows behind that barrier.  pair_settle, by one thread of each CTA
+// behind it: the CTA that filled fewer stages fills the missing ones (the MMAs
+// are done, what lands there is not used), and the even CTA waits for every
+// stage's last phase.  Another cluster barrier, and no copy is left in flight.
+__device__ __forceinline__ void pair_abort(SmemCtl* ctl, int crank) {
+    if ((threadIdx.x & 31) == 0 && *const_cast<volatile int*>(&ctl->abort) != 0)
+        ptx::st_cluster_u32(ptx::mapa(ptx::smem_u32(&ctl->abort), crank ^ 1), 1);
+}
+
+template <int STAGES, class Fill>
+__device__ __forceinline__ void pair_settle(SmemCtl* ctl, int crank, Fill fill) {
+    const uint32_t own = ctl->steps, peer = ptx::ld_cluster_u32(ptx::mapa(ptx::smem_u32(&ctl->steps), crank ^ 1));
+    const uint32_t all = own > peer ? own : peer;
+    for (uint32_t k = own; k < all; ++k) fill(static_cast<int>(k), static_cast<int>(k % STAGES));
+    if (crank == 0)
+        for (uint32_t q = 0; q < STAGES && q < all; ++q)
+            wait_drain(ptx::smem_u32(&ctl->full[q]), ((all - 1 - q) / STAGES) & 1);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
@@ -830,6 +857,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
         }
         ptx::mbar_init(ptx::smem_u32(&ctl->drain), 1);
         ctl->abort = 0;
+        ctl->steps = 0;
         ptx::fence_barrier_init();
     }
     if (warp == 1) {                // collective: one warp of each CTA of the pair
@@ -866,6 +894,29 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
         return p.tiles[t];
     };
     int slot = 0;
+    long long limit = kWaitLimit;                     // of the waits that the diagnostic's roles share
+    if constexpr (ALIGN) limit = p.wait_limit;
+    // this CTA's copies of k-step kb of a tile into a stage
+    auto fill = [&](const TcTile& tl, bool right, int kb, int stage) {
+        const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 1];
+        const CUtensorMap* bmap = &p.maps[tl.mod * kMaps + 2];
+        const CUtensorMap* lmap = &p.maps[tl.mod * kMaps + 9];
+        const int i0 = (2 * tl.t0 + crank) * K2_BM, n0 = tl.t1 * K2_BN;
+        const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
+        const uint32_t fb = ptx::mapa(own, 0);
+        if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * STAGE_BYTES);
+        const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
+        const uint32_t b = a + K2_A_BYTES;
+        ptx::tma_load_2d_pair(a, amap, fb, kb * K2_BK, i0);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = 2 * crank + h;
+            ptx::tma_load_2d_pair(b + h * 8192, bmap, fb, n0 + 64 * c, kb * K2_BK);
+            if (ALIGN && !right)
+                ptx::tma_load_2d_pair(b + K2_B_BYTES + h * 8192, lmap, fb, n0 + 64 * c, kb * K2_BK);
+        }
+        if (right) ptx::tma_load_2d_pair(b + K2_B_BYTES, lmap, fb, kb * K2_BK, i0);
+    };
     pdl_begin();
 
     if (warp == 0) {
@@ -875,40 +926,25 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t issued = 0, last_par = 0;
+            uint32_t issued = 0, last_par = 0, steps = 0;
             bool ok = true;
             for (int t = t_begin; t < t_end && ok; ++t) {
                 const TcTile tl = tile_of(t, slot);
                 const TcMod& md = p.mods[tl.mod];
-                const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 1];
-                const CUtensorMap* bmap = &p.maps[tl.mod * kMaps + 2];
-                const CUtensorMap* lmap = &p.maps[tl.mod * kMaps + 9];
-                const bool right = ALIGN && md.right != 0;
-                const int i0 = (2 * tl.t0 + crank) * K2_BM, n0 = tl.t1 * K2_BN;
                 const int nk = (md.r + K2_BK - 1) / K2_BK;
+                const bool right = ALIGN && md.right != 0;
                 for (int kb = 0; kb < nk; ++kb) {
                     if (!ptx::mbar_wait(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1, abort_flag, p.status,
-                                        MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
-                    const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
-                    const uint32_t fb = ptx::mapa(own, 0);
-                    if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * STAGE_BYTES);
-                    const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
-                    const uint32_t b = a + K2_A_BYTES;
-                    ptx::tma_load_2d_pair(a, amap, fb, kb * K2_BK, i0);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int c = 2 * crank + h;
-                        ptx::tma_load_2d_pair(b + h * 8192, bmap, fb, n0 + 64 * c, kb * K2_BK);
-                        if (ALIGN && !right)
-                            ptx::tma_load_2d_pair(b + K2_B_BYTES + h * 8192, lmap, fb, n0 + 64 * c, kb * K2_BK);
-                    }
-                    if (right) ptx::tma_load_2d_pair(b + K2_B_BYTES, lmap, fb, kb * K2_BK, i0);
+                                        MOARA_ERR_DEVICE_TIMEOUT, limit)) { ok = false; break; }
+                    fill(tl, right, kb, stage);
+                    ++steps;
                     issued |= 1u << stage;
                     last_par = (last_par & ~(1u << stage)) | (phase << stage);
                     if (++stage == K2_STAGES) { stage = 0; phase ^= 1; }
                 }
             }
-            if (!ok && crank == 0) {
+            if (ALIGN) ctl->steps = steps;
+            if (!ALIGN && !ok && crank == 0) {
                 for (int s = 0; s < K2_STAGES; ++s)
                     if (issued & (1u << s)) wait_drain(ptx::smem_u32(&ctl->full[s]), (last_par >> s) & 1);
             }
@@ -929,12 +965,12 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
                 const int nk = (md.r + K2_BK - 1) / K2_BK;
                 const bool right = ALIGN && md.right != 0;
                 if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->acce[buf]), acc_phase ^ 1, abort_flag, p.status,
-                                            MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
+                                            MOARA_ERR_DEVICE_TIMEOUT, limit)) { ok = false; break; }
                 ptx::tc_fence_after();
                 const uint32_t d0 = tmem + buf * 256;
                 for (int kb = 0; kb < nk; ++kb) {
                     if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag, p.status,
-                                                MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
+                                                MOARA_ERR_DEVICE_TIMEOUT, limit)) { ok = false; break; }
                     ptx::tc_fence_after();
                     const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
                     const uint32_t b = a + K2_A_BYTES;
@@ -1053,7 +1089,7 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
             float mg[NM], mgn[NM];
             load(c0, g, mg);
             const bool got = ptx::mbar_wait(ptx::smem_u32(&ctl->accf[buf]), acc_phase, abort_flag, p.status,
-                                            MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit);
+                                            MOARA_ERR_DEVICE_TIMEOUT, limit);
             if (!__all_sync(0xffffffffu, got)) break;
             ptx::tc_fence_after();
             float dot = 0.0f, na = 0.0f, gg = 0.0f;
@@ -1262,7 +1298,21 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
 
     ptx::tc_fence_before();
     __syncwarp();
+    if (ALIGN) pair_abort(ctl, crank);
+    __syncwarp();
     ptx::cluster_sync();            // no CTA leaves while its peer may still signal or fill it
+    if (ALIGN && *abort_flag) {     // the same in both CTAs
+        if (threadIdx.x == 0) {
+            // the copies of any k-step do: every stage takes as many bytes
+            pair_settle<K2_STAGES>(ctl, crank, [&](int, int stage) {
+                int first = 0;
+                const TcTile tl = tile_of(t_begin, first);
+                fill(tl, p.mods[tl.mod].right != 0, 0, stage);
+            });
+        }
+        __syncwarp();
+        ptx::cluster_sync();
+    }
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc2(tmem, 512);
@@ -1561,6 +1611,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KR_THREADS, 1) kr_pa
         ptx::mbar_init(ptx::smem_u32(&ctl->accf[0]), 1);
         ptx::mbar_init(ptx::smem_u32(&ctl->drain), 1);
         ctl->abort = 0;
+        ctl->steps = 0;
         ptx::fence_barrier_init();
     }
     if (warp == 1) {                // collective: one warp of each CTA of the pair
@@ -1574,41 +1625,40 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KR_THREADS, 1) kr_pa
     const uint32_t tmem = ctl->tmem_base;
     pdl_begin();
 
+    // this CTA's copies of k-step kb into a stage
+    const uint32_t bytes = (LO == 1 ? 2 : 1) * PLANE + (LO == 2 ? 2 : 1) * nb * 8192;
+    auto fill = [&](int kb, int stage) {
+        const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
+        const uint32_t fb = ptx::mapa(own, 0);
+        if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * bytes);
+        const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
+        const uint32_t b = a + (LO == 1 ? 2 : 1) * PLANE;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int x = KMAJOR ? kb * KR_BK : r0 + 64 * c;
+            const int y = KMAJOR ? r0 + 64 * c : kb * KR_BK;
+            ptx::tma_load_2d_pair(a + c * 8192, &p.amap[pi], fb, x, y);
+            if (LO == 1) ptx::tma_load_2d_pair(a + PLANE + c * 8192, &p.lmap[pi], fb, x, y);
+        }
+        for (int c = 0; c < nb; ++c) {
+            const int x = n0 + 64 * (nb * crank + c);
+            ptx::tma_load_2d_pair(b + c * 8192, &p.bmap[pi], fb, x, kb * KR_BK);
+            if (LO == 2) ptx::tma_load_2d_pair(b + PLANE + c * 8192, &p.lmap[pi], fb, x, kb * KR_BK);
+        }
+    };
+
     if (warp == 0) {
         if (lane == 0) {
             int stage = 0;
-            uint32_t phase = 0;
-            uint32_t issued = 0, last_par = 0;
-            bool ok = true;
-            const uint32_t bytes = (LO == 1 ? 2 : 1) * PLANE + (LO == 2 ? 2 : 1) * nb * 8192;
+            uint32_t phase = 0, steps = 0;
             for (int kb = 0; kb < nk; ++kb) {
                 if (!ptx::mbar_wait(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1, abort_flag, p.status,
-                                    MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) { ok = false; break; }
-                const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
-                const uint32_t fb = ptx::mapa(own, 0);
-                if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * bytes);
-                const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
-                const uint32_t b = a + (LO == 1 ? 2 : 1) * PLANE;
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int x = KMAJOR ? kb * KR_BK : r0 + 64 * c;
-                    const int y = KMAJOR ? r0 + 64 * c : kb * KR_BK;
-                    ptx::tma_load_2d_pair(a + c * 8192, &p.amap[pi], fb, x, y);
-                    if (LO == 1) ptx::tma_load_2d_pair(a + PLANE + c * 8192, &p.lmap[pi], fb, x, y);
-                }
-                for (int c = 0; c < nb; ++c) {
-                    const int x = n0 + 64 * (nb * crank + c);
-                    ptx::tma_load_2d_pair(b + c * 8192, &p.bmap[pi], fb, x, kb * KR_BK);
-                    if (LO == 2) ptx::tma_load_2d_pair(b + PLANE + c * 8192, &p.lmap[pi], fb, x, kb * KR_BK);
-                }
-                issued |= 1u << stage;
-                last_par = (last_par & ~(1u << stage)) | (phase << stage);
+                                    MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit)) break;
+                fill(kb, stage);
+                ++steps;
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
             }
-            if (!ok && crank == 0) {   // let the copies already in flight land before the CTA exits
-                for (int s = 0; s < STAGES; ++s)
-                    if (issued & (1u << s)) wait_drain(ptx::smem_u32(&ctl->full[s]), (last_par >> s) & 1);
-            }
+            ctl->steps = steps;
         }
     } else if (warp == 1) {
         if (crank == 0 && lane == 0) {
@@ -1617,7 +1667,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KR_THREADS, 1) kr_pa
             uint32_t phase = 0;
             for (int kb = 0; kb < nk; ++kb) {
                 if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag, p.status,
-                                            MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit)) break;
+                                            MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit)) break;
                 ptx::tc_fence_after();
                 const uint32_t a = ptx::smem_u32(smem + stage * STAGE_BYTES);
                 const uint32_t b = a + (LO == 1 ? 2 : 1) * PLANE;
@@ -1647,7 +1697,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KR_THREADS, 1) kr_pa
         // 8 epilogue warps: lane quarter q = warp % 4, every other 16-column chunk
         const int q = warp & 3;
         const bool got = ptx::mbar_wait(ptx::smem_u32(&ctl->accf[0]), 0, abort_flag, p.status,
-                                        MOARA_ERR_DEVICE_TIMEOUT, kWaitLimit);
+                                        MOARA_ERR_DEVICE_TIMEOUT, p.wait_limit);
         if (__all_sync(0xffffffffu, got)) {
             ptx::tc_fence_after();
             const int row = r0 + q * 32 + lane;
@@ -1668,7 +1718,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KR_THREADS, 1) kr_pa
 
     ptx::tc_fence_before();
     __syncwarp();
+    pair_abort(ctl, crank);
+    __syncwarp();
     ptx::cluster_sync();            // no CTA leaves while its peer may still signal or fill it
+    if (*abort_flag) {              // the same in both CTAs
+        if (threadIdx.x == 0) pair_settle<STAGES>(ctl, crank, fill);
+        __syncwarp();
+        ptx::cluster_sync();
+    }
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc2(tmem, 256);
@@ -2606,8 +2663,7 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
             kp.wait_limit = st->wait_limit;
             if (total == 0) continue;
             // CTA pairs where one tile's K outlasts what all tiles take on every
-            // SM (a pair works it off in half the time); the waits of a pair
-            // keep the default bound
+            // SM (a pair works it off in half the time)
             double longest = 0.0, work = 0.0;
             for (int q = 0; q < cnt; ++q) {
                 const TcGemmItem& x = items[sel[c0 + q]];
@@ -2616,7 +2672,7 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
                     work += 1.0 * x.K * (((x.lower ? std::min(x.N, i0 + KR_BM) : x.N) + KR_BN - 1) / KR_BN);
             }
             work /= st->sms;
-            const bool pair = st->wait_limit == kWaitLimit && std::max(0.5 * longest, 1.1 * work) < 0.95 * std::max(longest, work);
+            const bool pair = std::max(0.5 * longest, 1.1 * work) < 0.95 * std::max(longest, work);
             auto fn = pair ? (a_kmajor ? (with_lo == 0 ? kr_pair<true, 0> : with_lo == 1 ? kr_pair<true, 1> : kr_pair<true, 2>)
                                        : (with_lo == 0 ? kr_pair<false, 0>
                                                        : with_lo == 1 ? kr_pair<false, 1> : kr_pair<false, 2>))
@@ -2745,6 +2801,7 @@ int tc_alignment(TcState* st, const moara_hparams& hp, int n_mod, const int* ids
         const int cnt = std::min(kTcGroup, n_mod - c0);
         const std::vector<int> chunk(ids + c0, ids + c0 + cnt);
         K2AlignParams p2{};
+        p2.wait_limit = st->wait_limit;
         p2.mods = st->d_mods; p2.maps = st->d_maps; p2.status = st->d_status;
         p2.acc = acc + 3 * (size_t)c0;
         int clusters = 0;

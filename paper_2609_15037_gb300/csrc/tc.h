@@ -105,10 +105,9 @@ cudaError_t tc_transpose_bf16(const uint16_t* in, uint16_t* out, int rows, int c
 
 const char* tc_last_error(const TcState* st);
 
-// Clock cycles a bounded wait of the refresh and alignment products on KR and
-// KS spins before it gives up and records MOARA_ERR_DEVICE_TIMEOUT; <= 0
-// restores the default (~2 s); the alignment's second product, on the step
-// kernels' CTA pairs, keeps the default.
+// Clock cycles a bounded wait of the refresh's and the alignment's products
+// spins before it gives up and records MOARA_ERR_DEVICE_TIMEOUT; <= 0 restores
+// the default (~2 s).
 void tc_set_wait_limit(TcState* st, long long cycles);
 
 }  // namespace moara

@@ -119,6 +119,18 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
     return r;
 }
 
+// A word of another CTA's shared memory, by its shared::cluster address; ordered
+// by the cluster barrier.
+__device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+
 // Arrive (release at cluster scope) on an mbarrier of another CTA of the
 // cluster, given its shared::cluster address from mapa.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
