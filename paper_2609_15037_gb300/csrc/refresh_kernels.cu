@@ -585,10 +585,10 @@ __global__ void __launch_bounds__(kJacThreads) k_lead_jacobi(const __grid_consta
                     if (q < w) {
                         const float hpq = H[p][q];
                         if (fabsf(hpq) > 1e-30f) {
-                            // the angle to a few ulp (approximate division and
-                            // square root), the rotation orthonormal to
-                            // rounding: c from the tangent that sn uses, by
-                            // rsqrtf and one step of Newton's iteration
+                            // the angle to a few ulp (approximate division),
+                            // the rotation orthonormal to rounding: c from the
+                            // tangent that sn uses, by rsqrtf and one step of
+                            // Newton's iteration
                             const float tau = __fdividef(H[q][q] - H[p][p], 2.0f * hpq);
                             const float at = fabsf(tau);
                             // |tau| past 1e15: tan = 1 / (2 tau), below it (tau^2 does not overflow)

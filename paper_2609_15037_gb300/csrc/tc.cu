@@ -3,8 +3,9 @@
 //  K0  Decompose(G, B) of §3.1 / Appendix B.1 as a memory-bound prepass: block
 //      norms in fp32 and the direction matrix V written in bf16 (at the first
 //      Adam step also the residual V - V_hi, so that the projection carries
-//      ~16 bits there); a second, small pass runs Optimizer_M (Adam on the
-//      block magnitudes).
+//      ~16 bits there), and Optimizer_M (Adam on the block magnitudes) with it;
+//      as a pass of its own for blocks below 32 columns and where the clipping
+//      coefficient needs every norm first.
 //  K1  R = P^T V on tcgen05 (2-SM pairs: 256 ranks x 256 columns per CTA pair,
 //      P exact in bf16), then Optimizer_V (Adam) on R in the epilogue; writes
 //      the Adam update N as bf16.  (Algorithm 1.)
@@ -68,7 +69,7 @@ struct K0Item {
     const uint16_t* G;
     uint16_t* Vhi;
     uint16_t* Vlo;
-    float* mag;                        // m x kb block norms M (written when do_mag)
+    float* mag;                        // m x kb block norms M (written when do_mag, unless Optimizer_M runs in K0)
     float* mag_avg;
     float* mag_avg_sq;
     float* dM;
@@ -78,7 +79,7 @@ struct K0Item {
 struct K0Params {
     int count;
     int hilo;                          // also write V_lo = V - V_hi
-    int do_mag;                        // run Optimizer_M (off when only V is wanted)
+    int do_mag;                        // K0 without Optimizer_M: store the block norms (off when only V is wanted)
     float decomp_eps, beta1, beta2, adam_eps, bc1, bc2;
     const float* clip;                 // gradient clipping coefficient (device) for M, or null
     long long start[kTcGroup + 1];     // warp items (row, 1024-column segment) per module
@@ -2606,11 +2607,10 @@ void tc_set_wait_limit(TcState* st, long long cycles) {
 int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, cudaStream_t s,
                  int64_t* launches) {
     if (!st->kr_attrs) {
-        for (auto fn : {kr_product<true, 0>, kr_product<true, 1>, kr_product<true, 2>, kr_product<false, 0>,
-                        kr_product<false, 1>, kr_product<false, 2>})
+        for (auto fn : {kr_product<true, 0>, kr_product<true, 1>, kr_product<false, 0>, kr_product<false, 1>,
+                        kr_product<false, 2>})
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
-        for (auto fn : {kr_pair<true, 0>, kr_pair<true, 1>, kr_pair<true, 2>, kr_pair<false, 0>, kr_pair<false, 1>,
-                        kr_pair<false, 2>})
+        for (auto fn : {kr_pair<true, 0>, kr_pair<true, 1>, kr_pair<false, 0>, kr_pair<false, 1>, kr_pair<false, 2>})
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
         st->kr_attrs = true;
     }
@@ -2619,6 +2619,10 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
         const int a_inner = a_kmajor ? x.K : x.M;
         if (x.M < 1 || x.N < 1 || x.K < 1 || (a_inner % 8) != 0 || (x.N % 8) != 0) {
             st->err = "tensor-core refresh GEMM: row pitches must be multiples of 16 bytes";
+            return MOARA_ERR_UNSUPPORTED;
+        }
+        if (x.B_lo != nullptr && (a_kmajor || x.A_lo != nullptr)) {
+            st->err = "tensor-core refresh GEMM: B in two planes goes with one MN-major plane of A";
             return MOARA_ERR_UNSUPPORTED;
         }
     }
@@ -2673,12 +2677,13 @@ int tc_gemm_bf16(TcState* st, int a_kmajor, const TcGemmItem* items, int count, 
             }
             work /= st->sms;
             const bool pair = std::max(0.5 * longest, 1.1 * work) < 0.95 * std::max(longest, work);
-            auto fn = pair ? (a_kmajor ? (with_lo == 0 ? kr_pair<true, 0> : with_lo == 1 ? kr_pair<true, 1> : kr_pair<true, 2>)
-                                       : (with_lo == 0 ? kr_pair<false, 0>
-                                                       : with_lo == 1 ? kr_pair<false, 1> : kr_pair<false, 2>))
-                    : a_kmajor ? (with_lo == 0 ? kr_product<true, 0> : with_lo == 1 ? kr_product<true, 1> : kr_product<true, 2>)
-                               : (with_lo == 0 ? kr_product<false, 0>
-                                               : with_lo == 1 ? kr_product<false, 1> : kr_product<false, 2>);
+            auto single = a_kmajor ? (with_lo == 0 ? kr_product<true, 0> : kr_product<true, 1>)
+                                   : (with_lo == 0 ? kr_product<false, 0>
+                                                   : with_lo == 1 ? kr_product<false, 1> : kr_product<false, 2>);
+            auto paired = a_kmajor ? (with_lo == 0 ? kr_pair<true, 0> : kr_pair<true, 1>)
+                                   : (with_lo == 0 ? kr_pair<false, 0>
+                                                   : with_lo == 1 ? kr_pair<false, 1> : kr_pair<false, 2>);
+            auto fn = pair ? paired : single;
             // (the pairs' cluster shape is the kernel's own)
             const cudaError_t e = launch(fn, pair ? 2 * total : total, KR_THREADS, KR_SMEM, s, 1, kp);
             if (e != cudaSuccess) {

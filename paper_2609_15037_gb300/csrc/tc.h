@@ -50,7 +50,7 @@ struct TcGemmItem {
     int ktri;              // B upper triangular: column j needs k <= j only
     uint16_t* out_lo;      // M x N row-major bf16 residual out - bf16(out), or null
     int lower;             // 1: only output tiles on or below the diagonal (M = N)
-    const uint16_t* B_lo;  // residual plane of B (with A_lo null), or null
+    const uint16_t* B_lo;  // residual plane of B (A MN-major, A_lo null), or null
 };
 
 // Grouped launch of TcGemmItems (A read K-major when a_kmajor, else
