@@ -897,12 +897,9 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
     int slot = 0;
     long long limit = kWaitLimit;                     // of the waits that the diagnostic's roles share
     if constexpr (ALIGN) limit = p.wait_limit;
-    // this CTA's copies of k-step kb of a tile into a stage
-    auto fill = [&](const TcTile& tl, bool right, int kb, int stage) {
-        const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 1];
-        const CUtensorMap* bmap = &p.maps[tl.mod * kMaps + 2];
-        const CUtensorMap* lmap = &p.maps[tl.mod * kMaps + 9];
-        const int i0 = (2 * tl.t0 + crank) * K2_BM, n0 = tl.t1 * K2_BN;
+    // this CTA's copies of k-step kb of the tile at row i0, column n0 into a stage
+    auto fill = [&](const CUtensorMap* amap, const CUtensorMap* bmap, const CUtensorMap* lmap, bool right, int i0, int n0,
+                    int kb, int stage) {
         const uint32_t own = ptx::smem_u32(&ctl->full[stage]);
         const uint32_t fb = ptx::mapa(own, 0);
         if (crank == 0) ptx::mbar_arrive_expect_tx(own, 2 * STAGE_BYTES);
@@ -932,12 +929,16 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
             for (int t = t_begin; t < t_end && ok; ++t) {
                 const TcTile tl = tile_of(t, slot);
                 const TcMod& md = p.mods[tl.mod];
-                const int nk = (md.r + K2_BK - 1) / K2_BK;
+                const CUtensorMap* amap = &p.maps[tl.mod * kMaps + 1];
+                const CUtensorMap* bmap = &p.maps[tl.mod * kMaps + 2];
+                const CUtensorMap* lmap = &p.maps[tl.mod * kMaps + 9];
                 const bool right = ALIGN && md.right != 0;
+                const int i0 = (2 * tl.t0 + crank) * K2_BM, n0 = tl.t1 * K2_BN;
+                const int nk = (md.r + K2_BK - 1) / K2_BK;
                 for (int kb = 0; kb < nk; ++kb) {
                     if (!ptx::mbar_wait(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1, abort_flag, p.status,
                                         MOARA_ERR_DEVICE_TIMEOUT, limit)) { ok = false; break; }
-                    fill(tl, right, kb, stage);
+                    fill(amap, bmap, lmap, right, i0, n0, kb, stage);
                     ++steps;
                     issued |= 1u << stage;
                     last_par = (last_par & ~(1u << stage)) | (phase << stage);
@@ -1308,7 +1309,9 @@ k2_backproject(const __grid_constant__ typename std::conditional<ALIGN, K2AlignP
             pair_settle<K2_STAGES>(ctl, crank, [&](int, int stage) {
                 int first = 0;
                 const TcTile tl = tile_of(t_begin, first);
-                fill(tl, p.mods[tl.mod].right != 0, 0, stage);
+                const CUtensorMap* maps = &p.maps[tl.mod * kMaps];
+                fill(maps + 1, maps + 2, maps + 9, p.mods[tl.mod].right != 0, (2 * tl.t0 + crank) * K2_BM, tl.t1 * K2_BN, 0,
+                     stage);
             });
         }
         __syncwarp();
